@@ -339,16 +339,17 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * kernels, the planes of the z chunk each (x, y) tile marches through, where the staged
  * plaquette launches, whose tiles are twice as tall, split every chunk in two).  CL_OPT_STAGES: TMA stage buffers
  * of the fused pass, 2..6, or -1 for the loader without TMA staging (0 = library choice;
- * rows that are not a multiple of 16 bytes always use the loader without TMA; ensembles
- * clamp to 2..4 with the ring kernel and 3..6 ringless).  On a Runge-Kutta scalar lattice
+ * FP32 rows that are not a multiple of 16 bytes run their own staged kernel with 3 or 4
+ * buffers, reported as variant 0, unless variant 0 or stages -1 is asked for; FP64 ones always
+ * use the loader without TMA; ensembles clamp to 2..4 with the ring kernel and 3..6 ringless).  On a Runge-Kutta scalar lattice
  * the three options tile the stage kernel instead: CL_OPT_STAGES 3..6 stage buffers of the
  * TMA-staged stage kernel (2 counts as 3; -1 = the direct-load kernel), CL_OPT_TILE_BY its
  * rows per tile, CL_OPT_TILE_DZ its z chunks (0 = the library's: every y tile cut into the
  * same chunks, one wave of blocks; -1 = balanced persistent ranges).
  * CL_OPT_PASS_VARIANT (-1 = library choice, the default): TMA-staged pass kernel, 1 =
  * ringless (the library's choice: each warp drifts the neighbour rows it needs from the
- * stage buffers, no consumer barrier; 16-byte vectors, 2..5 stages (ensembles 3..6), other
- * rows fall back to 0), 0 = drifted rows shared through a ring in shared memory with one
+ * stage buffers, no consumer barrier; 16-byte vectors, 2..5 stages (ensembles 3..6), FP32 rows
+ * of any alignment 3 or 4, other rows fall back to 0), 0 = drifted rows shared through a ring in shared memory with one
  * consumer barrier per plane.  Both give bit-identical fields on the same tiles.  For an
  * axion-U(1) lattice, two launches per Runge-Kutta stage (plaquette fields through global
  * memory, then the stage) unless 1: 0 = every neighbour gathered from L1/L2, 2 = the

@@ -61,7 +61,8 @@ struct cl_lattice {
     void* kpi[2][2] = {};
     int rk_BY = 1, rk_DZ = 1, rk_nby = 1, rk_nbz = 1;
     int rk_stages = 0;              // TMA-staged Runge-Kutta kernel with this many stages (0: direct loads)
-    int variant = 0;          // TMA pass kernel in use (0 ring, 1 ringless)
+    int variant = 0;          // TMA pass kernel in use (0 ring, 1 ringless, 2 rows of any alignment)
+    bool any_rows = false;    // variant 2
     bool gauge = false;       // axion + compact U(1) links (one scalar field, Runge-Kutta)
     void* th[3][2] = {};      // link angles theta_i
     void* ef[3][2] = {};      // electric fields E_i
@@ -379,9 +380,28 @@ cl_status choose_tiles(cl_lattice* l)
             scalar_pass_smem_bytes(prec, l->nf, N, BY, 5, var) <= (size_t)kPassMaxSmem)
             stages = 5;
     }
-    const int var_eff = stages > 0 ? var : 0;
-    while (BY > 1 && scalar_pass_smem_bytes(prec, l->nf, N, BY, stages, var_eff) > (size_t)kPassMaxSmem) BY /= 2;
-    if (scalar_pass_threads(prec, N, BY) > 512 ||
+    int var_eff = stages > 0 ? var : 0;
+    // FP32 rows that are no multiple of 16 bytes: the staged pass for rows of any alignment
+    l->any_rows = false;
+    if (prec != CL_PREC_FP64 && l->VW * l->es != 16 && l->opt_stages != -1 && l->opt_variant != 0) {
+        auto fits = [&](int by, int st) {
+            return by >= 1 && scalar_pass_any_threads(N, by) <= 448 &&
+                   scalar_pass_smem_bytes(prec, l->nf, N, by, st, 2) <= (size_t)kPassMaxSmem;
+        };
+        int by = l->opt_BY > 0 ? std::min(l->opt_BY, N) : std::min(N, 32 * 14 * kAnySites / N);
+        const int want = l->opt_stages == 3 || l->opt_stages == 2 ? 3 : 4;
+        while (by > 1 && !fits(by, want)) --by;
+        const int st = fits(by, want) ? want : (fits(by, 3) ? 3 : 0);
+        if (st) {
+            const int tiles = (N + by - 1) / by;
+            BY = (N + tiles - 1) / tiles;  // rows shared evenly among as many tiles
+            stages = st;
+            var_eff = 2;
+            l->any_rows = true;
+        }
+    }
+    while (!l->any_rows && BY > 1 && scalar_pass_smem_bytes(prec, l->nf, N, BY, stages, var_eff) > (size_t)kPassMaxSmem) BY /= 2;
+    if ((!l->any_rows && scalar_pass_threads(prec, N, BY) > 512) ||
         scalar_pass_smem_bytes(prec, l->nf, N, BY, stages, var_eff) > (size_t)kPassMaxSmem)
         return fail(l, CL_EINVAL, "lattice too large for the fused pass tiling (N=%d)", N);
     l->variant = var_eff;
@@ -1369,7 +1389,8 @@ cl_status cl_init_lattice(cl_lattice** out, const cl_lattice_params* p)
         }
         l->own_stream = true;
     }
-    const size_t bytes = (size_t)l->V * l->es;
+    // whole multiples of 256 bytes: the staged kernels copy whole 16-byte units
+    const size_t bytes = ((size_t)l->V * l->es + 255) / 256 * 256;
     for (int f = 0; f < l->nf; ++f)
         for (int b = 0; b < 2; ++b) {
             if (cudaMalloc(&l->phi[f][b], bytes) != cudaSuccess || cudaMalloc(&l->pi[f][b], bytes) != cudaSuccess ||
@@ -1742,7 +1763,8 @@ cl_status cl_get_option(cl_lattice* l, int32_t option, int64_t* value)
         *value = ens ? l->ens_stages : (is_rk(l->p.integrator) && !l->gauge ? (l->rk_stages > 0 ? l->rk_stages : -1) : l->stages);
         return CL_OK;
     case CL_OPT_PASS_VARIANT:
-        *value = ens ? l->ens_variant : (l->gauge ? (l->u1_fused ? 1 : (l->u1_sfused ? 3 : (l->u1_staged ? 2 : 0))) : l->variant);
+        *value = ens ? l->ens_variant : (l->gauge ? (l->u1_fused ? 1 : (l->u1_sfused ? 3 : (l->u1_staged ? 2 : 0)))
+                                                   : (l->any_rows ? 0 : l->variant));
         return CL_OK;
     }
     return fail(l, CL_EINVAL, "unknown option %d", option);
@@ -1787,7 +1809,7 @@ static void report_tiles(const cl_lattice* l, double us, double* best)
     best[1] = ens ? l->hmem[0].BY : l->BY;
     best[2] = ens ? l->hmem[0].DZ : l->DZ;
     best[3] = us;
-    best[4] = ens ? l->ens_variant : l->variant;
+    best[4] = ens ? l->ens_variant : (l->any_rows ? 0 : l->variant);
 }
 
 static std::string tune_key(const cl_lattice* l)
@@ -1885,7 +1907,8 @@ cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
         cl_status s0 = apply_tiles(l, 0, 0, 0, 1);
         if (s0 != CL_OK) return s0;
         const int by_auto = l->BY;
-        const bool nr_ok = l->VW * l->es == 16;  // the ringless kernel takes 16-byte vectors
+        // the ringless kernels take 16-byte vectors, or FP32 rows of any alignment
+        const bool nr_ok = l->VW * l->es == 16 || l->any_rows;
         std::vector<int> st_list = {-1, 0};
         if (scalar_pass_tma_ok(l->p.precision, l->N))
             for (int st = 2; st <= 6; ++st) st_list.push_back(st);

@@ -104,7 +104,8 @@ struct ScalarPassArgs {
     int flags;
     int stages;         // TMA stage buffers (2..6), 0 = general loader
     int grid;           // persistent grid size (used when DZ < 0)
-    int variant;        // TMA kernel: 0 = shared ring of drifted rows, 1 = ringless
+    int variant;        // TMA kernel: 0 = shared ring of drifted rows, 1 = ringless,
+                        // 2 = ringless for rows of any alignment
 };
 
 // Launch one fused scalar pass (drift -> stencil kick -> energies -> scale-factor update).
@@ -126,6 +127,22 @@ size_t scalar_pass_smem(int precision, int nf, int N, int BY);
 size_t scalar_pass_smem_bytes(int precision, int nf, int N, int BY, int stages, int variant = 0);
 bool scalar_pass_tma_ok(int precision, int N);
 int scalar_pass_threads(int precision, int N, int BY);
+// Staged pass on rows of any alignment (FP32): sites per consumer thread, consumer threads of a
+// tile of BY rows, and the elements of a stage region that holds n elements at any shift of a
+// 16-byte boundary (E elements).
+constexpr int kAnySites = 4;
+int scalar_pass_any_threads(int N, int BY);
+template <int E>
+__host__ __device__ constexpr int any_region(int n)
+{
+    return (E - 1 + n + E - 1) / E * E;
+}
+// The region of a tile's own rows: room for every site of its consumer warps.
+template <int E>
+__host__ __device__ constexpr int any_own_region(int N, int BY)
+{
+    return any_region<E>((BY * N + 32 * kAnySites - 1) / (32 * kAnySites) * (32 * kAnySites));
+}
 
 // One 2N Runge-Kutta stage of the scalar fields and the scale factor.
 template <typename T>

@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(512) k_scalar_pass(const ScalarPassArgs<T> A)
 
 #include "scalar_pass_tma.cuh"
 #include "scalar_pass_tma_nr.cuh"
+#include "scalar_pass_tma_any.cuh"
 
 // ------------------------------------------------------------------ reduced lattices
 // The fused pass on a reduced (d+1)-dimensional lattice (section "Scalar dynamics in 1+1 and
@@ -424,6 +425,8 @@ size_t scalar_pass_smem_bytes(int precision, int nf, int N, int BY, int stages, 
     const size_t rows = (size_t)(BY + 2) * N * es;
     if (stages <= 0) return (size_t)nf * 3 * rows;  // direct loader: three-plane ring
     const size_t narr = (size_t)nf * (precision == CL_PREC_FP32_KAHAN ? 3 : 2);
+    if (variant == 2)  // rows of any alignment: three regions an array, each with room for its shift
+        return (size_t)stages * narr * (2 * any_region<4>(N) + any_own_region<4>(N, BY)) * es;
     if (variant == 1) return (size_t)stages * narr * rows;  // ringless: the stage buffers only
     // TMA loader: three-slot ring of drifted fields plus the stage buffers
     return (size_t)nf * 3 * rows + (size_t)stages * narr * rows;
@@ -469,6 +472,32 @@ static cudaError_t launch_nr(const ScalarPassArgs<T>& A, dim3 grid, dim3 block, 
     return cudaErrorInvalidValue;
 }
 
+// Rows of any alignment, staged (FP32): S = 3 or 4 stages, kAnySites sites per consumer thread.
+template <typename T, int NF, bool KAHAN>
+static cudaError_t launch_any(const ScalarPassArgs<T>& A, dim3 grid, cudaStream_t s, int* occ)
+{
+    if constexpr (sizeof(T) == 4) {
+        const int prec = KAHAN ? CL_PREC_FP32_KAHAN : CL_PREC_FP32;
+        const int block = scalar_pass_any_threads(A.N, A.BY) + 32;
+        const size_t smem = scalar_pass_smem_bytes(prec, NF, A.N, A.BY, A.stages, 2);
+        if (block > 480 || smem > (size_t)kPassMaxSmem || (A.stages != 3 && A.stages != 4)) return cudaErrorInvalidValue;
+        auto* k3 = k_scalar_pass_tma_any<T, NF, KAHAN, kAnySites, 3>;
+        auto* k4 = k_scalar_pass_tma_any<T, NF, KAHAN, kAnySites, 4>;
+        auto* k = A.stages == 3 ? k3 : k4;
+        static DevFlag attr[2];
+        DevFlag& set = attr[A.stages - 3];
+        if (!set) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassMaxSmem);
+            if (e != cudaSuccess) return e;
+            set = true;
+        }
+        if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, block, smem);
+        k<<<grid, block, smem, s>>>(A);
+        return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
+}
+
 template <typename T, int NF, bool KAHAN, int VW>
 static cudaError_t launch_one(const ScalarPassArgs<T>& A, cudaStream_t s, int* occ)
 {
@@ -477,6 +506,7 @@ static cudaError_t launch_one(const ScalarPassArgs<T>& A, cudaStream_t s, int* o
     dim3 block(((TX * A.BY + 31) / 32) * 32 + (A.stages > 0 ? 32 : 0));  // + producer warp
     dim3 grid(A.DZ > 0 ? A.nby * A.nbz : A.grid);  // DZ < 0: balanced persistent ranges
     const size_t smem = scalar_pass_smem_bytes(prec, NF, A.N, A.BY, A.stages, A.variant);
+    if (A.variant == 2 && A.stages > 0) return launch_any<T, NF, KAHAN>(A, grid, s, occ);
     if (A.variant == 1 && A.stages > 0) return launch_nr<T, NF, KAHAN, VW>(A, grid, block, smem, s, occ);
     static DevFlag attr_set[8];
     const int si = A.stages < 0 ? 0 : (A.stages > 7 ? 7 : A.stages);
@@ -559,6 +589,8 @@ bool scalar_pass_tma_ok(int precision, int N)
     const int es = precision == CL_PREC_FP64 ? 8 : 4;
     return (N * es) % 16 == 0;
 }
+
+int scalar_pass_any_threads(int N, int BY) { return (BY * N + 32 * kAnySites - 1) / (32 * kAnySites) * 32; }
 
 size_t scalar_pass_smem(int precision, int nf, int N, int BY)
 {

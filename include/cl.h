@@ -366,6 +366,10 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * drifted rows in registers; CL_OPT_TILE_DZ its rows per chunk, CL_OPT_TILE_BY how many rows
  * ahead it prefetches into L2, 0 = library choice) or 0 = one thread per site; both agree to
  * rounding.
+ * A small scalar lattice (up to about 2e6 sites in FP32, 4e5 to 1e6 in FP64) takes the leapfrog
+ * steps of a cl_step call in resident launches of many passes each, unless the caller set one of
+ * the tiling options (the library's choices that cl_get_option reports then still serve the
+ * passes outside cl_step).
  * Errors: CL_EINVAL, CL_EUNSUPPORTED. */
 enum { CL_OPT_GRAPH = 0, CL_OPT_TILE_BY = 1, CL_OPT_TILE_DZ = 2, CL_OPT_STAGES = 3, CL_OPT_PASS_VARIANT = 4 };
 cl_status cl_set_option(cl_lattice* l, int32_t option, int64_t value);
@@ -444,7 +448,7 @@ typedef struct {
 cl_status cl_fused_pass_noalloc(const cl_pass_noalloc_desc* d);
 
 /* Number of kernel launches queued by the most recent cl_step (graph replays count the
- * kernels inside the graph). */
+ * kernels inside the graph; where one resident launch runs many passes, every pass counts). */
 int64_t cl_last_launch_count(const cl_lattice* l);
 
 const char* cl_strerror(cl_status s);

@@ -81,6 +81,9 @@ struct cl_lattice {
                                     //   integer-time state of the last uncommitted close
     double hubble_limit = 0.0;
     bool use_graph = true;
+    bool user_tiles = false;        // a tiling option was set by the caller (not by the autotuner)
+    int ps_BY = 0, ps_BZ = 0, ps_grid = 0;  // resident multi-pass kernel: box of rows, blocks (0: not used)
+    unsigned* ps_barrier = nullptr;
     int opt_BY = 0, opt_DZ = 0, opt_stages = 0, opt_variant = -1;  // -1: library choice
     int u1_dz = 8;                  // planes per block of the U(1) kernels
     int u1_gdz = 8;                 // planes per block of the gather kernels beside staged ones
@@ -302,6 +305,22 @@ cl_status ens_tiles(cl_lattice* l)
     return CL_OK;
 }
 
+// Lattices up to this many sites take their steps in the resident multi-pass kernel, whose pass
+// starts sooner (3.9 us against 16.4 at 32^3) but reads a site's neighbours through L1 and L2
+// instead of staging them, and drifts them once per reader.  The lines lie where the two cross
+// (us a pass, per-pass kernel / resident).  FP32 + Kahan, one field: 24.4 / 22.1 at 128^3, 26.0 / 28.0
+// at 136^3; two fields: 31.8 / 30.2 at 120^3, 32.3 / 34.4 at 124^3; rows of other alignment, whose
+// staged kernel is slower: 45.1 / 43.8 at 131^3 and 46.6 / 48.4 at 135^3 (two fields).  Plain FP32:
+// 24.9 / 22.1 at 144^3 (one field), 40.5 / 30.3 at 131^3 (two).  FP64, where both are bound by the
+// FP64 pipe and the repeated drifts count: 67.8 / 66.5 at 100^3 (one field), 63.5 / 62.3 at 72^3 (two).
+int64_t persist_max_sites(const cl_lattice* l)
+{
+    if (is_fp64(l)) return l->nf == 1 ? 1000000 : 400000;
+    if (!has_kahan(l)) return l->nf == 1 ? 3000000 : 2300000;
+    if (l->VW * l->es != 16) return 2250000;
+    return l->nf == 1 ? 2150000 : 1750000;
+}
+
 cl_status choose_tiles(cl_lattice* l)
 {
     if (is_ens(l)) return ens_tiles(l);
@@ -478,6 +497,15 @@ cl_status choose_tiles(cl_lattice* l)
         if (nbz > N) nbz = N;
         l->gw_DZ = (int)((N + nbz - 1) / nbz);
         l->gw_nbz = (N + l->gw_DZ - 1) / l->gw_DZ;
+    }
+    l->ps_grid = 0;
+    if (!is_rk(l->p.integrator) && !l->gauge && !l->gw && !l->user_tiles && l->V <= persist_max_sites(l) &&
+        persist_tiles(prec, N, nsm, &l->ps_BY, &l->ps_BZ)) {
+        // small lattices: cl_step runs its passes in the resident kernel
+        if (!l->ps_barrier && cudaMalloc(&l->ps_barrier, 256) != cudaSuccess)
+            return fail(l, CL_ENOMEM, "cannot allocate the grid barrier");
+        l->ps_grid = ((N + l->ps_BY - 1) / l->ps_BY) * ((N + l->ps_BZ - 1) / l->ps_BZ);
+        if (3 * l->ps_grid > nblocks) nblocks = 3 * l->ps_grid;  // 2 (kMaxQ + 1) numbers a block
     }
     l->rk_stages = 0;
     if (is_rk(l->p.integrator) && l->VW * l->es == 16 && N % l->VW == 0 && l->opt_stages != -1) {
@@ -924,6 +952,46 @@ double open_kick(const cl_lattice* l)
     return 0.5 * w[0] * l->p.dt;
 }
 
+// nsteps steps of a small lattice in launches of the resident kernel (open leapfrog).
+template <typename T>
+cl_status run_persist_t(cl_lattice* l, const std::vector<PassCoef>& sched, int nsteps)
+{
+    PersistArgs<T> A{};
+    for (int f = 0; f < l->nf; ++f)
+        for (int b = 0; b < 2; ++b) {
+            A.phi[f][b] = (T*)l->phi[f][b];
+            A.pi[f][b] = (T*)l->pi[f][b];
+            A.c[f][b] = (T*)l->cc[f][b];
+        }
+    A.scal = l->scal;
+    A.partials = l->partials;
+    A.barrier = l->ps_barrier;
+    A.N = l->N; A.BY = l->ps_BY; A.BZ = l->ps_BZ; A.nby = (l->N + l->ps_BY - 1) / l->ps_BY;
+    A.pps = (int)sched.size();
+    A.dx = l->dx; A.alpha = l->p.alpha; A.kappa = l->p.kappa;
+    for (int i = 0; i < A.pps; ++i) {
+        A.d[i] = sched[i].d;
+        A.e[i] = sched[i].e;
+        A.k[i] = sched[i].k;
+    }
+    for (int f = 0; f < 2; ++f) { A.m2[f] = l->m2[f]; A.lam[f] = l->lam[f]; }
+    A.g2 = l->g2;
+    A.hubble_limit = l->hubble_limit;
+    A.flags = l->p.expansion ? P_EXPANSION : 0;
+    const int most = kPersistPasses / A.pps;  // steps of one launch
+    for (int done = 0; done < nsteps;) {
+        const int n = std::min(most, nsteps - done);
+        A.in0 = l->cur;
+        A.passes = n * A.pps;
+        CUDA_TRY(l, cudaMemsetAsync(l->ps_barrier, 0, sizeof(unsigned), l->stream));
+        const cudaError_t e = launch_scalar_persist(l->p.precision, l->nf, &A, l->ps_grid, l->stream);
+        if (e != cudaSuccess) return fail(l, CL_ECUDA, "resident pass launch failed: %s", cudaGetErrorString(e));
+        l->cur = (l->cur + A.passes) & 1;
+        done += n;
+    }
+    return CL_OK;
+}
+
 cl_status open_leapfrog(cl_lattice* l)
 {
     if (l->open) return CL_OK;
@@ -1306,6 +1374,7 @@ void cl_free(cl_lattice* l)
         if (l->u1s[q]) cudaFree(l->u1s[q]);
     if (l->scal) cudaFree(l->scal);
     if (l->partials) cudaFree(l->partials);
+    if (l->ps_barrier) cudaFree(l->ps_barrier);
     if (l->sg_buf) cudaFree(l->sg_buf);
     if (l->d_members) cudaFree(l->d_members);
     if (l->d_items) cudaFree(l->d_items);
@@ -1782,6 +1851,12 @@ cl_status cl_get_option(cl_lattice* l, int32_t option, int64_t* value)
     return fail(l, CL_EINVAL, "unknown option %d", option);
 }
 
+static cl_status retile(cl_lattice* l)
+{
+    l->user_tiles = l->opt_BY != 0 || l->opt_DZ != 0 || l->opt_stages != 0 || l->opt_variant != -1;
+    return choose_tiles(l);
+}
+
 cl_status cl_set_option(cl_lattice* l, int32_t option, int64_t value)
 {
     if (!l) return CL_EINVAL;
@@ -1790,22 +1865,22 @@ cl_status cl_set_option(cl_lattice* l, int32_t option, int64_t value)
     case CL_OPT_TILE_BY:
         if (value < 0 || value > l->N) return fail(l, CL_EINVAL, "tile BY out of range");
         l->opt_BY = (int)value;
-        return choose_tiles(l);
+        return retile(l);
     case CL_OPT_TILE_DZ:
         if (value < -1 || value > l->N) return fail(l, CL_EINVAL, "tile DZ out of range");
         l->opt_DZ = (int)value;
-        return choose_tiles(l);
+        return retile(l);
     case CL_OPT_PASS_VARIANT:
         if (value < -1 || value > (l->gauge ? 3 : 1))
             return fail(l, CL_EINVAL, "pass variant must be -1, 0 or 1 (2, 3 on an axion-U(1) lattice)");
         if (value == 1 && is_u1_lf(l))
             return fail(l, CL_EUNSUPPORTED, "the axion-U(1) leapfrog has no fused pass form");
         l->opt_variant = (int)value;
-        return choose_tiles(l);
+        return retile(l);
     case CL_OPT_STAGES:
         if (value < -1 || value == 1 || value > 6) return fail(l, CL_EINVAL, "stages must be -1, 0 or 2..6");
         l->opt_stages = (int)value;
-        return choose_tiles(l);
+        return retile(l);
     }
     return fail(l, CL_EINVAL, "unknown option %d", option);
 }
@@ -1843,6 +1918,7 @@ static std::string tune_key(const cl_lattice* l)
 
 static cl_status apply_tiles(cl_lattice* l, int stages, int by, int dz, int variant)
 {
+    l->user_tiles = false;
     l->opt_stages = stages;
     l->opt_BY = by;
     l->opt_DZ = dz;
@@ -1992,6 +2068,13 @@ cl_status cl_step(cl_lattice* l, int32_t nsteps)
     // the fused stages leave R of the final state behind; stages with a reduction launch leave
     // that of their last input state
     l->rbar_valid = nmc_f;
+    if (l->ps_grid > 0) {
+        cl_status s = is_fp64(l) ? run_persist_t<double>(l, sched, nsteps) : run_persist_t<float>(l, sched, nsteps);
+        if (s != CL_OK) return s;
+        l->last_launches += (int64_t)pps * nsteps;  // the passes that ran, as everywhere
+        l->diag_valid = true;
+        return CL_OK;
+    }
     for (int i = 0; i < nsteps; ++i) {
         if (l->use_graph) {
             const int par = l->cur;

@@ -144,6 +144,30 @@ __host__ __device__ constexpr int any_own_region(int N, int BY)
     return any_region<E>((BY * N + 32 * kAnySites - 1) / (32 * kAnySites) * (32 * kAnySites));
 }
 
+// Many fused passes in one cooperative launch, for small lattices (scalar_persist.cu).
+constexpr int kPersistSched = 81;      // passes of the longest composition's step (Yoshida-10)
+constexpr int kPersistPasses = 2048;   // passes a launch runs at most (about 10 ms)
+template <typename T>
+struct PersistArgs {
+    T* phi[2][2];  // [field][buffer]
+    T* pi[2][2];
+    T* c[2][2];
+    DevScal* scal;
+    double* partials;   // [2][kMaxQ + 1][grid]
+    unsigned* barrier;  // zero at the launch
+    int N, BY, BZ, nby; // box of rows of a block
+    int in0;            // buffer read by the first pass
+    int passes, pps;    // passes of this launch (a multiple of pps), passes per step
+    double dx, alpha, kappa;
+    double d[kPersistSched], e[kPersistSched], k[kPersistSched];
+    double m2[2], lam[2], g2;
+    double hubble_limit;
+    int flags;          // P_EXPANSION
+};
+constexpr int kPersistBlocks = 160;    // its blocks at most (one per SM)
+bool persist_tiles(int precision, int N, int nsm, int* BY, int* BZ);
+cudaError_t launch_scalar_persist(int precision, int nf, const void* args, int grid, cudaStream_t s);
+
 // One 2N Runge-Kutta stage of the scalar fields and the scale factor.
 template <typename T>
 struct RkStageArgs {

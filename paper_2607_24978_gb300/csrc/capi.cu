@@ -121,6 +121,9 @@ struct cl_lattice {
     int nitems = 0, ens_grid = 0, ens_stages = 0, ens_stage_stride = 0, ens_ring_slot = 0, ens_variant = 0;
     float* sg_buf = nullptr;        // surrogate jumps: packed input (3 V), output (2 V), snapshot (3 V)
     size_t ens_smem = 0;
+    void* sp_mem = nullptr;         // spectra: scratch kept between calls (see spec_acquire)
+    size_t sp_bytes = 0;
+    std::vector<std::pair<int, cufftHandle>> sp_plans;  // D2Z plans by lattice size
     char err[512] = {0};
 };
 
@@ -1323,6 +1326,80 @@ void* field_buffer(cl_lattice* l, int kind, int f, int buf)
 
 }  // namespace
 
+namespace {
+
+// Scratch and plan of one spectrum call.
+struct SpecWork {
+    double* real = nullptr;  // transform input
+    double2* F = nullptr;    // half spectra
+    double* bins = nullptr;  // S[nb], C[nb], k[nb], delta[nb]
+    int* table = nullptr;    // bin of every squared mode number
+    cufftHandle plan = 0;
+    void* temp = nullptr;    // scratch to free after the call
+    bool temp_plan = false;
+};
+
+// Bytes of scratch, and of a plan's work area, that a handle keeps from one spectrum call to the
+// next: a measurement every few steps paid three cudaMalloc / cudaFree pairs and a plan each time
+// (1.0 of 3.4 ms at 256^3, whose scratch is 270 MB).  Larger calls, long against that, allocate
+// and release their own, as all did, so that a lattice that fills the device leaves it the room.
+constexpr size_t kSpecKeep = (size_t)512 << 20;
+constexpr size_t kSpecPlans = 8;  // an ensemble's sizes
+
+cl_status spec_acquire(cl_lattice* l, int N, size_t nreal, size_t nF, int nb, SpecWork* w)
+{
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t b_real = up(nreal * sizeof(double)), b_F = up(nF * sizeof(double2)), b_bins = up(4 * (size_t)nb * sizeof(double));
+    const size_t bytes = b_real + b_F + b_bins + up(spectrum_table_bytes(N));
+    char* base = nullptr;
+    if (bytes <= kSpecKeep) {
+        if (l->sp_bytes < bytes) {
+            if (l->sp_mem) cudaFree(l->sp_mem);
+            l->sp_mem = nullptr;
+            l->sp_bytes = 0;
+            if (cudaMalloc(&l->sp_mem, bytes) != cudaSuccess) {
+                l->sp_mem = nullptr;
+                return fail(l, CL_ENOMEM, "spectrum scratch allocation failed");
+            }
+            l->sp_bytes = bytes;
+        }
+        base = (char*)l->sp_mem;
+    } else {
+        if (cudaMalloc(&w->temp, bytes) != cudaSuccess) {
+            w->temp = nullptr;
+            return fail(l, CL_ENOMEM, "spectrum scratch allocation failed");
+        }
+        base = (char*)w->temp;
+    }
+    w->real = (double*)base;
+    w->F = (double2*)(base + b_real);
+    w->bins = (double*)(base + b_real + b_F);
+    w->table = (int*)(base + b_real + b_F + b_bins);
+    for (const auto& pp : l->sp_plans)
+        if (pp.first == N) w->plan = pp.second;
+    if (!w->plan) {
+        if (cufftPlan3d(&w->plan, N, N, N, CUFFT_D2Z) != CUFFT_SUCCESS) {
+            w->plan = 0;
+            return fail(l, CL_ECUDA, "cufftPlan3d failed");
+        }
+        size_t ws = 0;
+        if (l->sp_plans.size() < kSpecPlans && cufftGetSize(w->plan, &ws) == CUFFT_SUCCESS && ws <= kSpecKeep)
+            l->sp_plans.push_back({N, w->plan});
+        else
+            w->temp_plan = true;
+    }
+    if (cufftSetStream(w->plan, l->stream) != CUFFT_SUCCESS) return fail(l, CL_ECUDA, "cufftSetStream failed");
+    return CL_OK;
+}
+
+void spec_release(SpecWork* w)
+{
+    if (w->temp_plan) cufftDestroy(w->plan);
+    if (w->temp) cudaFree(w->temp);
+}
+
+}  // namespace
+
 extern "C" {
 
 const char* cl_strerror(cl_status s)
@@ -1376,6 +1453,8 @@ void cl_free(cl_lattice* l)
     if (l->partials) cudaFree(l->partials);
     if (l->ps_barrier) cudaFree(l->ps_barrier);
     if (l->sg_buf) cudaFree(l->sg_buf);
+    if (l->sp_mem) cudaFree(l->sp_mem);
+    for (const auto& pp : l->sp_plans) cufftDestroy(pp.second);
     if (l->d_members) cudaFree(l->d_members);
     if (l->d_items) cudaFree(l->d_items);
     if (l->d_sched) cudaFree(l->d_sched);
@@ -1777,15 +1856,11 @@ cl_status cl_gw_spectrum(cl_lattice* l, double dn, int32_t type, double* k_out, 
     if (st != CL_OK) return st;
     const double a = hs[0].a;  // a at the integer time (the staggered form keeps a there)
     const size_t nh = (size_t)N * N * (N / 2 + 1);
-    double* real = nullptr;
-    double2* F = nullptr;
-    double* bins = nullptr;  // S[nb], C[nb], k[nb], delta[nb]
-    cufftHandle plan = 0;
-    if (cudaMalloc(&real, (size_t)V * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&F, 5 * nh * sizeof(double2)) != cudaSuccess || cudaMalloc(&bins, 4 * (size_t)nb * sizeof(double)) != cudaSuccess)
-        st = fail(l, CL_ENOMEM, "GW spectrum scratch allocation failed");
-    if (st == CL_OK && cufftPlan3d(&plan, N, N, N, CUFFT_D2Z) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "cufftPlan3d failed");
-    if (st == CL_OK && cufftSetStream(plan, l->stream) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "cufftSetStream failed");
+    SpecWork sw;
+    st = spec_acquire(l, N, (size_t)V, 5 * nh, nb, &sw);
+    double *real = sw.real, *bins = sw.bins;
+    double2* F = sw.F;
+    const cufftHandle plan = sw.plan;
     for (int c = 0; c < 5 && st == CL_OK; ++c) {
         // h' = a^(alpha-3) pi_v: the factor is applied to the binned sums below
         if (launch_field_to_double(l->p.precision, l->gpv[c][buf], real, V, l->stream) != cudaSuccess)
@@ -1814,10 +1889,7 @@ cl_status cl_gw_spectrum(cl_lattice* l, double dn, int32_t type, double* k_out, 
             delta_out[i] = ca * h[3 * nb + i];
         }
     }
-    if (plan) cufftDestroy(plan);
-    if (real) cudaFree(real);
-    if (F) cudaFree(F);
-    if (bins) cudaFree(bins);
+    spec_release(&sw);
     return st;
 }
 
@@ -2285,22 +2357,17 @@ cl_status cl_spectrum(cl_lattice* l, int32_t member, int32_t field, double dn, i
     }
     const void* src = (const char*)fb + mem_off_bytes(l, member);
     const size_t nh = (size_t)N * N * (N / 2 + 1);
-    double* real = nullptr;
-    double2* F = nullptr;
-    double* bins = nullptr;  // S[nb], C[nb], k[nb], delta[nb]
-    cufftHandle plan = 0;
-    cl_status st = CL_OK;
-    if (cudaMalloc(&real, (size_t)V * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&F, nh * sizeof(double2)) != cudaSuccess || cudaMalloc(&bins, 4 * (size_t)nb * sizeof(double)) != cudaSuccess)
-        st = fail(l, CL_ENOMEM, "spectrum scratch allocation failed");
-    if (st == CL_OK && cufftPlan3d(&plan, N, N, N, CUFFT_D2Z) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "cufftPlan3d failed");
-    if (st == CL_OK && cufftSetStream(plan, l->stream) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "cufftSetStream failed");
+    SpecWork w;
+    cl_status st = spec_acquire(l, N, (size_t)V, nh, nb, &w);
+    double *real = w.real, *bins = w.bins;
+    double2* F = w.F;
+    const cufftHandle plan = w.plan;
     if (st == CL_OK && launch_field_to_double(l->p.precision, src, real, V, l->stream) != cudaSuccess)
         st = fail(l, CL_ECUDA, "field conversion failed");
     if (st == CL_OK && cufftExecD2Z(plan, real, (cufftDoubleComplex*)F) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "D2Z failed");
     if (st == CL_OK && cudaMemsetAsync(bins, 0, 2 * (size_t)nb * sizeof(double), l->stream) != cudaSuccess)
         st = fail(l, CL_ECUDA, "memset failed");
-    if (st == CL_OK && launch_spectrum_bins(F, N, dn, nb, bins, bins + nb, l->stream) != cudaSuccess)
+    if (st == CL_OK && launch_spectrum_bins(F, w.table, N, dn, nb, bins, bins + nb, l->stream) != cudaSuccess)
         st = fail(l, CL_ECUDA, "binning failed");
     if (st == CL_OK &&
         launch_spectrum_finish(bins, bins + nb, N, mem_L(l, member), dn, type, nb, bins + 2 * nb, bins + 3 * nb, l->stream) != cudaSuccess)
@@ -2317,10 +2384,7 @@ cl_status cl_spectrum(cl_lattice* l, int32_t member, int32_t field, double dn, i
             delta_out[i] = h[3 * nb + i];
         }
     }
-    if (plan) cufftDestroy(plan);
-    if (real) cudaFree(real);
-    if (F) cudaFree(F);
-    if (bins) cudaFree(bins);
+    spec_release(&w);
     return st;
 }
 
@@ -2338,16 +2402,11 @@ cl_status cl_gauge_spectrum(cl_lattice* l, int32_t which, double dn, int32_t typ
     if (nbins) *nbins = nb;
     if (cap == 0) return CL_OK;
     const size_t nh = (size_t)N * N * (N / 2 + 1);
-    double* real = nullptr;
-    double2* F = nullptr;
-    double* bins = nullptr;  // S[nb], C[nb], k[nb], delta[nb]
-    cufftHandle plan = 0;
-    cl_status st = CL_OK;
-    if (cudaMalloc(&real, 3 * (size_t)V * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&F, 3 * nh * sizeof(double2)) != cudaSuccess || cudaMalloc(&bins, 4 * (size_t)nb * sizeof(double)) != cudaSuccess)
-        st = fail(l, CL_ENOMEM, "gauge spectrum scratch allocation failed");
-    if (st == CL_OK && cufftPlan3d(&plan, N, N, N, CUFFT_D2Z) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "cufftPlan3d failed");
-    if (st == CL_OK && cufftSetStream(plan, l->stream) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "cufftSetStream failed");
+    SpecWork sw;
+    cl_status st = spec_acquire(l, N, 3 * (size_t)V, 3 * nh, nb, &sw);
+    double *real = sw.real, *bins = sw.bins;
+    double2* F = sw.F;
+    const cufftHandle plan = sw.plan;
     if (st == CL_OK) {
         const cudaError_t e = is_fp64(l) ? gauge_fields_t<double>(l, which, real) : gauge_fields_t<float>(l, which, real);
         if (e != cudaSuccess) st = fail(l, CL_ECUDA, "gauge field conversion failed");
@@ -2374,10 +2433,7 @@ cl_status cl_gauge_spectrum(cl_lattice* l, int32_t which, double dn, int32_t typ
             delta_out[i] = h[3 * nb + i];
         }
     }
-    if (plan) cufftDestroy(plan);
-    if (real) cudaFree(real);
-    if (F) cudaFree(F);
-    if (bins) cudaFree(bins);
+    spec_release(&sw);
     return st;
 }
 

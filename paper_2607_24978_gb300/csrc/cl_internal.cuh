@@ -348,8 +348,10 @@ struct GaugeSpecArgs {
 cudaError_t launch_gauge_fields(int precision, const void* args, double* out, cudaStream_t s);
 cudaError_t launch_gauge_bins(const double2* F, int N, double dx, int which, double dn, int nbins, double* S,
                               double* C, cudaStream_t s);
-// Shell binning of |F|^2 over a real-to-complex half spectrum: S[l], C[l] (zeroed by the caller).
-cudaError_t launch_spectrum_bins(const double2* F, int N, double dn, int nbins, double* S, double* C,
+// Shell binning of |F|^2 over a real-to-complex half spectrum: S[l], C[l] (zeroed by the caller);
+// table: scratch of spectrum_table_bytes(N).
+size_t spectrum_table_bytes(int N);
+cudaError_t launch_spectrum_bins(const double2* F, int* table, int N, double dn, int nbins, double* S, double* C,
                                  cudaStream_t s);
 // delta[l] from S, C per the spectrum formula of cl_spectrum.
 cudaError_t launch_spectrum_finish(const double* S, const double* C, int N, double L, double dn, int type,

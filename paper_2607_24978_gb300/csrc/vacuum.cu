@@ -159,61 +159,113 @@ cudaError_t launch_fill(void* p, int precision, int64_t n, double v, cudaStream_
     return cudaGetLastError();
 }
 
-// Shell binning over the half spectrum.  Block-local histograms in shared memory when
-// they fit, then one atomic per bin and block.
-__global__ void k_spectrum_bins(const double2* __restrict__ F, int N, double dn, int nbins, double* S, double* C,
-                                int use_smem)
+// Bin of every squared mode number n2 = 0 .. 3 (N/2)^2: floor(sqrt(n2)/dn + 1/2), or -1 past the
+// last bin.  One FP64 square root and division for each value of n2 instead of one for each mode.
+__global__ void k_bin_table(int* __restrict__ bin, int n, double dn, int nbins)
+{
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const double l = floor(sqrt((double)q) / dn + 0.5);
+        bin[q] = l < (double)nbins ? (int)l : -1;
+    }
+}
+
+// Shell binning over the half spectrum.  A warp takes the rows (+-j, +-k) of one pair 0 <= j, k <=
+// N/2 together, lane by lane in i: the up to four modes of a lane share their |n|, hence their bin,
+// and along the lanes the bin does not decrease, so each run of equal bins is added up by shuffles
+// and only its first lane touches the block's histogram.  Modes 0 < i < N/2 stand for themselves
+// and their conjugate partner (-i), which is not stored; they are added once and doubled at the
+// end, the others halved.
+//
+// Bound by FP64 (two operations a mode, and one a shuffle step for four modes) and by the 16 bytes
+// a mode from HBM (20 us at 256^3).  Measured at 256^3: 77 us and 5 us for the table; 617 us with
+// a square root, a division and two shared FP64 atomics for every mode.
+__global__ void k_spectrum_bins(const double2* __restrict__ F, const int* __restrict__ bin, int N, int nbins, double* S,
+                                double* C, int use_smem)
 {
     extern __shared__ double sh[];
     double* sS = sh;
-    double* sC = sh + nbins;
+    int* sC = reinterpret_cast<int*>(sh + nbins);
     if (use_smem) {
-        for (int l = threadIdx.x; l < 2 * nbins; l += blockDim.x) sh[l] = 0.0;
+        for (int l = threadIdx.x; l < nbins; l += blockDim.x) {
+            sS[l] = 0.0;
+            sC[l] = 0;
+        }
         __syncthreads();
     }
-    const int NH = N / 2 + 1;
-    const int64_t total = (int64_t)N * N * NH;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(q % NH);
-        const int j = (int)((q / NH) % N);
-        const int k = (int)(q / ((int64_t)NH * N));
-        const int si = i, sj = signed_index(j, N), sk = signed_index(k, N);
-        const double nm = sqrt((double)si * si + (double)sj * sj + (double)sk * sk);
-        const int l = (int)floor(nm / dn + 0.5);
-        if (l >= nbins) continue;
-        // modes 0 < i < N/2 stand for themselves and their conjugate partner (-i)
-        const double w = (i == 0 || 2 * i == N) ? 1.0 : 2.0;
-        const double2 v = F[q];
-        const double p = w * (v.x * v.x + v.y * v.y);
-        if (use_smem) {
-            atomicAdd(&sS[l], p);
-            atomicAdd(&sC[l], w);
-        } else {
-            atomicAdd(&S[l], p);
-            atomicAdd(&C[l], w);
+    const int NH = N / 2 + 1, lane = threadIdx.x & 31;
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    for (int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < NH * NH; g += warps) {
+        const int k = g / NH, j = g - k * NH;
+        const bool mj = j != 0 && 2 * j != N, mk = k != 0 && 2 * k != N;  // the mirrored rows exist
+        const double2* r0 = F + ((size_t)k * N + j) * NH;
+        const double2* r1 = F + ((size_t)k * N + (N - j)) * NH;
+        const double2* r2 = F + ((size_t)(N - k) * N + j) * NH;
+        const double2* r3 = F + ((size_t)(N - k) * N + (N - j)) * NH;
+        const int modes = (mj ? 2 : 1) * (mk ? 2 : 1), jk2 = j * j + k * k;
+        for (int i0 = 0; i0 < NH; i0 += 32) {
+            const int i = i0 + lane;
+            const bool in = i < NH;
+            const double2 zero = make_double2(0.0, 0.0);
+            const double2 v0 = in ? __ldcs(&r0[i]) : zero;
+            const double2 v1 = in && mj ? __ldcs(&r1[i]) : zero;
+            const double2 v2 = in && mk ? __ldcs(&r2[i]) : zero;
+            const double2 v3 = in && mj && mk ? __ldcs(&r3[i]) : zero;
+            double p = fma(v0.x, v0.x, v0.y * v0.y);
+            if (mj) p = fma(v1.x, v1.x, fma(v1.y, v1.y, p));
+            if (mk) p = fma(v2.x, v2.x, fma(v2.y, v2.y, p));
+            if (mj && mk) p = fma(v3.x, v3.x, fma(v3.y, v3.y, p));
+            const bool twice = i != 0 && 2 * i != N;
+            int c = twice ? 2 * modes : modes;
+            if (__any_sync(0xffffffffu, !twice)) p = twice ? p : 0.5 * p;
+            const int l = in ? bin[i * i + jk2] : -1;
+            // sums of the runs of equal bins, at each run's first lane
+            for (int off = 1; off < 32; off *= 2) {
+                const int lo = __shfl_down_sync(0xffffffffu, l, off);
+                const bool same = lane + off < 32 && lo == l;
+                if (!__any_sync(0xffffffffu, same)) break;
+                const double po = __shfl_down_sync(0xffffffffu, p, off);
+                const int co = __shfl_down_sync(0xffffffffu, c, off);
+                if (same) {
+                    p += po;
+                    c += co;
+                }
+            }
+            const int before = __shfl_up_sync(0xffffffffu, l, 1);
+            if (l >= 0 && (lane == 0 || before != l)) {
+                if (use_smem) {
+                    atomicAdd(&sS[l], p);
+                    atomicAdd(&sC[l], c);
+                } else {
+                    atomicAdd(&S[l], 2.0 * p);
+                    atomicAdd(&C[l], (double)c);
+                }
+            }
         }
     }
     if (use_smem) {
         __syncthreads();
         for (int l = threadIdx.x; l < nbins; l += blockDim.x) {
-            if (sC[l] != 0.0) {
-                atomicAdd(&S[l], sS[l]);
-                atomicAdd(&C[l], sC[l]);
+            if (sC[l] != 0) {
+                atomicAdd(&S[l], 2.0 * sS[l]);
+                atomicAdd(&C[l], (double)sC[l]);
             }
         }
     }
 }
 
-cudaError_t launch_spectrum_bins(const double2* F, int N, double dn, int nbins, double* S, double* C,
+size_t spectrum_table_bytes(int N) { return ((size_t)3 * (N / 2) * (N / 2) + 1) * sizeof(int); }
+
+cudaError_t launch_spectrum_bins(const double2* F, int* table, int N, double dn, int nbins, double* S, double* C,
                                  cudaStream_t s)
 {
-    const int64_t total = (int64_t)N * N * (N / 2 + 1);
-    const size_t smem = (size_t)2 * nbins * sizeof(double);
+    const int n = 3 * (N / 2) * (N / 2) + 1;
+    k_bin_table<<<grid_for(n, 256), 256, 0, s>>>(table, n, dn, nbins);
+    const size_t smem = (size_t)nbins * (sizeof(double) + sizeof(int));
     const int use_smem = smem <= 40 * 1024;
-    const int threads = 512;
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((total + threads - 1) / threads, 152 * 4));
-    k_spectrum_bins<<<blocks, threads, use_smem ? smem : 0, s>>>(F, N, dn, nbins, S, C, use_smem);
+    const int threads = 512, rows = (N / 2 + 1) * (N / 2 + 1);
+    // two blocks per SM: every block adds its histogram to the global one, bin by bin
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((rows + threads / 32 - 1) / (threads / 32), 152 * 2));
+    k_spectrum_bins<<<blocks, threads, use_smem ? smem : 0, s>>>(F, table, N, nbins, S, C, use_smem);
     return cudaGetLastError();
 }
 

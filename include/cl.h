@@ -336,8 +336,8 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * choice).  CL_OPT_TILE_DZ: planes per block (0 = library choice: the y tiles are cut into
  * the same z chunks so that one wave of blocks covers the lattice; -1 = a persistent grid
  * of one wave, each block a balanced contiguous range of planes; for the axion-U(1)
- * kernels, the planes of the z chunk each (x, y) tile marches through, where the staged
- * plaquette launches, whose tiles are twice as tall, split every chunk in two).  CL_OPT_STAGES: TMA stage buffers
+ * kernels, the planes of the z chunk each (x, y) tile marches through, half as many in the staged
+ * plaquette launches, whose tiles are twice as tall).  CL_OPT_STAGES: TMA stage buffers
  * of the fused pass, 2..6, or -1 for the loader without TMA staging (0 = library choice;
  * FP32 rows that are not a multiple of 16 bytes run their own staged kernel with 3 or 4
  * buffers, reported as variant 0, unless variant 0 or stages -1 is asked for; FP64 ones always
@@ -353,8 +353,8 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * consumer barrier per plane.  Both give bit-identical fields on the same tiles.  For an
  * axion-U(1) lattice, two launches per Runge-Kutta stage (plaquette fields through global
  * memory, then the stage) unless 1: 0 = every neighbour gathered from L1/L2, 2 = the
- * neighbourhoods of each plane staged in shared memory by asynchronous copies (the library's
- * choice where N is a multiple of 32, else 0), 1 = one fused launch per stage with the
+ * neighbourhoods of each plane staged in shared memory by asynchronous copies (needs rows of
+ * whole 16-byte units, N >= 32; the library's choice for N = 32 and from N = 36, else 0), 1 = one fused launch per stage with the
  * plaquette fields in shared memory (N a multiple of 32; Runge-Kutta only, CL_EUNSUPPORTED
  * with the leapfrog), 3 = the staged neighbourhoods of 2 in one launch per stage or pass, the
  * plaquette fields computed into shared memory (N a multiple of 32).  All agree to rounding,

@@ -87,6 +87,7 @@ struct cl_lattice {
     int opt_BY = 0, opt_DZ = 0, opt_stages = 0, opt_variant = -1;  // -1: library choice
     int u1_dz = 8;                  // planes per block of the U(1) kernels
     int u1_gdz = 8;                 // planes per block of the gather kernels beside staged ones
+    int u1_pdz = 8;                 // planes per block of the staged plaquette launches
     bool u1_fused = false;          // U(1) stage as one fused launch (plaquettes in shared memory)
     bool u1_staged = false;         // U(1) launches with shared-memory staged neighbourhoods
     bool u1_sfused = false;         //   as one launch, the plaquette fields in shared memory
@@ -307,6 +308,9 @@ cl_status ens_tiles(cl_lattice* l)
     invalidate_graphs(l);
     return CL_OK;
 }
+
+// Whether the staged axion-U(1) launches beat the gather ones where they are possible.
+bool u1_staged_pays(int N) { return N % 32 == 0 || N >= 36; }
 
 // Lattices up to this many sites take their steps in the resident multi-pass kernel, whose pass
 // starts sooner (3.9 us against 16.4 at 32^3) but reads a site's neighbours through L1 and L2
@@ -599,7 +603,8 @@ cl_status choose_tiles(cl_lattice* l)
         l->u1_fused = l->opt_variant == 1 && u1_fused_ok(N) && !is_u1_lf(l);
         // the staged launches (neighbourhoods in shared memory) are the library's choice
         // where the tiles divide N
-        l->u1_staged = (l->opt_variant == -1 || l->opt_variant == 2 || l->opt_variant == 3) && u1_staged_ok(N);
+        l->u1_staged = u1_staged_ok(prec, N) && (l->opt_variant == 2 || (l->opt_variant == 3 && N % 32 == 0) ||
+                                                 (l->opt_variant == -1 && u1_staged_pays(N)));
         l->u1_sfused = l->u1_staged && l->opt_variant == 3;
         int bps = prec == CL_PREC_FP64 ? kU1BlocksPerSM64 : kU1BlocksPerSM32;
         if (l->u1_fused) {
@@ -609,15 +614,18 @@ cl_status choose_tiles(cl_lattice* l)
         int64_t nbz = (int64_t)bps * nsm / tiles;
         if (nbz < 1) nbz = 1;
         if (nbz > N) nbz = N;
-        const int auto_dz = l->u1_staged ? u1_staged_dz(prec, N, nsm) : (int)((N + nbz - 1) / nbz);
+        const int auto_dz = l->u1_staged ? u1_staged_dz(prec, N, nsm, false) : (int)((N + nbz - 1) / nbz);
         l->u1_dz = l->opt_DZ > 0 ? (l->opt_DZ > N ? N : l->opt_DZ) : auto_dz;
         // the gather kernels that run beside the staged launches (the Gauss diagnostic and its
         // plaquette fields) keep the gather form's one-wave chunks
         l->u1_gdz = l->u1_staged ? (int)((N + nbz - 1) / nbz) : l->u1_dz;
         if (2 * u1_grid_blocks(N, l->u1_dz) > nblocks) nblocks = 2 * u1_grid_blocks(N, l->u1_dz);  // stage + plaquette partials
         if (2 * u1_grid_blocks(N, l->u1_gdz) > nblocks) nblocks = 2 * u1_grid_blocks(N, l->u1_gdz);
-        if (l->u1_staged && 2 * u1_staged_blocks(prec, N, l->u1_dz) > nblocks)
-            nblocks = 2 * u1_staged_blocks(prec, N, l->u1_dz);
+        l->u1_pdz = l->opt_DZ > 0 ? (l->u1_dz + 1) / 2 : u1_staged_dz(prec, N, nsm, true);
+        if (l->u1_staged) {  // the stage's partials, then the plaquette launch's
+            const int need = u1_staged_blocks(prec, N, l->u1_dz, false) + u1_staged_blocks(prec, N, l->u1_pdz, true);
+            if (need > nblocks) nblocks = need;
+        }
     }
     s = grow_partials(l, nblocks);
     if (s != CL_OK) return s;
@@ -1081,6 +1089,11 @@ void u1_fill(cl_lattice* l, U1Args<T>& A, int in, int out)
     A.h = l->p.dt;
     A.hubble_limit = l->hubble_limit;
     A.dz = l->u1_dz;
+    if (l->u1_staged) {
+        A.pdz = l->u1_pdz;
+        A.pl_n = u1_staged_blocks(l->p.precision, l->N, l->u1_pdz, true);
+        A.pl_partials = l->partials + (size_t)u1_staged_blocks(l->p.precision, l->N, l->u1_dz, false) * kMaxQ;
+    }
 }
 
 // Component fields of a gauge spectrum (current buffer) as doubles.

@@ -246,6 +246,9 @@ struct U1Args {
     double hubble_limit;
     int flags;    // P_EXPANSION, P_FIRST_STAGE, P_COUNT_STEP, P_ENERGY_ONLY, P_HUBBLE_INIT
     int dz;       // planes per block (all three kernels)
+    int pdz;      // staged plaquette launches: planes per block, and where their pl_n partials go
+    int pl_n;
+    double* pl_partials;
     // Leapfrog passes (lf != 0; the stage launch only, the plaquette launch is unchanged).
     // The force f = (pi', E') is evaluated at positions (phi, theta, a) with the momenta of
     // pi_in / E_in and a' = scal->b; p~ denotes those momenta, base those of k_in[1], k_in[5..7].

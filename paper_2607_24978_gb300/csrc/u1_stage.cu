@@ -310,6 +310,23 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_u1_stage(const 
     }
 }
 
+// A thread's sum of squares: FP32 values as float pairs of the exact square, FP64 as they are.
+template <typename T> struct GaussSum;
+template <> struct GaussSum<float> {
+    F2 s{0.f, 0.f};
+    __device__ __forceinline__ void add(float x)
+    {
+        const float q = __fmul_rn(x, x);
+        s = f2_add(s, F2{q, __fmaf_rn(x, x, -q)});
+    }
+    __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
+};
+template <> struct GaussSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s = fma(x, x, s); }
+    __device__ __forceinline__ double value() const { return s; }
+};
+
 // Lattice Gauss charge G(n) = sum_i [P_i(n) - P_i(n - i)] / dx, P = a^(1-alpha) E + g W.
 // mode 0 writes diag[D_GV] = max_n |G(n)| / max_n sum_i (|P_i(n)| + |P_i(n - i)|) / dx;
 // mode 1 (per-step tracking, for the launch forms whose stage does not sum it itself) the
@@ -321,17 +338,19 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
     __shared__ int s_last;
     const uint32_t N = (uint32_t)A.N;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    // per-site arithmetic in the field precision (GB300's FP64 rate would make this
-    // diagnostic cost a millisecond at 192^3 in double), the maxima and sums in double
+    // per-site arithmetic and maxima in the field precision, FP32 sums of exact squares (square
+    // plus its rounding error) as float pairs: the two FP64 divisions, conversions and additions
+    // a site took before made 440 us at 192^3 and 92 us at 100^3 of this launch on GB300's FP64 pipe
     const T ca = (T)apow(A.scal->a, 1.0 - A.alpha);
     const T b4 = (T)(0.25 / (A.dx * A.dx)), gh = (T)(0.5 * A.g);
-    double gmax = 0.0, smax = 0.0, gsq = 0.0, e2 = 0.0;
+    T gmx = (T)0, smx = (T)0;
+    GaussSum<T> gsq_s, e2_s;
     const U1Tile tile(N, (uint32_t)A.dz);
     for (uint32_t z = tile.z0; z < tile.z1; ++z) {
         if (!tile.active) break;
         const uint32_t n = (z * N + tile.y) * N + tile.x;
         const Nbhd s(tile.x, tile.y, z, N);
-        T G = (T)0, sc = (T)0, ee = (T)0;
+        T G = (T)0, sc = (T)0;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const Off op(i, 1), om(i, -1);
@@ -343,13 +362,14 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
             const T Pm = ca * A.E_in[i][nm] + gh * (A.phi_in[nm] * Bm + A.phi_in[n] * Bn);
             G += Pn - Pm;
             sc += fabs(Pn) + fabs(Pm);
-            ee += A.E_in[i][n] * A.E_in[i][n];
+            if (mode == 1) e2_s.add(A.E_in[i][n]);
         }
-        gmax = fmax(gmax, fabs((double)G) / A.dx);
-        smax = fmax(smax, (double)sc / A.dx);
-        gsq += (double)G * (double)G;
-        e2 += (double)ee;
+        gmx = fmax(gmx, fabs(G));
+        smx = fmax(smx, sc);
+        if (mode == 1) gsq_s.add(G);
     }
+    const double gsq = gsq_s.value(), e2 = e2_s.value();
+    double gmax = (double)gmx / A.dx, smax = (double)smx / A.dx;
     if (mode == 1) {  // sums in a fixed order, then the last block stores the tracked value
         double v[2] = {gsq, e2};
         block_reduce<2>(v, s_red, tid, nthr);

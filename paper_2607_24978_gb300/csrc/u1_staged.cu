@@ -9,8 +9,7 @@
 // into registers; a thread can only keep as many loads in flight as it has registers, and
 // both kernels stall on memory latency at a fraction of the HBM bandwidth.  Here a block
 // owns a 32 x TY tile of (x, y) (stage launches: TY = 16 in FP32, 8 in FP64; plaquette
-// launches, which stage fewer arrays: twice that, over half the z chunk, so that both
-// launch the same blocks; one site per consumer thread) and marches up its z chunk with planes z-1, z, z+1 of every array that is read at a
+// launches, which stage fewer arrays: twice that, over z chunks of their own) and marches up its z chunk with planes z-1, z, z+1 of every array that is read at a
 // neighbour in shared memory: rows y0-1 .. y0+TY and columns x0-VE .. x0+31+VE (VE elements
 // per 16 bytes, so that every row is whole 16-byte units; only the first and last columns
 // are read).  Warp roles, synchronised by mbarriers only:
@@ -25,7 +24,8 @@
 //    counts one arrival per consumer warp), so no warp waits for another one's work.
 // Arrays read only at the site itself (theta and the Runge-Kutta auxiliaries) are loaded by
 // the consumers straight from global memory, one plane ahead.  Every wait is bounded and
-// reports through the status word.  Needs N % 32 == 0; other sizes use the gather kernels.
+// reports through the status word.  Needs rows of whole 16-byte units (u1_staged_ok); other sizes
+// use the gather kernels.
 #include <math.h>
 
 #include "cl_internal.cuh"
@@ -36,9 +36,8 @@
 namespace clk {
 
 // Tile geometry: TX x TY sites a block, RW tile rows a consumer warp (rows w, w + CW, ...),
-// PWARPS producer warps; SPLIT z parts of every z chunk of the stage grid, so that a geometry
-// with SPLIT times taller tiles launches the same number of blocks over the same chunks.
-template <typename T_, int TY_, int PWARPS_, int SPLIT_, int RW_>
+// PWARPS producer warps.
+template <typename T_, int TY_, int PWARPS_, int RW_>
 struct U1SGeomT {
     using T = T_;
     static constexpr int TX = 32;
@@ -46,7 +45,6 @@ struct U1SGeomT {
     static constexpr int RW = RW_;
     static constexpr int CW = TY / RW;         // consumer warps
     static constexpr int PWARPS = PWARPS_;     // producer warps
-    static constexpr int SPLIT = SPLIT_;
     static constexpr int PL = 32 * PWARPS;     // producer lanes
     static constexpr int NT = 32 * (CW + PWARPS);  // threads of a block (consumers, then the producers)
     static constexpr int VE = 16 / (int)sizeof(T);
@@ -60,15 +58,15 @@ struct U1SGeomT {
 
 // the stage launches: 32 x 16 tiles in FP32, 32 x 8 in FP64, six producer warps
 template <typename T>
-using U1SGeom = U1SGeomT<T, sizeof(T) == 4 ? 16 : 8, 6, 1, 1>;
-// the plaquette launches, which stage half as many arrays: tiles twice as tall over half z
-// chunks, six producer warps, and in FP32 two sites a consumer thread (two independent
+using U1SGeom = U1SGeomT<T, sizeof(T) == 4 ? 16 : 8, 6, 1>;
+// the plaquette launches, which stage half as many arrays: tiles twice as tall over z chunks of
+// their own, six producer warps, and in FP32 two sites a consumer thread (two independent
 // chains of shared-memory loads and trigonometry; measured at 192^3 FP32 with one site a
 // thread in 32 x 16 tiles: 113 us a launch, 61% of the issue slots active; this geometry:
 // 104 us, 10% fewer instructions; with four producer warps: 121 us, the consumers waiting on
 // the copies)
 template <typename T>
-using U1PGeom = U1SGeomT<T, 2 * U1SGeom<T>::TY, 6, 2, sizeof(T) == 4 ? 2 : 1>;
+using U1PGeom = U1SGeomT<T, 2 * U1SGeom<T>::TY, 6, sizeof(T) == 4 ? 2 : 1>;
 
 // arrays staged by the plaquette launch and by the stage launch, in slot order
 enum { PQ_PHI = 0, PQ_TH = 1, PQ_E = 4, PQ_NA = 7 };
@@ -93,26 +91,31 @@ static_assert(u1s_smem_bytes<U1PGeom<double>, PQ_NA>() + 2048 <= (size_t)kPassMa
 static_assert(u1s_smem_bytes<U1SGeom<float>, SG_NA>() + 2048 <= (size_t)kPassMaxSmem, "stage ring (FP32)");
 static_assert(u1s_smem_bytes<U1SGeom<double>, SG_NA>() + 2048 <= (size_t)kPassMaxSmem, "stage ring (FP64)");
 
-// Tile and z range of this block: part bz % SPLIT of the z chunk bz / SPLIT (dz planes; the
-// last chunk may be shorter).  A part may be empty (nz = 0) when its chunk has fewer planes
-// than SPLIT; its block stages the two halo planes and writes nothing.
+// Tile and z range of this block: chunk bz of dz planes (the last one may be shorter).  Where the
+// tiles do not divide N, the last tile of a row or column reaches past it: its copies wrap around
+// (they stage other sites' values, which nothing reads) and the sites past N compute on them
+// without storing or adding anything.
 template <typename G>
 struct U1STile {
     uint32_t N, x0, y0, z0, nz;
     __device__ __forceinline__ U1STile(uint32_t N_, uint32_t dz) : N(N_)
     {
-        const uint32_t ntx = N / G::TX, nty = N / G::TY;
+        const uint32_t ntx = (N + G::TX - 1) / G::TX, nty = (N + G::TY - 1) / G::TY;
         uint32_t b = blockIdx.x;
         const uint32_t bx = b % ntx;
         b /= ntx;
         const uint32_t by = b % nty, bz = b / nty;
         x0 = bx * G::TX;
         y0 = by * G::TY;
-        const uint32_t c0 = (bz / G::SPLIT) * dz;
-        const uint32_t cn = c0 + dz < N ? dz : N - c0;
-        const uint32_t per = (cn + G::SPLIT - 1) / G::SPLIT, skip = (bz % G::SPLIT) * per;
-        z0 = c0 + skip;
-        nz = cn > skip ? (cn - skip < per ? cn - skip : per) : 0u;
+        z0 = bz * dz;
+        nz = z0 + dz < N ? dz : N - z0;
+    }
+    // the site of tile column lx, row ly: whether it exists, and its index in plane 0 (a site past
+    // the lattice stands on the last one of its row or column)
+    __device__ __forceinline__ bool has(int lx, int ly) const { return x0 + lx < N && y0 + ly < N; }
+    __device__ __forceinline__ uint32_t at(int lx, int ly) const
+    {
+        return min(y0 + (uint32_t)ly, N - 1) * N + min(x0 + (uint32_t)lx, N - 1);
     }
 };
 
@@ -130,7 +133,7 @@ __device__ __forceinline__ void u1s_build_units(uint2* table, const U1STile<G>& 
         if (c < U::CH) {
             const int a = c / (G::PH * G::CPR), rem = c - a * (G::PH * G::CPR);
             const int r = rem / G::CPR, u = rem - r * G::CPR;
-            int gy = (int)t.y0 - 1 + r, gx = (int)t.x0 - G::VE + u * G::VE;  // in [-1, N] and [-VE, N]
+            int gy = (int)t.y0 - 1 + r, gx = (int)t.x0 - G::VE + u * G::VE;  // in [-1, N + TY) and [-VE, N + TX)
             gy = gy < 0 ? gy + N : (gy >= N ? gy - N : gy);
             gx = gx < 0 ? gx + N : (gx >= N ? gx - N : gx);
             v.x = ((uint32_t)a << 16) | (uint32_t)(a * G::ARR + r * G::PW + u * G::VE);
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
         s_fail = 0;
     }
     __syncthreads();
-    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.dz);
+    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.pdz);
     T* ring_sm = reinterpret_cast<T*>(u1s_dyn);
     uint2* table = reinterpret_cast<uint2*>(ring_sm + G::SLOTS * NA * G::ARR);
     u1s_build_units<G, NA>(table, t, tid, G::NT);
@@ -315,12 +318,13 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
                 o_r[r][k] = cp * R;
                 o_z[r][k] = cp * ((T)0.5 * qs);
                 o_c[r][k] = cp;
-                accGB.add((T)2 * sh * sh);
+                accGB.add(t.has(lane, warp + r * G::CW) ? (T)2 * sh * sh : (T)0);
             }
             ring.release(j, lane);
 #pragma unroll
             for (int r = 0; r < G::RW; ++r) {
-                const uint32_t n = ((t.z0 + j) * N + t.y0 + warp + r * G::CW) * N + t.x0 + lane;
+                if (!t.has(lane, warp + r * G::CW)) continue;
+                const uint32_t n = (t.z0 + j) * N * N + t.at(lane, warp + r * G::CW);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     A.sP[k][n] = o_s[r][k];
@@ -338,7 +342,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
     const Acc<T>* av[1] = {&accGB};
     block_reduce_acc<T, 1>(av, v, s_red, tid, 32 * G::CW);  // (the producers' sums are zero)
     if (tid == 0) {
-        A.partials[(size_t)gridDim.x * kMaxQ + blockIdx.x] = v[0];
+        A.pl_partials[blockIdx.x] = v[0];
         if (s_fail) atomicOr(&A.scal->status, ST_TIMEOUT);
     }
 }
@@ -372,7 +376,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
         s_fail = 0;
     }
     __syncthreads();
-    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.dz);
+    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.pdz);
     T* ring_sm = reinterpret_cast<T*>(u1s_dyn);
     uint2* table = reinterpret_cast<uint2*>(ring_sm + G::SLOTS * NA * G::ARR);
     u1s_build_units<G, NA>(table, t, tid, G::NT);
@@ -385,24 +389,27 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
         const T dx = (T)A.dx;
         // cos P of the sites' three plaquettes, loaded one plane ahead
         T cc[G::RW][3];
-        auto load_c = [&](uint32_t m) {
+        uint32_t at[G::RW];
+#pragma unroll
+        for (int r = 0; r < G::RW; ++r) at[r] = t.at(lane, warp + r * G::CW);
+        auto load_c = [&](uint32_t plane) {
 #pragma unroll
             for (int r = 0; r < G::RW; ++r)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) cc[r][k] = A.cP[k][m + (uint32_t)(r * G::CW) * N];
+                for (int k = 0; k < 3; ++k) cc[r][k] = A.cP[k][plane + at[r]];
         };
-        if (t.nz > 0) load_c((t.z0 * N + t.y0 + warp) * N + t.x0 + lane);
+        load_c(t.z0 * N * N);
         ring.acquire(0);
         ring.acquire(1);
         for (int j = 0; j < (int)t.nz; ++j) {
             ring.acquire(j + 2);
-            const uint32_t n = ((t.z0 + j) * N + t.y0 + warp) * N + t.x0 + lane;  // row warp; row warp + r CW at + r CW N
+            const uint32_t plane = (t.z0 + j) * N * N;
             T cp3[G::RW][3];
 #pragma unroll
             for (int r = 0; r < G::RW; ++r)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) cp3[r][k] = cc[r][k];
-            if (j + 1 < (int)t.nz) load_c(n + N * N);
+            if (j + 1 < (int)t.nz) load_c(plane + N * N);
             T o_r[G::RW][3], o_z[G::RW][3];
 #pragma unroll
             for (int r = 0; r < G::RW; ++r)
@@ -424,12 +431,14 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
             }
             ring.release(j, lane);
 #pragma unroll
-            for (int r = 0; r < G::RW; ++r)
+            for (int r = 0; r < G::RW; ++r) {
+                if (!t.has(lane, warp + r * G::CW)) continue;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    A.rP[k][n + (uint32_t)(r * G::CW) * N] = o_r[r][k];
-                    A.Z[k][n + (uint32_t)(r * G::CW) * N] = o_z[r][k];
+                    A.rP[k][plane + at[r]] = o_r[r][k];
+                    A.Z[k][plane + at[r]] = o_z[r][k];
                 }
+            }
         }
         ring.release((int)t.nz, lane);
         ring.release((int)t.nz + 1, lane);
@@ -525,13 +534,15 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                 for (int q = 0; q < 8; ++q) kc[q] = first ? (T)0 : A.k_in[q][m];
             }
         };
-        if (update) load_site((t.z0 * N + t.y0 + warp) * N + t.x0 + lane);
+        const bool has = t.has(lane, warp);
+        const uint32_t at = t.at(lane, warp);
+        if (update) load_site(t.z0 * N * N + at);
         ring.acquire(0);
         ring.acquire(1);
         for (int j = 0; j < (int)t.nz; ++j) {
             ring.acquire(j + 2);
             const U1SNb<G> S = ring.nb(j, lane, warp);
-            const uint32_t n = ((t.z0 + j) * N + t.y0 + warp) * N + t.x0 + lane;
+            const uint32_t n = (t.z0 + j) * N * N + at;
             T thv[3], kv[8];
 #pragma unroll
             for (int i = 0; i < 3; ++i) thv[i] = thc[i];
@@ -571,11 +582,11 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
             }
             const T F_phi = c_dphi * pv;
             const T F_pi = cL * lap - cV * dV + ws2 * g * eb;
-            if (!LF) {  // (leapfrog pass 1 sums the kinetic energies of its output momenta)
+            if (!LF && has) {  // (leapfrog pass 1 sums the kinetic energies of its output momenta)
                 accK.add(pv * pv);
                 accKE.add(e2);
             }
-            if (!LF || lf == 1) {
+            if ((!LF || lf == 1) && has) {
                 accG.add((pxp - ph) * (pxp - ph) + (pyp - ph) * (pyp - ph) + (pzp - ph) * (pzp - ph));
                 accV.add(ph * ph * ((T)0.5 * m2 + (T)0.25 * lam * ph * ph));
             }
@@ -588,7 +599,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                     // three lower neighbours, loaded here)
                     T ec[3], em[3];
                     if constexpr (LF) {
-                        const uint32_t x = t.x0 + lane, y = t.y0 + warp, z = t.z0 + j;
+                        const uint32_t x = at % N, y = at / N, z = t.z0 + j;
                         const uint32_t nm[3] = {x == 0 ? n + N - 1 : n - 1, y == 0 ? n + (N - 1) * N : n - N,
                                                 z == 0 ? n + (N - 1) * N * N : n - N * N};
 #pragma unroll
@@ -596,7 +607,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                             ec[i] = kv[5 + i];
                             em[i] = A.k_in[5 + i][nm[i]];
                         }
-                        accKE.add(ec[0] * ec[0] + ec[1] * ec[1] + ec[2] * ec[2]);
+                        if (has) accKE.add(ec[0] * ec[0] + ec[1] * ec[1] + ec[2] * ec[2]);
                     } else {
 #pragma unroll
                         for (int i = 0; i < 3; ++i) {
@@ -612,7 +623,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                         gd += ca * (ec[i] - em[i]) +
                               (T)0.5 * g * (S(SG_PHI, U1S_E(i, 1)) * Bpi - S(SG_PHI, U1S_E(i, -1)) * Bmi);
                     }
-                    accGs.add(gd * gd);
+                    if (has) accGs.add(gd * gd);
                 }
                 // link forces
                 T F_E[3];
@@ -631,6 +642,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                     F_E[i] = cE * (-cE * mag * inv_dx3 + g * (cs * inv4dx - wdot)) - cfr * Ecur[i];
                 }
                 ring.release(j, lane);
+                if (!has) continue;
                 if constexpr (LF) {
                     if (lf == 1) {  // closing half-kick (integer-time momenta) and the first iterate
                         T En[3], Eo[3], en2 = (T)0;
@@ -708,8 +720,8 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     if (tid >= 32) return;  // one warp sums the grid's partials, its lane 0 runs the epilogue
     double ws[kMaxQ];  // the stage's sums; slot 4 is the Gauss sum
     warp_sum_partials<kMaxQ>(A.partials, (int)gridDim.x, tid, ws);
-    double gb = 0.0;  // the magnetic energy from the plaquette launch (same grid, one value a block)
-    for (int b = tid; b < (int)gridDim.x; b += 32) gb += __ldcg(&A.partials[(size_t)gridDim.x * kMaxQ + b]);
+    double gb = 0.0;  // the magnetic energy from the plaquette launch, one value a block
+    for (int b = tid; b < A.pl_n; b += 32) gb += __ldcg(&A.pl_partials[b]);
     for (int off = 16; off > 0; off >>= 1) gb += __shfl_xor_sync(0xffffffffu, gb, off);
     double w[kMaxQ] = {ws[0], ws[1], ws[2], ws[3], gb};
     double wg[1] = {ws[kMaxQ - 1]};
@@ -1115,20 +1127,27 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1f_stage(const U1Args<T>
 
 #undef U1S_E
 
-bool u1_staged_ok(int N) { return N >= 32 && N % 32 == 0; }
+// Copies are whole 16-byte units of a row, the wrap at its end included; a tile's halo is at most
+// one row and unit past the lattice's width.
+bool u1_staged_ok(int precision, int N) { return N >= 32 && N % (precision == CL_PREC_FP64 ? 2 : 4) == 0; }
 
-int u1_staged_blocks(int precision, int N, int dz)
+static int u1s_tiles(int precision, int N, bool plaquettes)
 {
-    const int ty = precision == CL_PREC_FP64 ? U1SGeom<double>::TY : U1SGeom<float>::TY;
-    return (N / 32) * (N / ty) * ((N + dz - 1) / dz);
+    const int ty = precision == CL_PREC_FP64 ? (plaquettes ? U1PGeom<double>::TY : U1SGeom<double>::TY)
+                                             : (plaquettes ? U1PGeom<float>::TY : U1SGeom<float>::TY);
+    return ((N + 31) / 32) * ((N + ty - 1) / ty);
+}
+
+int u1_staged_blocks(int precision, int N, int dz, bool plaquettes)
+{
+    return u1s_tiles(precision, N, plaquettes) * ((N + dz - 1) / dz);
 }
 
 // z chunk of the staged launches: one block per SM at a time, so the chunk count minimises
 // waves x (planes + 2 halo planes) of the busiest SM.
-int u1_staged_dz(int precision, int N, int nsm)
+int u1_staged_dz(int precision, int N, int nsm, bool plaquettes)
 {
-    const int ty = precision == CL_PREC_FP64 ? U1SGeom<double>::TY : U1SGeom<float>::TY;
-    const long long tiles = (long long)(N / 32) * (N / ty);
+    const long long tiles = u1s_tiles(precision, N, plaquettes);
     long long best = -1;
     int best_dz = N;
     for (int nbz = 1; nbz <= N; ++nbz) {
@@ -1148,8 +1167,12 @@ template <typename T>
 static cudaError_t launch_u1s_t(const U1Args<T>& A, int what, cudaStream_t s)
 {
     using G = U1SGeom<T>;
-    if (!u1_staged_ok(A.N) || A.dz < 1 || A.dz > A.N) return cudaErrorInvalidValue;
-    const int grid = u1_staged_blocks(sizeof(T) == 8 ? CL_PREC_FP64 : CL_PREC_FP32, A.N, A.dz);
+    const int prec = sizeof(T) == 8 ? CL_PREC_FP64 : CL_PREC_FP32;
+    if (!u1_staged_ok(prec, A.N) || A.dz < 1 || A.dz > A.N) return cudaErrorInvalidValue;
+    if (what != 2 && (A.pdz < 1 || A.pdz > A.N || !A.pl_partials)) return cudaErrorInvalidValue;
+    if (what == 2 && A.N % 32 != 0) return cudaErrorInvalidValue;  // the fused form's tiles divide N
+    const int grid = u1_staged_blocks(prec, A.N, A.dz, false);
+    const int pgrid = what != 2 ? u1_staged_blocks(prec, A.N, A.pdz, true) : 0;
     static DevFlag attr[5];
     if (what == 0) {
         constexpr size_t smem = u1s_smem_bytes<U1PGeom<T>, PQ_NA>();
@@ -1159,7 +1182,7 @@ static cudaError_t launch_u1s_t(const U1Args<T>& A, int what, cudaStream_t s)
             if (e != cudaSuccess) return e;
             attr[0] = true;
         }
-        k_u1s_plaquettes<T><<<grid, U1PGeom<T>::NT, smem, s>>>(A);
+        k_u1s_plaquettes<T><<<pgrid, U1PGeom<T>::NT, smem, s>>>(A);
     } else if (what == 3) {
         constexpr size_t smem = u1s_smem_bytes<U1PGeom<T>, RQ_NA>();
         if (!A.cP[0] || !A.cP[1] || !A.cP[2]) return cudaErrorInvalidValue;
@@ -1170,7 +1193,7 @@ static cudaError_t launch_u1s_t(const U1Args<T>& A, int what, cudaStream_t s)
             if (e != cudaSuccess) return e;
             rattr = true;
         }
-        k_u1s_plaquette_rates<T><<<grid, U1PGeom<T>::NT, smem, s>>>(A);
+        k_u1s_plaquette_rates<T><<<pgrid, U1PGeom<T>::NT, smem, s>>>(A);
     } else if (what == 2) {
         constexpr size_t smem = u1f_smem_bytes<T>();
         const int form = A.lf ? (A.lf == 2 ? 4 : 3) : ((A.flags & P_FIRST_STAGE) && !(A.flags & P_ENERGY_ONLY) ? 2 : 1);

@@ -106,6 +106,7 @@ struct cl_lattice {
     void* gv[5][2] = {};            // v11, v12, v13, v22, v23 (ping-pong)
     void* gpv[5][2] = {};           // their momenta a^(3-alpha) v'
     int gw_BY = 1, gw_DZ = 1, gw_nby = 1, gw_nbz = 1;
+    int gw_stages = 0, gw_grid = 1;  // staged GW pass: stage buffers (0: the direct one), blocks
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     int64_t last_launches = 0;
     // batched ensemble (members > 1): per-member sizes, boxes, arena offsets and couplings
@@ -486,7 +487,12 @@ cl_status choose_tiles(cl_lattice* l)
         nblocks = (int)(units < wave ? units : wave);
         l->grid = nblocks;
     }
-    if (l->gw) {
+    l->gw_stages = 0;
+    if (l->gw && l->opt_stages != -1 && gw_tma_tiles(prec, l->nf, N, nsm, &l->gw_BY, &l->gw_DZ, &l->gw_stages)) {
+        l->gw_nby = (N + l->gw_BY - 1) / l->gw_BY;
+        l->gw_nbz = (N + l->gw_DZ - 1) / l->gw_DZ;
+        l->gw_grid = std::min(nsm, 5 * l->gw_nby * l->gw_nbz);
+    } else if (l->gw) {
         // GW pass (direct loads, as the Runge-Kutta stage kernel): about 256 threads per block,
         // two blocks per SM, the y tiles cut into z chunks so that about one wave covers the
         // lattice.  (Measured at 256^3 FP32, two fields, Yoshida-4: 10.5 Gsite-updates/s; a pass
@@ -773,7 +779,8 @@ cl_status run_gw_pass_t(cl_lattice* l, const PassCoef& pc, int in, int out)
     A.dx = l->dx; A.alpha = l->p.alpha; A.kappa = l->p.kappa;
     A.d = pc.d; A.k = pc.k;
     A.flags = (pc.flags & P_DRIFT) | (l->p.expansion ? P_EXPANSION : 0);
-    cudaError_t e = launch_gw_pass(l->p.precision, l->nf, &A, l->VW, l->stream);
+    const cudaError_t e = l->gw_stages > 0 ? launch_gw_pass_tma(l->nf, &A, l->gw_stages, l->gw_grid, l->stream)
+                                           : launch_gw_pass(l->p.precision, l->nf, &A, l->VW, l->stream);
     if (e != cudaSuccess) return fail(l, CL_ECUDA, "GW pass launch failed: %s", cudaGetErrorString(e));
     return CL_OK;
 }

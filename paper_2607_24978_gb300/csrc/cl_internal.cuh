@@ -204,7 +204,7 @@ struct GwPassArgs {
     const T* pv_in[5];
     T* v_out[5];
     T* pv_out[5];
-    const DevScal* scal;
+    DevScal* scal;
     int N, BY, DZ, nby, nbz;
     double dx, alpha, kappa;
     double d, k;        // pass coefficients (already x dt), as in ScalarPassArgs; the pass
@@ -213,6 +213,10 @@ struct GwPassArgs {
 };
 cudaError_t launch_gw_pass(int precision, int nf, const void* args, int vw, cudaStream_t s);
 size_t gw_pass_smem(int nf, int N, int BY, int es);
+// The staged pass (gw_pass_tma.cuh): its tiling where it can run (false elsewhere), `grid`
+// persistent blocks.
+bool gw_tma_tiles(int precision, int nf, int N, int nsm, int* BY, int* DZ, int* stages);
+cudaError_t launch_gw_pass_tma(int nf, const void* args, int stages, int grid, cudaStream_t s);
 // TT energy spectrum sums of the five transformed momenta F[5][N][N][N/2+1] (h'_33 = -h'_11 - h'_22)
 cudaError_t launch_gw_bins(const double2* F, int N, double dx, double dn, int nbins, double* S, double* C,
                            cudaStream_t s);

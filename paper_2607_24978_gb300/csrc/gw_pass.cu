@@ -19,13 +19,16 @@
 // amplitudes and its own momentum.
 #include <math.h>
 
+#include <algorithm>
+
 #include "cl_internal.cuh"
 #include "kernel_common.cuh"
 #include "scalar_pass_common.cuh"
 
 namespace clk {
 
-constexpr int kGwC = 5;  // stored components
+constexpr int kGwC = 5;       // stored components
+constexpr int kGwStages = 6;  // stage buffers of the staged pass at most
 
 template <typename T, int NF, bool KAHAN, int VW>
 __global__ void __launch_bounds__(256) k_gw_pass(const GwPassArgs<T> A)
@@ -231,6 +234,8 @@ cudaError_t launch_gw_pass(int precision, int nf, const void* args, int vw, cuda
 }
 
 size_t gw_pass_smem(int nf, int N, int BY, int es) { return (size_t)(nf + kGwC) * 3 * (BY + 2) * N * es; }
+
+#include "gw_pass_tma.cuh"
 
 // ---------------------------------------------------------------- GW energy spectrum
 

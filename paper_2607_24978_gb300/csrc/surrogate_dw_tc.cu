@@ -20,15 +20,20 @@
 // The first group stages h of plane z-1: rows 0-63 accumulate the tz = 0 taps of output
 // plane z and rows 64-127 the tz = 1 taps of plane z-1 (each plane is the z-1 of exactly
 // one unit, periodic in z).  The second group stages h of plane z+1 (tz = 2; its rows
-// 64-127 stay zero).  B carries one more channel block that holds the constant 1 (and a
-// zero block to round N up to a multiple of 16): the first x tap's MMA (N = 3 CIP + 16)
-// then also accumulates db[co] = sum_n g[n][co].  A block accumulates its units in TMEM
-// and writes one partial per tap (and per bias); a second kernel sums the partials in a
-// fixed order.
+// 64-127 stay zero) and multiplies g by a constant block of ones as well (N = 16), which sums
+// db[co] = sum_n g[n][co].  A block accumulates its units in TMEM and writes one partial per
+// tap (and per bias); a second kernel sums the partials in a fixed order.
+//
+// A block's units follow each other in y, so a unit needs one new row of h: the rows live in a
+// ring of their own (kDwRowsExtra more than the units in flight, which keeps every row that an
+// unfinished unit reads), and an MMA is split in two where its three rows wrap around the ring.
+// Staging all three rows with every unit moved 4.5 GB through L2 for a 48-channel layer at 128^3,
+// 9 TB/s in 500 us.
 //
 // Warp roles, synchronised by mbarriers only: warp 0, lane 0 issues the MMAs; warps 1-3
-// stage units with cp.async into a ring of slots; warps 4-7 read the accumulators back at
-// the end.  All waits are bounded and report through the status word.
+// stage units with cp.async (FP32 operands: loaded into registers a unit ahead, converted while
+// the copies of the unit before land); warps 4-7 read the accumulators back at the end.  All
+// waits are bounded and report through the status word.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -39,42 +44,38 @@
 
 namespace clk {
 
-constexpr int kDwMaxSlots = 4;
-constexpr int kDwStage = 96;  // staging threads (warps 1-3)
+constexpr int kDwMaxSlots = 4;   // units in flight (slots of A) at most
+constexpr int kDwStage = 96;     // staging threads (warps 1-3)
+// Rows of the h ring beyond the units in flight: a unit reads three rows, and the next one's rows
+// start one further, or three further where a new plane begins (at most once in kDwMaxSlots
+// units, N being 16 or more).  When unit s is staged, unit s - slots is done; the rows of the
+// slots - 1 units in between and of s itself number at most slots - 1 + 2 + 3 = slots + 4.
+constexpr int kDwRowsExtra = 4;
+constexpr int kDwF32 = 8;        // FP32 entries a staging thread holds a unit ahead
 
-// 16-byte entries of one slot: A (16 channel blocks of N + 1 sites, the +1 spreads the
-// blocks over the shared-memory banks) and B (3 rows x CIP/8 groups, then the ones block and
-// a zero block, of N + 2 sites each).
+// 16-byte entries of an A slot (16 channel blocks of N + 1 sites, the +1 spreads the blocks over
+// the shared-memory banks), of a row of h (CIP / 8 groups of N + 2 sites), and of the block of
+// ones and its zero block (16 sites each).
 __host__ __device__ inline int dw_a_entries(int N) { return 16 * (N + 1); }
-__host__ __device__ inline int dw_slot_entries(int CIP, int N) { return dw_a_entries(N) + (3 * (CIP / 8) + 2) * (N + 2); }
+__host__ __device__ inline int dw_row_entries(int CIP, int N) { return (CIP / 8) * (N + 2); }
+constexpr int kDwOnes = 32;
 
 template <int CIP, int COP>
 struct DwTCShape {
     static constexpr int CGA = COP / 8;     // channel groups of g (A, per half)
     static constexpr int CG = CIP / 8;      // channel groups of h (B)
     static constexpr int NT = 3 * CIP;      // MMA N of an x tap: three y taps x CIP input channels
-    static constexpr int NT1 = NT + 16;     // first x tap: plus the ones (bias) block
-    static constexpr int COLS = NT1 + 2 * NT;
+    static constexpr int COLS = 3 * NT + 16;  // the x taps, then the ones (bias) block
     static constexpr int TMEM_COLS = COLS <= 256 ? 256 : 512;
     static_assert(COLS <= 512, "accumulators exceed TMEM");
     static_assert(kDwStage % CGA == 0 && kDwStage % CG == 0, "staging threads per channel group");
 };
 
-// 16-byte entry of 8 channels (from channel c0) of FP32 site data with `nc` channels, BF16,
-// zero beyond nc.
-__device__ __forceinline__ uint4 f32_entry(const float* site, int nc, int c0)
-{
-    float f[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) f[c] = c0 + c < nc ? __ldg(site + c0 + c) : 0.f;
-    return pack_bf16x8(f);
-}
-
 template <int CIP, int COP, bool GF32, bool HF32>
 __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
 {
     using S = DwTCShape<CIP, COP>;
-    constexpr int CGA = S::CGA, CG = S::CG, NT = S::NT, NT1 = S::NT1;
+    constexpr int CGA = S::CGA, CG = S::CG, NT = S::NT;
     extern __shared__ __align__(128) uint4 smem[];
     __shared__ __align__(8) uint64_t s_full[kDwMaxSlots];   // unit staged in the slot (96 arrivals)
     __shared__ __align__(8) uint64_t s_freeb[kDwMaxSlots];  // slot's unit read by its MMAs (commit)
@@ -82,26 +83,31 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int N = A.N, NS = A.nslot, grp = blockIdx.y;
+    const int N = A.N, NS = A.nslot, HR = NS + kDwRowsExtra, grp = blockIdx.y;
     const int AST = N + 1, BST = N + 2;  // entries between channel blocks of A, of B
-    const int AENT = dw_a_entries(N), SLOT = dw_slot_entries(CIP, N);
+    const int AENT = dw_a_entries(N), ROW = dw_row_entries(CIP, N);
+    uint4* const hring = smem + (size_t)NS * AENT;
+    uint4* const ones = hring + (size_t)HR * ROW;
     const long long units = (long long)N * N;
     const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
     const int nblk_a = grp == 0 ? 2 : 1;  // g rows staged into A (rows 0-63, and 64-127)
+    // channel groups that are staged: FP32 operands have at most three channels, one group
+    constexpr int GA = GF32 ? 1 : CGA, GB = HF32 ? 1 : CG;
 
-    // constant blocks, written once: the padding channel blocks of A (zero), and the ones
-    // block (channel 0 = 1) and zero block that follow the h rows in B
+    // constant blocks, written once: the padding channel blocks of A and of the h rows (zero), and
+    // the block of ones (channel 0 = 1) beside a zero block
     for (int s = 0; s < NS; ++s) {
-        uint4* sa = smem + (size_t)s * SLOT;
+        uint4* sa = smem + (size_t)s * AENT;
         for (int e = tid; e < 16 * AST; e += blockDim.x) {
             const int b = e / AST;
-            const bool used = (b < CGA) || (nblk_a == 2 && b >= 8 && b < 8 + CGA);
+            const bool used = (b < GA) || (nblk_a == 2 && b >= 8 && b < 8 + GA);
             if (!used) sa[e] = make_uint4(0u, 0u, 0u, 0u);
         }
-        uint4* sk = sa + AENT + 3 * CG * BST;
-        const uint4 one = make_uint4(0x3F80u, 0u, 0u, 0u);  // BF16 1.0 in channel 0
-        for (int e = tid; e < 2 * BST; e += blockDim.x) sk[e] = e < BST ? one : make_uint4(0u, 0u, 0u, 0u);
     }
+    if (GB < CG)
+        for (int e = tid; e < HR * ROW; e += blockDim.x)
+            if (e % ROW >= GB * BST) hring[e] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < kDwOnes) ones[tid] = make_uint4(tid < kDwOnes / 2 ? 0x3F80u : 0u, 0u, 0u, 0u);  // BF16 1.0
     if (tid == 0) {
         for (int k = 0; k < NS; ++k) {
             mbar_init(&s_full[k], kDwStage);
@@ -127,27 +133,42 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
 
     if (warp == 0) {
         // ------------------------------------------------------------ MMA issuer
-        // accumulator columns: x tap 0 (with the bias block) [0, NT1), x tap 1 [NT1, NT1 + NT),
-        // x tap 2 [NT1 + NT, NT1 + 2 NT)
+        // accumulator columns: x tap dx at dx NT, the bias at 3 NT
         if (lane == 0) {
             uint32_t full_ph = 0;
-            int seq = 0;
-            constexpr uint32_t idesc0 = idesc_bf16_mn(128, NT1), idesc = idesc_bf16_mn(128, NT);
-            const uint32_t sbo_a = (uint32_t)AST * 16, sbo_b = (uint32_t)BST * 16;
+            int seq = 0, row = 0;  // ring slot of the unit's row y - 1
+            const uint32_t sbo_a = (uint32_t)AST * 16, sbo_b = (uint32_t)BST * 16, h0 = smem_u32(hring);
+            const uint64_t odesc = smem_desc(smem_u32(ones), 128, kDwOnes / 2 * 16);
+            constexpr uint32_t idesc1 = idesc_bf16_mn(128, 16);
+            int y = (int)(u0 % N);
             for (long long u = u0; u < u1; ++u, ++seq) {
                 const int slot = seq % NS;
                 wait(&s_full[slot], full_ph, slot);
                 tc_fence_after();
-                const uint32_t a0 = smem_u32(smem + (size_t)slot * SLOT), b0 = a0 + (uint32_t)AENT * 16;
+                const uint32_t a0 = smem_u32(smem + (size_t)slot * AENT);
+                // the rows y-1, y, y+1: n1 of them before the ring's end, the others from its start
+                const int n1 = min(3, HR - row);
+                const uint32_t b1 = h0 + (uint32_t)(row * ROW) * 16;
+                const uint32_t id1 = idesc_bf16_mn(128, CIP) + (uint32_t)((n1 - 1) * (CIP >> 3) << 17);
+                const uint32_t id2 = idesc_bf16_mn(128, CIP) + (uint32_t)((2 - n1) * (CIP >> 3) << 17);
 #pragma unroll 1
                 for (int kc = 0; kc < N / 16; ++kc) {
                     const uint64_t adesc = smem_desc(a0 + kc * 256, 128, sbo_a);
                     const uint32_t acc = (u == u0 && kc == 0) ? 0u : 1u;
-                    tc_mma(tbase, adesc, smem_desc(b0 + kc * 256, 128, sbo_b), idesc0, acc);
-                    tc_mma(tbase + NT1, adesc, smem_desc(b0 + kc * 256 + 16, 128, sbo_b), idesc, acc);
-                    tc_mma(tbase + NT1 + NT, adesc, smem_desc(b0 + kc * 256 + 32, 128, sbo_b), idesc, acc);
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+                        tc_mma(tbase + dx * NT, adesc, smem_desc(b1 + kc * 256 + dx * 16, 128, sbo_b), id1, acc);
+                    if (n1 < 3) {
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx)
+                            tc_mma(tbase + dx * NT + n1 * CIP, adesc, smem_desc(h0 + kc * 256 + dx * 16, 128, sbo_b), id2, acc);
+                    }
+                    if (grp == 1) tc_mma(tbase + 3 * NT, adesc, odesc, idesc1, acc);
                 }
                 tc_commit(&s_freeb[slot]);  // the slot may be restaged once these MMAs completed
+                y = y + 1 == N ? 0 : y + 1;
+                row += y == 0 ? 3 : 1;  // a new plane starts with three rows of its own
+                if (row >= HR) row -= HR;
             }
             if (u1 > u0) tc_commit(&s_done);
         }
@@ -158,44 +179,94 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
         // through the sites: no division in the loops.
         const int st = tid - 32;
         const int dzh = grp == 0 ? -1 : 1;  // plane of h relative to the unit
-        constexpr int SXA = kDwStage / CGA, SXB = kDwStage / CG;
-        const int cga = st % CGA, xa0 = st / CGA;
-        const int cgb = st % CG, pb0 = st / CG;
+        constexpr int SXA = kDwStage / GA, SXB = kDwStage / GB;
+        const int cga = st % GA, xa0 = st / GA;
+        const int cgb = st % GB, pb0 = st / GB;
         uint32_t free_ph = 0;
-        int seq = 0, pend_slot = -1;
+        int seq = 0, pend_slot = -1, row = 0;
         auto land = [&](int slot) {
             fence_proxy_async_smem();
             mbar_arrive(&s_full[slot]);
         };
+        auto wrap = [&](int v) { return v < 0 ? v + N : (v >= N ? v - N : v); };
+        // FP32 operands: channels (up to three) of the entries xa0, xa0 + 96, .. of the unit's g
+        // rows, or pb0, pb0 + 96, .. of its row y + 1 of h, in registers
+        float fr[kDwF32][3];
+        auto site3 = [&](const float* p, int nc, float (&f)[3]) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f[c] = c < nc ? __ldg(p + c) : 0.f;
+        };
+        auto entry3 = [&](const float (&f)[3]) {
+            const float v[8] = {f[0], f[1], f[2], 0.f, 0.f, 0.f, 0.f, 0.f};
+            return pack_bf16x8(v);
+        };
+        auto load_f32 = [&](long long u) {
+            if constexpr (GF32) {
+                const int z = (int)(u / N), y = (int)(u - (long long)z * N);
+#pragma unroll
+                for (int i = 0; i < kDwF32; ++i) {
+                    const int e = xa0 + i * kDwStage, half = e >= N ? 1 : 0, x = e - half * N;
+                    if (e < nblk_a * N)
+                        site3(reinterpret_cast<const float*>(A.g) + (((size_t)(half ? wrap(z - 1) : z) * N + y) * N + x) * A.g_c,
+                              A.g_c, fr[i]);
+                }
+            }
+            if constexpr (HF32) {
+                const int z = (int)(u / N), y = (int)(u - (long long)z * N);
+                const size_t r0 = ((size_t)wrap(z + dzh) * N + wrap(y + 1)) * N;
+#pragma unroll
+                for (int i = 0; i < kDwF32; ++i) {
+                    const int p = pb0 + i * kDwStage;
+                    if (p < BST) site3(reinterpret_cast<const float*>(A.h) + (r0 + wrap(p - 1)) * A.h_c, A.h_c, fr[i]);
+                }
+            }
+        };
+        if (u1 > u0) load_f32(u0);
         for (long long u = u0; u < u1; ++u, ++seq) {
             const int slot = seq % NS;
             if (seq >= NS) wait(&s_freeb[slot], free_ph, slot);
             const int z = (int)(u / N), y = (int)(u - (long long)z * N);
-            uint4* sa = smem + (size_t)slot * SLOT;
-            uint4* sb = sa + AENT;
+            uint4* sa = smem + (size_t)slot * AENT;
             // A: g of row (z, y) into channel blocks 0.., and of row (z-1, y) into blocks 8..
-            for (int half = 0; half < nblk_a; ++half) {
-                const int zz = half == 0 ? z : (z == 0 ? N - 1 : z - 1);
-                const size_t row = ((size_t)zz * N + y) * N;
-                uint4* d = sa + (half * 8 + cga) * AST;
-                for (int x = xa0; x < N; x += SXA) {
-                    if (!GF32) cp_async16(d + x, reinterpret_cast<const __nv_bfloat16*>(A.g) + (row + x) * COP + cga * 8);
-                    else d[x] = f32_entry(reinterpret_cast<const float*>(A.g) + (row + x) * A.g_c, A.g_c, cga * 8);
-                }
-            }
-            // B: h of rows y-1, y, y+1 of plane z + dzh, x from -1 to N (periodic)
-            const int zh = z + dzh < 0 ? N - 1 : (z + dzh >= N ? 0 : z + dzh);
+            if constexpr (GF32) {
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-                const int yy = y + dy - 1 < 0 ? N - 1 : (y + dy - 1 >= N ? 0 : y + dy - 1);
-                const size_t row = ((size_t)zh * N + yy) * N;
-                uint4* d = sb + (dy * CG + cgb) * BST;
-                for (int p = pb0; p < BST; p += SXB) {
-                    const int xx = p == 0 ? N - 1 : (p == N + 1 ? 0 : p - 1);
-                    if (!HF32) cp_async16(d + p, reinterpret_cast<const __nv_bfloat16*>(A.h) + (row + xx) * CIP + cgb * 8);
-                    else d[p] = f32_entry(reinterpret_cast<const float*>(A.h) + (row + xx) * A.h_c, A.h_c, cgb * 8);
+                for (int i = 0; i < kDwF32; ++i) {
+                    const int e = xa0 + i * kDwStage, half = e >= N ? 1 : 0;
+                    if (e < nblk_a * N) sa[half * 8 * AST + (e - half * N)] = entry3(fr[i]);
+                }
+            } else {
+                for (int half = 0; half < nblk_a; ++half) {
+                    const size_t r0 = ((size_t)(half ? wrap(z - 1) : z) * N + y) * N;
+                    uint4* d = sa + (half * 8 + cga) * AST;
+                    for (int x = xa0; x < N; x += SXA)
+                        cp_async16(d + x, reinterpret_cast<const __nv_bfloat16*>(A.g) + (r0 + x) * COP + cga * 8);
                 }
             }
+            // B: h of row y+1 of plane z + dzh, x from -1 to N (periodic); at the start of a plane
+            // (and of the block) the rows y-1 and y before it
+            const int zh = wrap(z + dzh);
+            for (int dy = (u == u0 || y == 0) ? 0 : 2; dy < 3; ++dy) {
+                const int rs = row + dy >= HR ? row + dy - HR : row + dy;
+                const size_t r0 = ((size_t)zh * N + wrap(y + dy - 1)) * N;
+                uint4* d = hring + (size_t)rs * ROW + cgb * BST;
+                if constexpr (HF32) {
+#pragma unroll
+                    for (int i = 0; i < kDwF32; ++i) {
+                        const int p = pb0 + i * kDwStage;
+                        if (p < BST) {
+                            float f[3];
+                            if (dy < 2) site3(reinterpret_cast<const float*>(A.h) + (r0 + wrap(p - 1)) * A.h_c, A.h_c, f);
+                            d[p] = entry3(dy < 2 ? f : fr[i]);
+                        }
+                    }
+                } else {
+                    for (int p = pb0; p < BST; p += SXB)
+                        cp_async16(d + p, reinterpret_cast<const __nv_bfloat16*>(A.h) + (r0 + wrap(p - 1)) * CIP + cgb * 8);
+                }
+            }
+            row += y + 1 == N ? 3 : 1;
+            if (row >= HR) row -= HR;
+            if (u + 1 < u1) load_f32(u + 1);
             cp_async_commit();
             if (pend_slot >= 0) {  // the previous unit's copies have landed once one group is left
                 cp_async_wait1();
@@ -231,7 +302,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
         };
 #pragma unroll 1
         for (int dx = 0; dx < 3; ++dx) {
-            const int cbase = dx == 0 ? 0 : NT1 + (dx - 1) * NT;
+            const int cbase = dx * NT;
 #pragma unroll 1
             for (int c16 = 0; c16 < NT / 16; ++c16) {
                 uint32_t raw[16];
@@ -249,7 +320,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
         }
         {  // the ones column: sum of g over this block's sites (the second group's rows 0-63)
             uint32_t raw[16];
-            load16(NT, raw);
+            load16(3 * NT, raw);
             if (grp == 1 && half == 0 && co < COP) A.bpart[(size_t)blockIdx.x * COP + co] = __uint_as_float(raw[0]);
         }
         tc_fence_before();
@@ -286,11 +357,17 @@ __global__ void k_conv_dw_tc_reduce(const ConvDWTCArgs A, int CIP, int COP)
     }
 }
 
-size_t conv_dw_tc_smem(int CIP, int N, int nslot) { return (size_t)nslot * dw_slot_entries(CIP, N) * 16; }
+size_t conv_dw_tc_smem(int CIP, int N, int nslot)
+{
+    return ((size_t)nslot * dw_a_entries(N) + (size_t)(nslot + kDwRowsExtra) * dw_row_entries(CIP, N) + kDwOnes) * 16;
+}
 
 int conv_dw_tc_slots(int CIP, int N)
 {
     if ((CIP != 16 && CIP != 32 && CIP != 48) || N < 16 || N % 16 != 0) return 0;
+    // larger lattices keep their weight gradients in FP32 on the CUDA cores
+    if (N > (CIP == 16 ? 288 : CIP == 32 ? 224 : 192)) return 0;
+    static_assert(2 * 288 <= kDwF32 * kDwStage, "FP32 entries a staging thread holds");
     for (int s = kDwMaxSlots; s >= 2; --s)
         if (conv_dw_tc_smem(CIP, N, s) <= (size_t)kPassMaxSmem) return s;
     return 0;

@@ -265,7 +265,7 @@ cl_status cl_surrogate_create(cl_surrogate** out, const cl_surrogate_params* p)
          cudaMalloc(&s->dx, (size_t)s->V * p->in_channels * 4) == cudaSuccess &&
          cudaMalloc(&s->partial, part * 4) == cudaSuccess && cudaMalloc(&s->status, sizeof(int)) == cudaSuccess &&
          cudaMemset(s->status, 0, sizeof(int)) == cudaSuccess;
-    if (ok && p->precision == CL_SG_BF16 && conv_dw_tc_slots(16, p->N) >= 2) {
+    if (ok && p->precision == CL_SG_BF16 && conv_dw_tc_slots(16, 16, p->N) >= 2) {
         // weight gradients on the tensor cores: about 64 or more rows per block, two tap
         // groups sharing the SMs; partials sized for the widest layer (hidden x hidden)
         const int C = p->hidden;
@@ -372,7 +372,7 @@ cl_status cl_surrogate_backward(cl_surrogate* s, const float* g, float* dx, int3
         // BF16 mode: every layer's weight gradients on the tensor cores (the thin FP32 network
         // input and loss gradient are rounded to BF16 while staged, as in the forward)
         const int cip = tc_width(s->cin[l]), cop = tc_width(s->cout[l]);
-        if (s->dw_nb > 0 && !h_act && conv_dw_tc_slots(cip, s->p.N) >= 2) {
+        if (s->dw_nb > 0 && !h_act && conv_dw_tc_slots(cip, cop, s->p.N) >= 2) {
             ConvDWTCArgs A{};
             A.h = h;
             A.h_f32 = h_bf16 ? 0 : 1;
@@ -383,7 +383,7 @@ cl_status cl_surrogate_backward(cl_surrogate* s, const float* g, float* dx, int3
             A.CI = s->cin[l];
             A.CO = s->cout[l];
             A.N = s->p.N;
-            A.nslot = conv_dw_tc_slots(cip, s->p.N);
+            A.nslot = conv_dw_tc_slots(cip, cop, s->p.N);
             A.nb = s->dw_nb;
             A.part0 = s->dw_part0;
             A.part1 = s->dw_part1;

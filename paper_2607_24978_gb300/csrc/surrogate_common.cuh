@@ -144,7 +144,7 @@ struct ConvDWTCArgs {
     int g_f32, g_c;
     int CI, CO;                 // real channels (the padded ones read as zeros)
     int N;                      // multiple of 16
-    int nslot;                  // staging slots, 2 .. conv_dw_tc_slots(CIP, N)
+    int nslot;                  // staging slots, 2 .. conv_dw_tc_slots(CIP, COP, N)
     int nb;                     // blocks per tap group (grid nb x 2)
     float* part0;               // [nb][18][COP][CIP]: taps of planes tz = 0, 1
     float* part1;               // [nb][9][COP][CIP]: taps of plane tz = 2
@@ -153,8 +153,7 @@ struct ConvDWTCArgs {
     float* db;                  // [CO]
     int* status;                // ST_TIMEOUT on a bounded wait that gave up
 };
-int conv_dw_tc_slots(int CIP, int N);  // 0: shape not supported on the tensor cores
-size_t conv_dw_tc_smem(int CIP, int N, int nslot);
+int conv_dw_tc_slots(int CIP, int COP, int N);  // 0: shape not supported on the tensor cores
+size_t conv_dw_tc_smem(int CIP, int COP, int N, int nslot);
 cudaError_t launch_conv_dw_tc(int CIP, int COP, const ConvDWTCArgs& A, cudaStream_t s);
-
 }  // namespace clk

@@ -15,12 +15,11 @@
 //  * B (N rows) is h of the three rows y-1, y, y+1 of one plane, staged [row][group][x]
 //    with a one-site periodic halo in x: the 3 CIP rows (y tap, input channel) are evenly
 //    strided, so the three y taps are one MMA (N = 3 CIP);
-//  * A (M = 128 rows) is g of row (z, y) in rows 0-63 (channels padded with zeros) and, in
-//    the first block group, g of row (z-1, y) in rows 64-127.
-// The first group stages h of plane z-1: rows 0-63 accumulate the tz = 0 taps of output
-// plane z and rows 64-127 the tz = 1 taps of plane z-1 (each plane is the z-1 of exactly
-// one unit, periodic in z).  The second group stages h of plane z+1 (tz = 2; its rows
-// 64-127 stay zero) and multiplies g by a constant block of ones as well (N = 16), which sums
+//  * A (M = 128 rows) is g of row (z, y) in rows 0 .. COP-1 and, in the first block group, g of
+//    row (z-1, y) in the COP rows after them; the other rows are nobody's.
+// The first group stages h of plane z-1: the first rows accumulate the tz = 0 taps of output
+// plane z and the next ones the tz = 1 taps of plane z-1 (each plane is the z-1 of exactly
+// one unit, periodic in z).  The second group stages h of plane z+1 (tz = 2) and multiplies g by a constant block of ones as well (N = 16), which sums
 // db[co] = sum_n g[n][co].  A block accumulates its units in TMEM and writes one partial per
 // tap (and per bias); a second kernel sums the partials in a fixed order.
 //
@@ -30,9 +29,10 @@
 // Staging all three rows with every unit moved 4.5 GB through L2 for a 48-channel layer at 128^3,
 // 9 TB/s in 500 us.
 //
-// Warp roles, synchronised by mbarriers only: warp 0, lane 0 issues the MMAs; warps 1-3
-// stage units with cp.async (FP32 operands: loaded into registers a unit ahead, converted while
-// the copies of the unit before land); warps 4-7 read the accumulators back at the end.  All
+// Warp roles, synchronised by mbarriers only: warp 0, lane 0 issues the MMAs; warps 1-6 stage
+// units with cp.async, whose arrivals on the slot's barrier come when they land, as many units
+// ahead as there are slots (FP32 operands: loaded into registers a unit ahead, converted and
+// stored); warps 7-10 read the accumulators back at the end.  All
 // waits are bounded and report through the status word.
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -44,19 +44,21 @@
 
 namespace clk {
 
-constexpr int kDwMaxSlots = 4;   // units in flight (slots of A) at most
-constexpr int kDwStage = 96;     // staging threads (warps 1-3)
+constexpr int kDwMaxSlots = 6;   // units in flight (slots of A) at most
+constexpr int kDwStage = 192;    // staging threads (warps 1-6)
 // Rows of the h ring beyond the units in flight: a unit reads three rows, and the next one's rows
 // start one further, or three further where a new plane begins (at most once in kDwMaxSlots
 // units, N being 16 or more).  When unit s is staged, unit s - slots is done; the rows of the
 // slots - 1 units in between and of s itself number at most slots - 1 + 2 + 3 = slots + 4.
 constexpr int kDwRowsExtra = 4;
-constexpr int kDwF32 = 8;        // FP32 entries a staging thread holds a unit ahead
+constexpr int kDwThreads = 32 + kDwStage + 128;
+constexpr int kDwF32 = 4;        // FP32 entries a staging thread holds a unit ahead
 
-// 16-byte entries of an A slot (16 channel blocks of N + 1 sites, the +1 spreads the blocks over
-// the shared-memory banks), of a row of h (CIP / 8 groups of N + 2 sites), and of the block of
-// ones and its zero block (16 sites each).
-__host__ __device__ inline int dw_a_entries(int N) { return 16 * (N + 1); }
+// 16-byte entries of an A slot (the channel blocks of the two g rows, N + 1 sites each: the +1
+// spreads the blocks over the shared-memory banks; an MMA's M = 128 rows read 16 blocks, those past
+// the slot into whatever follows, rows of the accumulator that nobody reads), of a row of h (CIP / 8
+// groups of N + 2 sites), and of the block of ones and its zero block (16 sites each).
+__host__ __device__ inline int dw_a_entries(int COP, int N) { return 2 * (COP / 8) * (N + 1); }
 __host__ __device__ inline int dw_row_entries(int CIP, int N) { return (CIP / 8) * (N + 2); }
 constexpr int kDwOnes = 32;
 
@@ -72,12 +74,12 @@ struct DwTCShape {
 };
 
 template <int CIP, int COP, bool GF32, bool HF32>
-__global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
+__global__ void __launch_bounds__(kDwThreads, 1) k_conv_dw_tc(const ConvDWTCArgs A)
 {
     using S = DwTCShape<CIP, COP>;
     constexpr int CGA = S::CGA, CG = S::CG, NT = S::NT;
     extern __shared__ __align__(128) uint4 smem[];
-    __shared__ __align__(8) uint64_t s_full[kDwMaxSlots];   // unit staged in the slot (96 arrivals)
+    __shared__ __align__(8) uint64_t s_full[kDwMaxSlots];   // unit staged in the slot (an arrival a staging thread)
     __shared__ __align__(8) uint64_t s_freeb[kDwMaxSlots];  // slot's unit read by its MMAs (commit)
     __shared__ __align__(8) uint64_t s_done;                // every MMA of the block complete (commit)
     __shared__ uint32_t s_tmem;
@@ -85,32 +87,22 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int N = A.N, NS = A.nslot, HR = NS + kDwRowsExtra, grp = blockIdx.y;
     const int AST = N + 1, BST = N + 2;  // entries between channel blocks of A, of B
-    const int AENT = dw_a_entries(N), ROW = dw_row_entries(CIP, N);
+    const int AENT = dw_a_entries(COP, N), ROW = dw_row_entries(CIP, N);
     uint4* const hring = smem + (size_t)NS * AENT;
     uint4* const ones = hring + (size_t)HR * ROW;
     const long long units = (long long)N * N;
     const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
-    const int nblk_a = grp == 0 ? 2 : 1;  // g rows staged into A (rows 0-63, and 64-127)
+    const int nblk_a = grp == 0 ? 2 : 1;  // g rows staged into A
     // channel groups that are staged: FP32 operands have at most three channels, one group
     constexpr int GA = GF32 ? 1 : CGA, GB = HF32 ? 1 : CG;
 
-    // constant blocks, written once: the padding channel blocks of A and of the h rows (zero), and
+    // zeros once: channels that are not staged, and everything an MMA may read past an A slot
+    for (int e = tid; e < NS * AENT + HR * ROW; e += blockDim.x) smem[e] = make_uint4(0u, 0u, 0u, 0u);
     // the block of ones (channel 0 = 1) beside a zero block
-    for (int s = 0; s < NS; ++s) {
-        uint4* sa = smem + (size_t)s * AENT;
-        for (int e = tid; e < 16 * AST; e += blockDim.x) {
-            const int b = e / AST;
-            const bool used = (b < GA) || (nblk_a == 2 && b >= 8 && b < 8 + GA);
-            if (!used) sa[e] = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
-    if (GB < CG)
-        for (int e = tid; e < HR * ROW; e += blockDim.x)
-            if (e % ROW >= GB * BST) hring[e] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < kDwOnes) ones[tid] = make_uint4(tid < kDwOnes / 2 ? 0x3F80u : 0u, 0u, 0u, 0u);  // BF16 1.0
     if (tid == 0) {
         for (int k = 0; k < NS; ++k) {
-            mbar_init(&s_full[k], kDwStage);
+            mbar_init(&s_full[k], kDwStage * (1 + (GF32 || HF32)));  // copies landed (, stores done)
             mbar_init(&s_freeb[k], 1);
         }
         mbar_init(&s_done, 1);
@@ -144,26 +136,31 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
             for (long long u = u0; u < u1; ++u, ++seq) {
                 const int slot = seq % NS;
                 wait(&s_full[slot], full_ph, slot);
+                fence_proxy_async_smem();  // the copies wrote through the generic proxy
                 tc_fence_after();
-                const uint32_t a0 = smem_u32(smem + (size_t)slot * AENT);
                 // the rows y-1, y, y+1: n1 of them before the ring's end, the others from its start
                 const int n1 = min(3, HR - row);
-                const uint32_t b1 = h0 + (uint32_t)(row * ROW) * 16;
                 const uint32_t id1 = idesc_bf16_mn(128, CIP) + (uint32_t)((n1 - 1) * (CIP >> 3) << 17);
                 const uint32_t id2 = idesc_bf16_mn(128, CIP) + (uint32_t)((2 - n1) * (CIP >> 3) << 17);
-#pragma unroll 1
-                for (int kc = 0; kc < N / 16; ++kc) {
-                    const uint64_t adesc = smem_desc(a0 + kc * 256, 128, sbo_a);
-                    const uint32_t acc = (u == u0 && kc == 0) ? 0u : 1u;
-#pragma unroll
-                    for (int dx = 0; dx < 3; ++dx)
-                        tc_mma(tbase + dx * NT, adesc, smem_desc(b1 + kc * 256 + dx * 16, 128, sbo_b), id1, acc);
+                // descriptors of chunk 0; one step of their start address is 16 bytes: a chunk of 16
+                // sites is 16 steps on, an x tap one.  One thread issues every MMA, so what it
+                // computes for each is time the tensor core waits: building both descriptors per
+                // MMA took 160 cycles each, where M = 128, N = 144 runs at 72
+                uint64_t ad = smem_desc(smem_u32(smem + (size_t)slot * AENT), 128, sbo_a);
+                uint64_t b1 = smem_desc(h0 + (uint32_t)(row * ROW) * 16, 128, sbo_b), b2 = smem_desc(h0, 128, sbo_b);
+                const uint32_t t2 = tbase + n1 * CIP;
+                uint32_t acc = u == u0 ? 0u : 1u;
+#pragma unroll 2
+                for (int kc = 0; kc < N / 16; ++kc, ad += 16, b1 += 16, b2 += 16, acc = 1u) {
+                    tc_mma(tbase, ad, b1, id1, acc);
+                    tc_mma(tbase + NT, ad, b1 + 1, id1, acc);
+                    tc_mma(tbase + 2 * NT, ad, b1 + 2, id1, acc);
                     if (n1 < 3) {
-#pragma unroll
-                        for (int dx = 0; dx < 3; ++dx)
-                            tc_mma(tbase + dx * NT + n1 * CIP, adesc, smem_desc(h0 + kc * 256 + dx * 16, 128, sbo_b), id2, acc);
+                        tc_mma(t2, ad, b2, id2, acc);
+                        tc_mma(t2 + NT, ad, b2 + 1, id2, acc);
+                        tc_mma(t2 + 2 * NT, ad, b2 + 2, id2, acc);
                     }
-                    if (grp == 1) tc_mma(tbase + 3 * NT, adesc, odesc, idesc1, acc);
+                    if (grp == 1) tc_mma(tbase + 3 * NT, ad, odesc, idesc1, acc);
                 }
                 tc_commit(&s_freeb[slot]);  // the slot may be restaged once these MMAs completed
                 y = y + 1 == N ? 0 : y + 1;
@@ -173,7 +170,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
             if (u1 > u0) tc_commit(&s_done);
         }
         __syncwarp();
-    } else if (warp < 4) {
+    } else if (warp < 1 + kDwStage / 32) {
         // ------------------------------------------------------------ staging warps
         // Each thread keeps one channel group (its index mod the groups of a site) and steps
         // through the sites: no division in the loops.
@@ -183,11 +180,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
         const int cga = st % GA, xa0 = st / GA;
         const int cgb = st % GB, pb0 = st / GB;
         uint32_t free_ph = 0;
-        int seq = 0, pend_slot = -1, row = 0;
-        auto land = [&](int slot) {
-            fence_proxy_async_smem();
-            mbar_arrive(&s_full[slot]);
-        };
+        int seq = 0, row = 0;
         auto wrap = [&](int v) { return v < 0 ? v + N : (v >= N ? v - N : v); };
         // FP32 operands: channels (up to three) of the entries xa0, xa0 + 96, .. of the unit's g
         // rows, or pb0, pb0 + 96, .. of its row y + 1 of h, in registers
@@ -227,17 +220,17 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
             if (seq >= NS) wait(&s_freeb[slot], free_ph, slot);
             const int z = (int)(u / N), y = (int)(u - (long long)z * N);
             uint4* sa = smem + (size_t)slot * AENT;
-            // A: g of row (z, y) into channel blocks 0.., and of row (z-1, y) into blocks 8..
+            // A: g of row (z, y) into channel blocks 0.., and of row (z-1, y) into the blocks after them
             if constexpr (GF32) {
 #pragma unroll
                 for (int i = 0; i < kDwF32; ++i) {
                     const int e = xa0 + i * kDwStage, half = e >= N ? 1 : 0;
-                    if (e < nblk_a * N) sa[half * 8 * AST + (e - half * N)] = entry3(fr[i]);
+                    if (e < nblk_a * N) sa[half * CGA * AST + (e - half * N)] = entry3(fr[i]);
                 }
             } else {
                 for (int half = 0; half < nblk_a; ++half) {
                     const size_t r0 = ((size_t)(half ? wrap(z - 1) : z) * N + y) * N;
-                    uint4* d = sa + (half * 8 + cga) * AST;
+                    uint4* d = sa + (half * CGA + cga) * AST;
                     for (int x = xa0; x < N; x += SXA)
                         cp_async16(d + x, reinterpret_cast<const __nv_bfloat16*>(A.g) + (r0 + x) * COP + cga * 8);
                 }
@@ -266,30 +259,28 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
             }
             row += y + 1 == N ? 3 : 1;
             if (row >= HR) row -= HR;
-            if (u + 1 < u1) load_f32(u + 1);
-            cp_async_commit();
-            if (pend_slot >= 0) {  // the previous unit's copies have landed once one group is left
-                cp_async_wait1();
-                land(pend_slot);
+            // the slot is full when every thread's copies have landed: the arrivals come by
+            // themselves, so the next unit's copies wait for its slot only
+            cp_async_arrive(&s_full[slot]);
+            if constexpr (GF32 || HF32) {
+                fence_proxy_async_smem();
+                mbar_arrive(&s_full[slot]);
             }
-            pend_slot = slot;
+            if (u + 1 < u1) load_f32(u + 1);
         }
-        if (pend_slot >= 0) {
-            cp_async_wait0();
-            land(pend_slot);
-        }
+        cp_async_wait0();
     } else {
         // ------------------------------------------------------------ epilogue warps
         const int q = warp & 3;           // TMEM lane quarter of this warp
         const int r = 32 * q + lane;      // accumulator row
-        const int half = r >> 6, co = r & 63;
+        const int half = r / COP, co = r - half * COP;
         const bool any = u1 > u0;
         uint32_t done_ph = 0;
         if (any) {
             wait(&s_done, done_ph, 0);
             tc_fence_after();
         }
-        const bool valid = co < COP && (grp == 0 || half == 0);
+        const bool valid = half < nblk_a;
         float* P = grp == 0 ? A.part0 + (size_t)blockIdx.x * 18 * COP * CIP : A.part1 + (size_t)blockIdx.x * 9 * COP * CIP;
         auto load16 = [&](int col, uint32_t (&raw)[16]) {
             if (any) {
@@ -321,7 +312,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_dw_tc(const ConvDWTCArgs A)
         {  // the ones column: sum of g over this block's sites (the second group's rows 0-63)
             uint32_t raw[16];
             load16(3 * NT, raw);
-            if (grp == 1 && half == 0 && co < COP) A.bpart[(size_t)blockIdx.x * COP + co] = __uint_as_float(raw[0]);
+            if (grp == 1 && half == 0) A.bpart[(size_t)blockIdx.x * COP + co] = __uint_as_float(raw[0]);
         }
         tc_fence_before();
     }
@@ -357,30 +348,33 @@ __global__ void k_conv_dw_tc_reduce(const ConvDWTCArgs A, int CIP, int COP)
     }
 }
 
-size_t conv_dw_tc_smem(int CIP, int N, int nslot)
+size_t conv_dw_tc_smem(int CIP, int COP, int N, int nslot)
 {
-    return ((size_t)nslot * dw_a_entries(N) + (size_t)(nslot + kDwRowsExtra) * dw_row_entries(CIP, N) + kDwOnes) * 16;
+    // (the last slot's MMAs read up to 16 blocks from its start)
+    const size_t rest = (size_t)(nslot + kDwRowsExtra) * dw_row_entries(CIP, N) + kDwOnes;
+    const size_t past = (size_t)16 * (N + 1) - dw_a_entries(COP, N);
+    return ((size_t)nslot * dw_a_entries(COP, N) + (rest > past ? rest : past)) * 16;
 }
 
-int conv_dw_tc_slots(int CIP, int N)
+int conv_dw_tc_slots(int CIP, int COP, int N)
 {
-    if ((CIP != 16 && CIP != 32 && CIP != 48) || N < 16 || N % 16 != 0) return 0;
+    if ((CIP != 16 && CIP != 32 && CIP != 48) || (COP != 16 && COP != 32 && COP != 48) || N < 16 || N % 16 != 0) return 0;
     // larger lattices keep their weight gradients in FP32 on the CUDA cores
     if (N > (CIP == 16 ? 288 : CIP == 32 ? 224 : 192)) return 0;
     static_assert(2 * 288 <= kDwF32 * kDwStage, "FP32 entries a staging thread holds");
     for (int s = kDwMaxSlots; s >= 2; --s)
-        if (conv_dw_tc_smem(CIP, N, s) <= (size_t)kPassMaxSmem) return s;
+        if (conv_dw_tc_smem(CIP, COP, N, s) <= (size_t)kPassMaxSmem) return s;
     return 0;
 }
 
 template <int CIP, int COP, bool GF32, bool HF32>
 static cudaError_t launch_dw_tc_t(const ConvDWTCArgs& A, cudaStream_t s)
 {
-    const size_t smem = conv_dw_tc_smem(CIP, A.N, A.nslot);
+    const size_t smem = conv_dw_tc_smem(CIP, COP, A.N, A.nslot);
     cudaError_t e = cudaFuncSetAttribute(k_conv_dw_tc<CIP, COP, GF32, HF32>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_conv_dw_tc<CIP, COP, GF32, HF32><<<dim3(A.nb, 2), 256, smem, s>>>(A);
+    k_conv_dw_tc<CIP, COP, GF32, HF32><<<dim3(A.nb, 2), kDwThreads, smem, s>>>(A);
     return cudaGetLastError();
 }
 
@@ -393,7 +387,7 @@ static cudaError_t launch_dw_tc_t(const ConvDWTCArgs& A, cudaStream_t s)
 
 cudaError_t launch_conv_dw_tc(int CIP, int COP, const ConvDWTCArgs& A, cudaStream_t s)
 {
-    if (A.nslot < 2 || A.nslot > kDwMaxSlots || A.nslot > conv_dw_tc_slots(CIP, A.N) || A.nb < 1 || A.CI < 1 ||
+    if (A.nslot < 2 || A.nslot > kDwMaxSlots || A.nslot > conv_dw_tc_slots(CIP, COP, A.N) || A.nb < 1 || A.CI < 1 ||
         A.CI > CIP || A.CO < 1 || A.CO > COP || (A.h_f32 && A.h_c != A.CI) || (A.g_f32 && A.g_c != A.CO) ||
         (!A.h_f32 && A.CI != CIP) || (!A.g_f32 && A.CO != COP) || (A.g_f32 && A.h_f32))
         return cudaErrorInvalidValue;

@@ -144,41 +144,37 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                     }
                     tc_fence_after();
                     const uint32_t a_plane = smem_u32(sA + slot * PLANE);
-                    // MMAs of taps oz in [a, b] (contiguous accumulators) for one (ox, oy, kc)
-                    auto mma_run = [&](uint32_t a_addr, uint32_t b_tap, int a, int b, uint32_t accum) {
-                        const int sl = acc_slot(cbase + i - a);
-                        const uint32_t bdesc_addr = b_tap + a * NG * 128;
-                        const int n = (b - a + 1) * CO;
-                        tc_mma(tbase + sl * CO, smem_desc(a_addr, LBO_A, SBO_A), smem_desc(bdesc_addr, LBO_B3, SBO_B),
-                               idesc_bf16(128, n), accum);
-                    };
-                    auto mma_range = [&](uint32_t a_addr, uint32_t b_tap, int a, int b, uint32_t accum) {
-                        // split where the accumulator ring wraps
-                        const int sl = acc_slot(cbase + i - a);
-                        const int room = NA - sl;  // slots before the wrap
-                        if (b - a + 1 <= room) {
-                            mma_run(a_addr, b_tap, a, b, accum);
-                        } else {
-                            mma_run(a_addr, b_tap, a, a + room - 1, accum);
-                            mma_run(a_addr, b_tap, a + room, b, accum);
-                        }
-                    };
-#pragma unroll 1
-                    for (int t9 = 0; t9 < 9; ++t9) {
-                        const int ox = t9 % 3, oy = t9 / 3;
-                        const uint32_t a0 = a_plane + (oy * HX + ox) * 16;
-#pragma unroll
-                        for (int kc = 0; kc < KC; ++kc) {
-                            const uint32_t a_addr = a0 + kc * 2 * LBO_A;
-                            const uint32_t b_tap = smem_u32(sB) + ((t9 * KG + 2 * kc) * 3 * NG) * 128;
-                            if (t9 == 0 && kc == 0 && lo == 0) {
-                                mma_range(a_addr, b_tap, 0, 0, 0);  // first contribution to output i
-                                if (hi >= 1) mma_range(a_addr, b_tap, 1, hi, 1);
-                            } else {
-                                mma_range(a_addr, b_tap, lo, hi, 1);
-                            }
-                        }
+                    // the taps oz = lo .. hi in runs of contiguous accumulators: n1 of them, and the
+                    // others from the ring's start where it wraps
+                    const int sl = acc_slot(cbase + i - lo), n1 = min(hi - lo + 1, NA - sl), n2 = hi - lo + 1 - n1;
+                    const uint64_t ad = smem_desc(a_plane, LBO_A, SBO_A);
+                    const uint64_t bd1 = smem_desc(smem_u32(sB) + lo * NG * 128, LBO_B3, SBO_B);
+                    const uint64_t bd2 = bd1 + (uint64_t)(n1 * NG * 8);
+                    const uint32_t d1 = tbase + sl * CO, d2 = tbase;
+                    const uint32_t id1 = idesc_bf16(128, 0) + ((uint32_t)(n1 * NG) << 17);
+                    const uint32_t id2 = idesc_bf16(128, 0) + ((uint32_t)(n2 * NG) << 17);
+                    if (lo == 0) {  // the plane's first tap starts output i: oz = 0 overwrites alone
+                        constexpr uint32_t idx = idesc_bf16(128, CO);
+                        tc_mma(d1, ad, bd1, idx, 0);
+                        if (n1 > 1) tc_mma(d1 + CO, ad, bd1 + NG * 8, id1 - ((uint32_t)NG << 17), 1);
+                    } else {
+                        tc_mma(d1, ad, bd1, id1, 1);
                     }
+                    if (n2 > 0) tc_mma(d2, ad, bd2, id2, 1);
+                    // The other taps and K chunks of the plane.  One thread issues every MMA, so the
+                    // offsets are constants: working out slot, descriptors and shape for each MMA
+                    // took 160 cycles, where M = 128, N = 144 runs at 72 (hidden layer at 128^3:
+                    // 287 us, see launch_conv_tc)
+                    auto rest = [&](uint32_t d, uint64_t bd, uint32_t id) {
+#pragma unroll
+                        for (int q = 1; q < 9 * KC; ++q) {
+                            const int t9 = q / KC, kc = q - t9 * KC, ox = t9 % 3, oy = t9 / 3;
+                            tc_mma(d, ad + (uint64_t)(oy * HX + ox + kc * 2 * HY * HX),
+                                   bd + (uint64_t)((t9 * KG + 2 * kc) * 3 * NG * 8), id, 1);
+                        }
+                    };
+                    rest(d1, bd1, id1);
+                    if (n2 > 0) rest(d2, bd2, id2);
                     tc_commit(&s_freeb[slot]);  // the staged plane was read by this plane's MMAs only
                     if (i >= 2) tc_commit(&s_done[acc_slot(cbase + i - 2)]);  // output i-2 complete
                 }
@@ -225,7 +221,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                     dst[(kg * HY + hy) * HX + hx] = __ldg(reinterpret_cast<const uint4*>(in + site * CI + kg * 8));
                 }
             }
-            if (!A.in_f32 && A.in_act) {
+            if (A.in_act) {
                 if (tma) named_barrier_sync(1, NSTAGE);  // every patch is in place
                 for (int e = st; e < PLANE; e += NSTAGE) {
                     const int kg = e % KG, s2 = e / KG;
@@ -237,6 +233,8 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
             mbar_arrive(&s_full[slot]);
         };
         constexpr int EMAX = (PLANE + NSTAGE - 1) / NSTAGE;  // entries of a plane per staging thread
+        // thin FP32 input (at most three channels): this thread's entries, loaded a plane ahead
+        float fr[EMAX][3];
         for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
             int x0, y0, z0, nz;
             unit_geom(unit, x0, y0, z0, nz);
@@ -254,6 +252,18 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                 soff[q] = (kg * HY + hy) * HX + hx;
                 goff[q] = gy * N + gx;
             }
+            auto load_f32 = [&](int i) {
+                const int p = z0 - 1 + i;
+                const size_t zbase = (size_t)(p < 0 ? p + N : (p >= N ? p - N : p)) * N * N;
+#pragma unroll
+                for (int q = 0; q < EMAX; ++q) {
+                    const int e = st + q * NSTAGE;
+                    const float* in = reinterpret_cast<const float*>(A.in) + (zbase + goff[q]) * A.in_c;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) fr[q][c] = e < PLANE && e % KG == 0 && c < A.in_c ? __ldg(in + c) : 0.f;
+                }
+            };
+            if (A.in_f32) load_f32(0);
             for (int i = 0; i < nz + 2; ++i, ++seq) {
                 const int slot = (int)(seq % NSLOT);
                 if (seq >= NSLOT) wait(&s_freeb[slot], free_ph, slot);
@@ -261,6 +271,18 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                 const int pz = ((p % N) + N) % N;
                 const size_t zbase = (size_t)pz * N * N;
                 uint4* dst = sA + slot * PLANE;
+                if (A.in_f32) {  // converted and zero-padded to CI channels
+#pragma unroll
+                    for (int q = 0; q < EMAX; ++q) {
+                        if (st + q * NSTAGE >= PLANE) break;
+                        const float f[8] = {fr[q][0], fr[q][1], fr[q][2], 0.f, 0.f, 0.f, 0.f, 0.f};
+                        dst[soff[q]] = pack_bf16x8(f);
+                    }
+                    fence_proxy_async_smem();
+                    mbar_arrive(&s_full[slot]);
+                    if (i + 1 < nz + 2) load_f32(i + 1);
+                    continue;
+                }
                 if (tma) {
                     if (st == 0) {  // one tensor copy: the plane with its halo (zeros outside the box)
                         mbar_arrive_expect_tx(&s_tma[slot], (uint32_t)(PLANE * 16));
@@ -278,17 +300,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                         if (e >= PLANE) break;
                         const int kg = e % KG;
                         const size_t site = zbase + goff[q];
-                        if (!A.in_f32) {
-                            cp_async16(dst + soff[q], reinterpret_cast<const __nv_bfloat16*>(A.in) + site * CI + kg * 8);
-                        } else {  // thin FP32 input: convert and zero-pad to CI channels
-                            float f[8];
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) {
-                                const int ch = kg * 8 + c;
-                                f[c] = ch < A.in_c ? __ldg(reinterpret_cast<const float*>(A.in) + site * A.in_c + ch) : 0.f;
-                            }
-                            dst[soff[q]] = pack_bf16x8(f);
-                        }
+                        cp_async16(dst + soff[q], reinterpret_cast<const __nv_bfloat16*>(A.in) + site * CI + kg * 8);
                     }
                     cp_async_commit();
                 }
@@ -316,6 +328,13 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
             unit_geom(unit, x0, y0, z0, nz);
             for (int k = 0; k < nz; ++k, ++c) {
                 const int buf = (int)(S::NACC - 1 - (int)(c % S::NACC));  // accumulator slot of output c
+                const size_t site = ((size_t)(z0 + k) * N + (y0 + (r >> 3))) * N + (x0 + (r & 7));
+                uint4 graw[CO / 8];  // the gate's values come in while the MMAs finish
+                if (A.gate_act) {
+#pragma unroll
+                    for (int c8 = 0; c8 < CO / 8; ++c8)
+                        graw[c8] = __ldg(reinterpret_cast<const uint4*>(A.gate + site * CO + c8 * 8));
+                }
                 wait(&s_done[buf], done_ph, buf);
                 tc_fence_after();
                 uint32_t raw[CO];
@@ -330,12 +349,11 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                 float v[CO];
 #pragma unroll
                 for (int e = 0; e < CO; ++e) v[e] = __uint_as_float(raw[e]) + s_bias[e];
-                const size_t site = ((size_t)(z0 + k) * N + (y0 + (r >> 3))) * N + (x0 + (r & 7));
                 if (A.gate_act) {
 #pragma unroll
                     for (int c8 = 0; c8 < CO / 8; ++c8) {
                         float gf[8];
-                        unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(A.gate + site * CO + c8 * 8)), gf);
+                        unpack_bf16x8(graw[c8], gf);
 #pragma unroll
                         for (int e = 0; e < 8; ++e) v[c8 * 8 + e] *= act_grad_f(A.gate_act, gf[e]);
                     }

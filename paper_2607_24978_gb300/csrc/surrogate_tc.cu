@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
     __shared__ float s_bias[CO];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int N = A.N;
     const int ntx = N / kSgTileX, nty = N / kSgTileY, nzc = (N + A.DZ - 1) / A.DZ;
     const int units = ntx * nty * nzc;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
         // acc_slot(c) = (NACC - 1 - c) mod NACC: consecutive oz map to consecutive slots,
         // except where the ring wraps (the MMA is split there).  An output's first
         // contribution (i = k, oz = 0) overwrites, all others accumulate.
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr int NA = S::NACC;
             uint32_t full_ph = 0, accfree_ph = 0;
             uint32_t seq = 0, cbase = 0;  // staged planes and outputs of earlier units
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256, 1) k_conv_tc(const __grid_constant__ Conv
                     // The other taps and K chunks of the plane.  One thread issues every MMA, so the
                     // offsets are constants: working out slot, descriptors and shape for each MMA
                     // took 160 cycles, where M = 128, N = 144 runs at 72 (hidden layer at 128^3:
-                    // 287 us, see launch_conv_tc)
+                    // 287 -> 209 us)
                     auto rest = [&](uint32_t d, uint64_t bd, uint32_t id) {
 #pragma unroll
                         for (int q = 1; q < 9 * KC; ++q) {

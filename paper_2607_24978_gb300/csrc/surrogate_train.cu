@@ -42,20 +42,22 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const LossArgs A)
     if (threadIdx.x == 0) A.partial[blockIdx.x] = v[0];
 }
 
-__global__ void k_sum_partials(const double* p, int n, double* out)
+// Sum of the blocks' partials by one block, in a fixed order (one thread adding them in turn waits
+// 70 cycles for each FP64 addition: 50 us for 1216 of them, on the training step of 128^3).
+__global__ void __launch_bounds__(kRedThreads) k_sum_partials(const double* p, int n, double* out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += p[i];  // fixed order
-        *out = s;
-    }
+    __shared__ double s_red[32][kMaxQ];
+    double v[1] = {0.0};
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v[0] += p[i];
+    block_reduce<1>(v, s_red, threadIdx.x, blockDim.x);
+    if (threadIdx.x == 0) *out = v[0];
 }
 
 cudaError_t launch_loss(const LossArgs& A, double* result, cudaStream_t s)
 {
     const int g = red_grid(A.n * A.C);
     k_loss<<<g, kRedThreads, 0, s>>>(A);
-    k_sum_partials<<<1, 32, 0, s>>>(A.partial, g, result);
+    k_sum_partials<<<1, kRedThreads, 0, s>>>(A.partial, g, result);
     return cudaGetLastError();
 }
 

@@ -119,7 +119,7 @@ struct cl_lattice {
     std::vector<EnsItem> hitems;
     EnsMember* d_members = nullptr;
     EnsItem* d_items = nullptr;
-    int* d_sched = nullptr;         // items by decreasing size
+    int* d_first = nullptr;         // first item of each block of a whole pass (library's cuts)
     int nitems = 0, ens_grid = 0, ens_stages = 0, ens_stage_stride = 0, ens_ring_slot = 0, ens_variant = 0;
     float* sg_buf = nullptr;        // surrogate jumps: packed input (3 V), output (2 V), snapshot (3 V)
     size_t ens_smem = 0;
@@ -200,13 +200,57 @@ cl_status upload_members(cl_lattice* l)
     return CL_OK;
 }
 
-// Ensemble work items.  Per member: BY full rows (as many as one block's threads cover)
-// by all N planes (or CL_OPT_TILE_DZ planes), both balanced within the member; long items
-// amortise the per-item pipeline start and epilogue (measured: 16-plane items ran at 37%
-// of HBM bandwidth, whole columns at 67% on 32..64^3 members).  The items of a member are
-// consecutive in the table (their partials are reduced in that order); blocks take items
-// in order of decreasing size (largest first balances the persistent grid's tail).  The
-// persistent grid is one wave of resident blocks.
+// One column of an ensemble: BY full rows of a member, the planes from z0.
+struct EnsColumn {
+    int member, y0, z0, planes;
+    int64_t row;  // work of one plane of it
+};
+
+// Work of an item, in units of one site's bandwidth share: a plane of it takes the time of its sites
+// or, where the block waits rather than copies, about that of kEnsPlane sites (1550 cycles); the two
+// halo planes and the start and the end of an item (prefactors, partial sums, the member's epilogue:
+// 15000 to 25000 cycles) that of kEnsExtra planes.  Measured (us a pass; one field, FP32 with
+// compensated sums; members of 32, 48, 64 sites in turn / 16, 32 / 27, 33, 50 / 24, 40, 56): whole
+// columns dealt out by decreasing size 184 (256 members), 33 (8), 146 (100), 50 (40); cut by sites
+// alone with kEnsExtra = 8 177, 40, 119, 35; so 162, 22, 101, 32.
+constexpr int kEnsPlane = 1024, kEnsExtra = 18;
+constexpr int kEnsMinPlanes = 8;  // (16: 165, 23, 113, 35)
+
+// Cut the columns, one after the other, into blocks of at most `target` work each; an item keeps at
+// least min_planes planes (columns no longer than that stay whole).  Returns the number of blocks
+// (0: no block can hold the shortest item); with `items`, also the items and each block's first one.
+int ens_cut(const std::vector<EnsColumn>& cols, double target, int min_planes, std::vector<EnsItem>* items,
+            std::vector<int>* first)
+{
+    int blocks = 1, n = 0;
+    double load = 0.0;
+    if (first) first->assign(1, 0);
+    for (const EnsColumn& c : cols)
+        for (int z = 0; z < c.planes;) {
+            const int left = c.planes - z;
+            const double room = (target - load) / (double)c.row - kEnsExtra;
+            int p = room >= left ? left : (int)room;
+            if (p < left && left - p < min_planes) p = left - min_planes;
+            if (p < (left < min_planes ? left : min_planes)) {
+                if (load == 0.0) return 0;
+                ++blocks;
+                load = 0.0;
+                if (first) first->push_back(n);
+                continue;
+            }
+            if (items) items->push_back({c.member, c.y0, c.z0 + z, p});
+            ++n;
+            load += ((double)p + kEnsExtra) * (double)c.row;
+            z += p;
+        }
+    if (first) first->push_back(n);
+    return blocks;
+}
+
+// Ensemble work items.  Per member: columns of BY full rows (as many as one block's threads
+// cover, balanced within the member).  The columns of all members, one after the other, are cut
+// into one wave of resident blocks of equal work, each a run of consecutive items (whole columns
+// and at most two parts), by the smallest target that a wave holds.
 cl_status ens_tiles(cl_lattice* l)
 {
     const int B = l->members, prec = l->p.precision;
@@ -215,6 +259,7 @@ cl_status ens_tiles(cl_lattice* l)
     size_t smem = 0;
     int64_t stage_max = 0, ring_max = 0;
     const int narr = l->nf * (has_kahan(l) ? 3 : 2);
+    std::vector<EnsColumn> cols;
     for (int m = 0; m < B; ++m) {
         const int N = l->mN[m], TX = N / l->VW;
         int BY = kEnsThreads / TX;
@@ -233,12 +278,14 @@ cl_status ens_tiles(cl_lattice* l)
         M.N = N;
         M.BY = BY;
         M.DZ = DZ;
-        M.item0 = (int)l->hitems.size();
-        M.nitems = nby * nbz;
         M.dx = l->mL[m] / N;
         if ((nby - 1) * BY >= N || (nbz - 1) * DZ >= N) return fail(l, CL_EINVAL, "ensemble tiling error");
+        M.item0 = M.nitems = 0;
         for (int bz = 0; bz < nbz; ++bz)
-            for (int by = 0; by < nby; ++by) l->hitems.push_back({m, by * BY, bz * DZ, 0});
+            for (int by = 0; by < nby; ++by) {
+                const int R = BY < N - by * BY ? BY : N - by * BY, nz = DZ < N - bz * DZ ? DZ : N - bz * DZ;
+                cols.push_back({m, by * BY, bz * DZ, nz, (int64_t)R * N + kEnsPlane});
+            }
         const size_t sm = (size_t)l->nf * 3 * (BY + 2) * N * l->es;
         if (sm > smem) smem = sm;
         if ((int64_t)narr * (BY + 2) * N > stage_max) stage_max = (int64_t)narr * (BY + 2) * N;
@@ -268,42 +315,46 @@ cl_status ens_tiles(cl_lattice* l)
     l->ens_variant = var;
     l->ens_stage_stride = (int)stage_max;
     l->ens_ring_slot = (int)ring_max;
-    l->nitems = (int)l->hitems.size();
     l->ens_smem = smem;
-    if (l->d_items) cudaFree(l->d_items);
-    l->d_items = nullptr;
-    if (l->d_sched) cudaFree(l->d_sched);
-    l->d_sched = nullptr;
-    if (!l->d_members && cudaMalloc(&l->d_members, sizeof(EnsMember) * B) != cudaSuccess)
-        return fail(l, CL_ENOMEM, "cannot allocate the member table");
-    if (cudaMalloc(&l->d_items, sizeof(EnsItem) * l->hitems.size()) != cudaSuccess)
-        return fail(l, CL_ENOMEM, "cannot allocate the item table");
-    CUDA_TRY(l, cudaMemcpy(l->d_items, l->hitems.data(), sizeof(EnsItem) * l->hitems.size(), cudaMemcpyHostToDevice));
-    {
-        std::vector<int> order(l->hitems.size());
-        std::vector<int64_t> size(l->hitems.size());
-        for (size_t i = 0; i < order.size(); ++i) {
-            const EnsItem& I = l->hitems[i];
-            const EnsMember& M = l->hmem[I.member];
-            const int R = M.BY < M.N - I.y0 ? M.BY : M.N - I.y0, NZ = M.DZ < M.N - I.z0 ? M.DZ : M.N - I.z0;
-            order[i] = (int)i;
-            size[i] = (int64_t)R * NZ * M.N;
-        }
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return size[a] > size[b]; });
-        if (cudaMalloc(&l->d_sched, sizeof(int) * order.size()) != cudaSuccess)
-            return fail(l, CL_ENOMEM, "cannot allocate the item schedule");
-        CUDA_TRY(l, cudaMemcpy(l->d_sched, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice));
-    }
-    cl_status s = upload_members(l);
-    if (s != CL_OK) return s;
     int dev = 0, nsm = 0, per_sm = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
         return fail(l, CL_ECUDA, "cannot query the SM count");
     CUDA_TRY(l, ensemble_pass_blocks_per_sm(prec, l->nf, l->VW, stages, var, smem, &per_sm));
     if (per_sm < 1) return fail(l, CL_EINVAL, "ensemble pass does not fit on an SM");
-    const int64_t wave = (int64_t)per_sm * nsm;
-    l->ens_grid = (int)(wave < l->nitems ? wave : l->nitems);
+    const int wave = per_sm * nsm;
+    std::vector<int> first;
+    const int min_planes = l->opt_DZ > 0 ? kEnsMaxN : kEnsMinPlanes;  // CL_OPT_TILE_DZ's chunks stay as they are
+    double lo = 0.0, hi = 0.0;  // hi: one block takes everything
+    for (const EnsColumn& c : cols) hi += ((double)c.planes + kEnsExtra + 1.0) * (double)c.row;
+    for (int i = 0; i < 60 && hi - lo > 1.0; ++i) {
+        const double mid = 0.5 * (lo + hi);
+        const int n = ens_cut(cols, mid, min_planes, nullptr, nullptr);
+        if (n > 0 && n <= wave) hi = mid;
+        else lo = mid;
+    }
+    ens_cut(cols, hi, min_planes, &l->hitems, &first);
+    l->ens_grid = (int)first.size() - 1;
+    l->nitems = (int)l->hitems.size();
+    for (int i = l->nitems - 1; i >= 0; --i) {  // a member's items are consecutive
+        EnsMember& M = l->hmem[l->hitems[i].member];
+        M.item0 = i;
+        ++M.nitems;
+    }
+    if (l->d_items) cudaFree(l->d_items);
+    l->d_items = nullptr;
+    if (l->d_first) cudaFree(l->d_first);
+    l->d_first = nullptr;
+    if (!l->d_members && cudaMalloc(&l->d_members, sizeof(EnsMember) * B) != cudaSuccess)
+        return fail(l, CL_ENOMEM, "cannot allocate the member table");
+    if (cudaMalloc(&l->d_items, sizeof(EnsItem) * l->hitems.size()) != cudaSuccess)
+        return fail(l, CL_ENOMEM, "cannot allocate the item table");
+    CUDA_TRY(l, cudaMemcpy(l->d_items, l->hitems.data(), sizeof(EnsItem) * l->hitems.size(), cudaMemcpyHostToDevice));
+    if (cudaMalloc(&l->d_first, sizeof(int) * first.size()) != cudaSuccess)
+        return fail(l, CL_ENOMEM, "cannot allocate the item schedule");
+    CUDA_TRY(l, cudaMemcpy(l->d_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
+    cl_status s = upload_members(l);
+    if (s != CL_OK) return s;
     s = grow_partials(l, l->nitems);
     if (s != CL_OK) return s;
     invalidate_graphs(l);
@@ -819,7 +870,7 @@ cl_status run_ens_pass_t(cl_lattice* l, const PassCoef& pc, int in, int out, int
     }
     A.members = l->d_members;
     A.items = l->d_items;
-    A.sched = (m0 == 0 && m1 == l->members) ? l->d_sched : nullptr;  // whole passes: largest items first
+    A.first = (m0 == 0 && m1 == l->members) ? l->d_first : nullptr;  // whole passes: the blocks' runs
     A.scal = l->scal;
     A.partials = l->partials;
     A.item_begin = l->hmem[m0].item0;
@@ -833,7 +884,7 @@ cl_status run_ens_pass_t(cl_lattice* l, const PassCoef& pc, int in, int out, int
     A.ring_slot = l->ens_ring_slot;
     A.variant = l->ens_variant;
     const int n = A.item_end - A.item_begin;
-    const int grid = n < l->ens_grid ? n : l->ens_grid;
+    const int grid = n < l->ens_grid && !A.first ? n : l->ens_grid;
     cudaError_t e = launch_ensemble_pass(l->p.precision, l->nf, &A, l->VW, grid, l->ens_smem, l->stream);
     if (e != cudaSuccess) return fail(l, CL_ECUDA, "ensemble pass launch failed: %s", cudaGetErrorString(e));
     return CL_OK;
@@ -1477,7 +1528,7 @@ void cl_free(cl_lattice* l)
     for (const auto& pp : l->sp_plans) cufftDestroy(pp.second);
     if (l->d_members) cudaFree(l->d_members);
     if (l->d_items) cudaFree(l->d_items);
-    if (l->d_sched) cudaFree(l->d_sched);
+    if (l->d_first) cudaFree(l->d_first);
     if (l->own_stream && l->stream) cudaStreamDestroy(l->stream);
     delete l;
 }

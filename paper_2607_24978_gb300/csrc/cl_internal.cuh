@@ -295,7 +295,7 @@ struct EnsMember {
     double m2[2], lam[2], g2;
 };
 struct EnsItem {
-    int member, y0, z0, pad;
+    int member, y0, z0, nz;  // rows from y0 (the member's BY, or what is left), nz planes from z0
 };
 template <typename T>
 struct EnsPassArgs {
@@ -307,7 +307,8 @@ struct EnsPassArgs {
     T* c_out[2];
     const EnsMember* members;
     const EnsItem* items;
-    const int* sched;     // processing order of all items (nullptr: items item_begin.. in order)
+    const int* first;     // block b takes items first[b] .. first[b + 1] - 1 (nullptr: the items
+                          // item_begin + b, + grid, ... below item_end)
     DevScal* scal;        // one per member
     double* partials;     // [items][kMaxQ]
     int item_begin, item_end;

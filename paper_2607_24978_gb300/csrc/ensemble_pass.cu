@@ -2,9 +2,10 @@
 //
 // Many small lattices (each with its own size, box, couplings, a and a') advance by one
 // pass of the staggered kick-drift scheme in a single persistent launch.  The work is a
-// table of items, each BY full x rows times DZ planes of one member; block b takes the
-// items b, b + grid, b + 2 grid, ... of a schedule (largest first) and runs the same per-site arithmetic as the
-// single-lattice direct loader on it (drift while loading, stencil kick, energies).
+// table of items, each BY full x rows times some planes of one member; block b takes a run of
+// consecutive items (the library cuts the members' columns of planes so that every block has the
+// same work) and runs the same per-site arithmetic as the single-lattice direct loader on it
+// (drift while loading, stencil kick, energies).
 // Reductions: every item writes its FP64 partial sums; the block that completes the last
 // item of a member (an arrival counter per member) sums that member's partials in a fixed
 // order and runs the member's scale-factor epilogue.  Reading a, a' happens at item
@@ -18,6 +19,17 @@
 
 namespace clk {
 
+// Items of this block: it, it + step, ... below end.
+struct EnsRange {
+    int it, end, step;
+    template <typename A_>
+    __device__ __forceinline__ explicit EnsRange(const A_& A)
+        : it(A.first ? A.first[blockIdx.x] : A.item_begin + (int)blockIdx.x),
+          end(A.first ? A.first[blockIdx.x + 1] : A.item_end), step(A.first ? 1 : (int)gridDim.x)
+    {
+    }
+};
+
 template <typename T, int NF, bool KAHAN, int VW>
 __global__ void __launch_bounds__(kEnsThreads) k_ensemble_pass(const EnsPassArgs<T> A)
 {
@@ -30,8 +42,8 @@ __global__ void __launch_bounds__(kEnsThreads) k_ensemble_pass(const EnsPassArgs
     const bool do_drift = (A.flags & P_DRIFT) != 0;
     const bool expand = (A.flags & P_EXPANSION) != 0;
 
-    for (int k = blockIdx.x; k < A.item_end - A.item_begin; k += gridDim.x) {
-        const int it = A.sched ? A.sched[k] : A.item_begin + k;
+    const EnsRange W(A);
+    for (int it = W.it; it < W.end; it += W.step) {
         const EnsItem I = A.items[it];
         const EnsMember& M = A.members[I.member];
         const int N = M.N, BY = M.BY;
@@ -53,7 +65,7 @@ __global__ void __launch_bounds__(kEnsThreads) k_ensemble_pass(const EnsPassArgs
             F.c_out[f] = KAHAN ? A.c_out[f] + off : nullptr;
         }
         Acc<T> accK[NF], accG[NF], accV;
-        const int R = min(BY, N - I.y0), NZ = min(M.DZ, N - I.z0);
+        const int R = min(BY, N - I.y0), NZ = I.nz;
         march_tile<T, NF, KAHAN, VW>(F, N, BY, I.y0, R, I.z0, NZ, sm, tid, nthr, do_drift, C, P, accK, accG, accV);
 
         double v[kMaxQ];
@@ -129,12 +141,12 @@ __global__ void __launch_bounds__(kEnsTmaThreads, NF == 1 ? 2 : 1) k_ensemble_pa
         int st = 0;
         uint32_t empty_phase = 0;
         int issued = 0;
-        for (int k = blockIdx.x; k < A.item_end - A.item_begin; k += gridDim.x) {
-            const int it = A.sched ? A.sched[k] : A.item_begin + k;
+        const EnsRange W(A);
+        for (int it = W.it; it < W.end; it += W.step) {
             const EnsItem I = A.items[it];
             const EnsMember& M = A.members[I.member];
             const int N = M.N, BY = M.BY, y0 = I.y0, z0 = I.z0;
-            const int R = min(BY, N - y0), NZ = min(M.DZ, N - z0);
+            const int R = min(BY, N - y0), NZ = I.nz;
             const int ylo = y0 == 0 ? N - 1 : y0 - 1;
             const int yhi = y0 + R == N ? 0 : y0 + R;
             const int arr_stride = (BY + 2) * N;
@@ -175,12 +187,12 @@ __global__ void __launch_bounds__(kEnsTmaThreads, NF == 1 ? 2 : 1) k_ensemble_pa
             if (lane == 0) mbar_arrive(&s_empty[s_idx]);
         };
         ZMarch<T, NF, VW> Z;
-        for (int k = blockIdx.x; k < A.item_end - A.item_begin; k += gridDim.x) {
-            const int it = A.sched ? A.sched[k] : A.item_begin + k;
+        const EnsRange W(A);
+        for (int it = W.it; it < W.end; it += W.step) {
             const EnsItem I = A.items[it];
             const EnsMember& M = A.members[I.member];
             const int N = M.N, BY = M.BY, y0 = I.y0, z0 = I.z0;
-            const int R = min(BY, N - y0), NZ = min(M.DZ, N - z0);
+            const int R = min(BY, N - y0), NZ = I.nz;
             const double dx = M.dx;
             DevScal* Sm = A.scal + I.member;
             pass_coefficients_warps(tid, Sm->a, Sm->b, A.d, A.alpha, dx, expand, s_coef);

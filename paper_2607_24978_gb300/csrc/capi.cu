@@ -119,6 +119,7 @@ struct cl_lattice {
     std::vector<EnsItem> hitems;
     EnsMember* d_members = nullptr;
     EnsItem* d_items = nullptr;
+    int* h_status = nullptr;        // page-locked: the members' status words, joined (check_status)
     int* d_first = nullptr;         // first item of each block of a whole pass (library's cuts)
     int nitems = 0, ens_grid = 0, ens_stages = 0, ens_stage_stride = 0, ens_ring_slot = 0, ens_variant = 0;
     float* sg_buf = nullptr;        // surrogate jumps: packed input (3 V), output (2 V), snapshot (3 V)
@@ -1353,6 +1354,20 @@ cl_status read_status(cl_lattice* l, std::vector<DevScal>& host)
     return CL_OK;
 }
 
+// Wait for the stream; report and clear the device status (as read_status, which this calls if there
+// is one to report).  A launch joins the members' status words in one word of host memory: copying
+// the scalar state of 256 members (70 KB of pageable memory) to look at them took 23 us a call, this
+// kernel and the wait take 12.
+cl_status check_status(cl_lattice* l)
+{
+    std::vector<DevScal> h;
+    if (!l->h_status) return read_status(l, h);
+    const cudaError_t e = launch_status_any(l->scal, l->members, l->h_status, l->stream);
+    if (e != cudaSuccess) return fail(l, CL_ECUDA, "status launch failed: %s", cudaGetErrorString(e));
+    CUDA_TRY(l, cudaStreamSynchronize(l->stream));
+    return *l->h_status ? read_status(l, h) : CL_OK;
+}
+
 // 0 = scalar field f, 1 = its momentum, 2 = link angle theta_f, 3 = electric field E_f.
 int field_kind(const cl_lattice* l, int field, int* f)
 {
@@ -1521,6 +1536,7 @@ void cl_free(cl_lattice* l)
     for (int q = 0; q < 9; ++q)
         if (l->u1s[q]) cudaFree(l->u1s[q]);
     if (l->scal) cudaFree(l->scal);
+    if (l->h_status) cudaFreeHost(l->h_status);
     if (l->partials) cudaFree(l->partials);
     if (l->ps_barrier) cudaFree(l->ps_barrier);
     if (l->sg_buf) cudaFree(l->sg_buf);
@@ -1654,6 +1670,11 @@ cl_status cl_init_lattice(cl_lattice** out, const cl_lattice_params* p)
             return CL_ENOMEM;
         }
     }
+    // (without it the status words are read with the rest of the scalar state)
+    if (ens && cudaHostAlloc(&l->h_status, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        l->h_status = nullptr;
+    }
     if (cudaMalloc(&l->scal, sizeof(DevScal) * l->members) != cudaSuccess) {
         cl_free(l);
         return CL_ENOMEM;
@@ -1766,8 +1787,7 @@ cl_status cl_get_state(cl_lattice* l, int32_t member, int32_t field, void* dst, 
     const void* srcp = (const char*)fb + mem_off_bytes(l, member);
     CUDA_TRY(l, cudaMemcpyAsync(dst, srcp, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                                 l->stream));
-    std::vector<DevScal> h;
-    return read_status(l, h);
+    return check_status(l);
 }
 
 cl_status cl_set_scalars(cl_lattice* l, int32_t member, double a, double adot, double t)
@@ -2263,8 +2283,7 @@ cl_status cl_step(cl_lattice* l, int32_t nsteps)
 cl_status cl_sync(cl_lattice* l)
 {
     if (!l) return CL_EINVAL;
-    std::vector<DevScal> h;
-    return read_status(l, h);
+    return check_status(l);
 }
 
 cl_status cl_energies(cl_lattice* l, cl_energy* out, int32_t count)

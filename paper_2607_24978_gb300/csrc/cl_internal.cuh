@@ -325,6 +325,8 @@ constexpr int kEnsTmaThreads = kEnsThreads + 32;  // consumers + one producer wa
 // One pass over the items [item_begin, item_end) with `grid` persistent blocks.
 cudaError_t launch_ensemble_pass(int precision, int nf, const void* args, int vw, int grid, size_t smem,
                                  cudaStream_t s);
+// The members' status words together, into host memory that the device can write.
+cudaError_t launch_status_any(const DevScal* scal, int members, int* out, cudaStream_t s);
 cudaError_t ensemble_pass_blocks_per_sm(int precision, int nf, int vw, int stages, int variant, size_t smem,
                                         int* blocks);
 

@@ -351,4 +351,22 @@ cudaError_t ensemble_pass_blocks_per_sm(int precision, int nf, int vw, int stage
     return ens_dispatch(precision, nf, nullptr, vw, stages, variant, 0, smem, nullptr, blocks);
 }
 
+// One block: the OR of every member's status word.
+__global__ void __launch_bounds__(1024) k_status_any(const DevScal* scal, int members, int* out)
+{
+    __shared__ int s_any;
+    if (threadIdx.x == 0) s_any = 0;
+    __syncthreads();
+    for (int m = threadIdx.x; m < members; m += blockDim.x)
+        if (scal[m].status) atomicOr(&s_any, scal[m].status);
+    __syncthreads();
+    if (threadIdx.x == 0) *out = s_any;
+}
+
+cudaError_t launch_status_any(const DevScal* scal, int members, int* out, cudaStream_t s)
+{
+    k_status_any<<<1, members < 1024 ? (members + 31) / 32 * 32 : 1024, 0, s>>>(scal, members, out);
+    return cudaGetLastError();
+}
+
 }  // namespace clk

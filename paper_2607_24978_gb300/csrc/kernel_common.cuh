@@ -201,29 +201,6 @@ template <> struct Acc<double> {
     __device__ __forceinline__ double value() const { return s; }
 };
 
-// Sum v[q] over the block; the result is valid in thread 0.  Fixed reduction order.
-template <int Q>
-__device__ __forceinline__ void block_reduce(double (&v)[Q], double (*s_red)[kMaxQ], int tid, int nthr)
-{
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-        for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-    const int warp = tid >> 5, lane = tid & 31, nw = (nthr + 31) >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < Q; ++q) s_red[warp][q] = v[q];
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            double x = lane < nw ? s_red[lane][q] : 0.0;
-            for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-            v[q] = x;
-        }
-    }
-    __syncthreads();
-}
-
 // Float-pair (hi + lo) addition with the two-sum error term, for the warp-level stage of the
 // FP32 passes' energy sums: about 44 significant bits on the FP32 pipe.  GB300 executes FP64
 // additions two lanes per SM and cycle, so a warp butterfly of doubles on every lane is slow
@@ -241,49 +218,140 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b)
     return {h, __fsub_rn(e, __fsub_rn(h, s))};
 }
 
+// Sums of Q values over the lanes of a warp.  A butterfly of every value on every lane is Q x 5
+// additions, and an FP64 instruction occupies its scheduler for 64 cycles whatever lanes it has: 25
+// of them in a row for the five sums of a pass.  Here each step sends half of the values to one half
+// of the lanes and half to the other, so the five sums take 3 + 2 + 1 + 1 + 1 additions, of the same
+// pairs as the butterfly and hence the same values.  Value q's sum arrives in lane
+// warp_sum_lane<Q>(q) (and others).
+__device__ __forceinline__ double plus(double a, double b) { return a + b; }
+__device__ __forceinline__ F2 plus(F2 a, F2 b) { return f2_add(a, b); }
+__device__ __forceinline__ double from_lane_xor(double x, int off) { return __shfl_xor_sync(0xffffffffu, x, off); }
+__device__ __forceinline__ F2 from_lane_xor(F2 x, int off)
+{
+    return {__shfl_xor_sync(0xffffffffu, x.hi, off), __shfl_xor_sync(0xffffffffu, x.lo, off)};
+}
+__device__ __forceinline__ void set_zero(double& x) { x = 0.0; }
+__device__ __forceinline__ void set_zero(F2& x) { x = {0.f, 0.f}; }
+
+template <int Q, int OFF = 16, typename V>
+__device__ __forceinline__ V warp_sums(const V (&v)[Q], int lane)
+{
+    if constexpr (Q == 1) {
+        V x = v[0];
+#pragma unroll
+        for (int off = OFF; off > 0; off >>= 1) x = plus(x, from_lane_xor(x, off));
+        return x;
+    } else {
+        constexpr int H = (Q + 1) / 2;
+        const bool up = (lane & OFF) != 0;
+        V w[H];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            V a;
+            set_zero(a);
+            if (i + H < Q) a = v[i + H];
+            const V keep = up ? a : v[i], send = up ? v[i] : a;
+            w[i] = plus(keep, from_lane_xor(send, OFF));
+        }
+        return warp_sums<H, OFF / 2>(w, lane);
+    }
+}
+template <int Q>
+__host__ __device__ constexpr int warp_sum_lane(int q)
+{
+    int lane = 0, n = Q;
+    for (int off = 16; n > 1; off >>= 1) {
+        const int h = (n + 1) / 2;
+        if (q >= h) {
+            lane |= off;
+            q -= h;
+        }
+        n = h;
+    }
+    return lane;
+}
+// warp_sums' results to every lane
+template <int Q>
+__device__ __forceinline__ void warp_sums_all(double (&v)[Q], int lane)
+{
+    const double x = warp_sums<Q>(v, lane);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = __shfl_sync(0xffffffffu, x, warp_sum_lane<Q>(q));
+}
+
+__device__ __forceinline__ double as_double(double x) { return x; }
+__device__ __forceinline__ double as_double(F2 x) { return (double)x.hi + (double)x.lo; }
+
+// The two stages of a block's sums, before and after its barrier: each warp's sums into its row of
+// s_red, in FP64 (float pairs convert once); the nw rows' sums, by warp 0.
+template <int Q, typename V>
+__device__ __forceinline__ void warp_sums_to(const V (&v)[Q], double (*s_red)[kMaxQ], int warp, int lane)
+{
+    const double x = as_double(warp_sums<Q>(v, lane));
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        if (lane == warp_sum_lane<Q>(q)) s_red[warp][q] = x;
+}
+template <int Q>
+__device__ __forceinline__ void sum_rows(double (&v)[Q], double (*s_red)[kMaxQ], int nw, int lane)
+{
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = lane < nw ? s_red[lane][q] : 0.0;
+    warp_sums_all<Q>(v, lane);
+}
+
+// Sum v[q] over the block; the result is valid in thread 0.  Fixed reduction order.
+template <int Q>
+__device__ __forceinline__ void block_reduce(double (&v)[Q], double (*s_red)[kMaxQ], int tid, int nthr)
+{
+    const int warp = tid >> 5, lane = tid & 31, nw = (nthr + 31) >> 5;
+    warp_sums_to<Q>(v, s_red, warp, lane);
+    __syncthreads();
+    if (warp == 0) sum_rows<Q>(v, s_red, nw, lane);
+    __syncthreads();
+}
+
 // Sum over the block of per-thread values hi[q] + lo[q] (e.g. a compensated FP32 sum s - c),
-// the result in FP64, valid in thread 0.  Each warp adds its lanes as float pairs, lane 0
-// converts once to FP64, warp 0 adds the warps in FP64.  Fixed reduction order.
+// the result in FP64, valid in thread 0.  Each warp adds its lanes as float pairs and converts its
+// sums once to FP64, warp 0 adds the warps in FP64.  Fixed reduction order.
 template <int Q>
 __device__ __forceinline__ void block_reduce_pairs(const float (&hi)[Q], const float (&lo)[Q], double (&v)[Q],
                                                    double (*s_red)[kMaxQ], int tid, int nthr)
 {
     const int warp = tid >> 5, lane = tid & 31, nw = (nthr + 31) >> 5;
+    F2 x[Q];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        F2 x{hi[q], lo[q]};
-        for (int off = 16; off > 0; off >>= 1) {
-            const F2 o{__shfl_xor_sync(0xffffffffu, x.hi, off), __shfl_xor_sync(0xffffffffu, x.lo, off)};
-            x = f2_add(x, o);
-        }
-        if (lane == 0) s_red[warp][q] = (double)x.hi + (double)x.lo;
-    }
+    for (int q = 0; q < Q; ++q) x[q] = {hi[q], lo[q]};
+    warp_sums_to<Q>(x, s_red, warp, lane);
     __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            double x = lane < nw ? s_red[lane][q] : 0.0;
-            for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-            v[q] = x;
-        }
-    }
+    if (warp == 0) sum_rows<Q>(v, s_red, nw, lane);
     __syncthreads();
 }
 
 // Sum of the grid's block partials partials[b * kMaxQ + q] (b < nb) by one warp, in FP64 and a
-// fixed order (each lane adds the blocks b = lane, lane + 32, ... in turn, then a butterfly);
+// fixed order (each lane adds the blocks b = lane, lane + 32, ... in turn, then the lanes' sums);
 // call with all 32 lanes of the warp; the result is valid in every lane.
 template <int Q>
 __device__ __forceinline__ void warp_sum_partials(const double* partials, int nb, int lane, double (&w)[Q])
 {
 #pragma unroll
     for (int q = 0; q < Q; ++q) w[q] = 0.0;
-    for (int b = lane; b < nb; b += 32)
+    for (int b = lane; b < nb; b += 64) {  // two blocks' values under way at once
+        double x[2][Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) w[q] += __ldcg(&partials[(size_t)b * kMaxQ + q]);
+        for (int i = 0; i < 2; ++i)
+            if (b + 32 * i < nb)
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
-        for (int off = 16; off > 0; off >>= 1) w[q] += __shfl_xor_sync(0xffffffffu, w[q], off);
+                for (int q = 0; q < Q; ++q) x[i][q] = __ldcg(&partials[(size_t)(b + 32 * i) * kMaxQ + q]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (b + 32 * i < nb)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) w[q] += x[i][q];
+    }
+    __syncwarp();
+    warp_sums_all<Q>(w, lane);
 }
 
 // Block sum of per-thread accumulators acc[q] (nullptr: 0) into v[q], valid in thread 0:
@@ -309,61 +377,26 @@ __device__ __forceinline__ void block_reduce_acc(const Acc<T>* const (&acc)[Q], 
 }
 
 // block_reduce over the first nthr threads only (a multiple of 32), synchronising on the
-// named barrier `bar` instead of the whole block.
-template <int Q>
-__device__ __forceinline__ void group_reduce(double (&v)[Q], double (*s_red)[kMaxQ], int tid, int nthr, int bar)
-{
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-        for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-    const int warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < Q; ++q) s_red[warp][q] = v[q];
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            double x = lane < nw ? s_red[lane][q] : 0.0;
-            for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-            v[q] = x;
-        }
-    }
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
-}
-
-// group_reduce of per-thread accumulators acc[q] (nullptr: 0): compensated FP32 ones through
-// a float-pair warp stage, FP64 ones as group_reduce does.  Valid in thread 0 of the group.
+// named barrier `bar` instead of the whole block, of per-thread accumulators acc[q] (nullptr: 0):
+// compensated FP32 ones through a float-pair warp stage.  Valid in thread 0 of the group.
 template <typename T, int Q>
 __device__ __forceinline__ void group_reduce_acc(const Acc<T>* const (&acc)[Q], double (&v)[Q],
                                                  double (*s_red)[kMaxQ], int tid, int nthr, int bar)
 {
+    const int warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
     if constexpr (sizeof(T) == 4) {
-        const int warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
+        F2 x[Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            F2 x{acc[q] ? acc[q]->s : 0.f, acc[q] ? -acc[q]->c : 0.f};
-            for (int off = 16; off > 0; off >>= 1) {
-                const F2 o{__shfl_xor_sync(0xffffffffu, x.hi, off), __shfl_xor_sync(0xffffffffu, x.lo, off)};
-                x = f2_add(x, o);
-            }
-            if (lane == 0) s_red[warp][q] = (double)x.hi + (double)x.lo;
-        }
-        asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
-        if (warp == 0) {
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                double x = lane < nw ? s_red[lane][q] : 0.0;
-                for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-                v[q] = x;
-            }
-        }
-        asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
+        for (int q = 0; q < Q; ++q) x[q] = {acc[q] ? acc[q]->s : 0.f, acc[q] ? -acc[q]->c : 0.f};
+        warp_sums_to<Q>(x, s_red, warp, lane);
     } else {
 #pragma unroll
         for (int q = 0; q < Q; ++q) v[q] = acc[q] ? acc[q]->value() : 0.0;
-        group_reduce<Q>(v, s_red, tid, nthr, bar);
+        warp_sums_to<Q>(v, s_red, warp, lane);
     }
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
+    if (warp == 0) sum_rows<Q>(v, s_red, nw, lane);
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
 }
 
 // ---------------------------------------------------------------- lattice tiling and potential

@@ -87,7 +87,7 @@ struct cl_lattice {
     int opt_BY = 0, opt_DZ = 0, opt_stages = 0, opt_variant = -1;  // -1: library choice
     int u1_dz = 8;                  // planes per block of the U(1) kernels
     int u1_gdz = 8;                 // planes per block of the gather kernels beside staged ones
-    int u1_pdz = 8;                 // planes per block of the staged plaquette launches
+    U1Tile u1_tile{32, 8, 8}, u1_ptile{32, 8, 8};  // tiles of the staged stage and plaquette launches
     bool u1_fused = false;          // U(1) stage as one fused launch (plaquettes in shared memory)
     bool u1_staged = false;         // U(1) launches with shared-memory staged neighbourhoods
     bool u1_sfused = false;         //   as one launch, the plaquette fields in shared memory
@@ -672,16 +672,21 @@ cl_status choose_tiles(cl_lattice* l)
         int64_t nbz = (int64_t)bps * nsm / tiles;
         if (nbz < 1) nbz = 1;
         if (nbz > N) nbz = N;
-        const int auto_dz = l->u1_staged ? u1_staged_dz(prec, N, nsm, false) : (int)((N + nbz - 1) / nbz);
+        if (l->u1_staged) {
+            l->u1_tile = u1_staged_tile(prec, N, nsm, false, l->u1_sfused);
+            l->u1_ptile = u1_staged_tile(prec, N, nsm, true, false);
+        }
+        const int auto_dz = l->u1_staged ? l->u1_tile.dz : (int)((N + nbz - 1) / nbz);
         l->u1_dz = l->opt_DZ > 0 ? (l->opt_DZ > N ? N : l->opt_DZ) : auto_dz;
         // the gather kernels that run beside the staged launches (the Gauss diagnostic and its
         // plaquette fields) keep the gather form's one-wave chunks
         l->u1_gdz = l->u1_staged ? (int)((N + nbz - 1) / nbz) : l->u1_dz;
         if (2 * u1_grid_blocks(N, l->u1_dz) > nblocks) nblocks = 2 * u1_grid_blocks(N, l->u1_dz);  // stage + plaquette partials
         if (2 * u1_grid_blocks(N, l->u1_gdz) > nblocks) nblocks = 2 * u1_grid_blocks(N, l->u1_gdz);
-        l->u1_pdz = l->opt_DZ > 0 ? (l->u1_dz + 1) / 2 : u1_staged_dz(prec, N, nsm, true);
         if (l->u1_staged) {  // the stage's partials, then the plaquette launch's
-            const int need = u1_staged_blocks(prec, N, l->u1_dz, false) + u1_staged_blocks(prec, N, l->u1_pdz, true);
+            l->u1_tile.dz = l->u1_dz;
+            if (l->opt_DZ > 0) l->u1_ptile.dz = (l->u1_dz + 1) / 2;
+            const int need = u1_staged_blocks(l->u1_tile, N) + u1_staged_blocks(l->u1_ptile, N);
             if (need > nblocks) nblocks = need;
         }
     }
@@ -1149,9 +1154,13 @@ void u1_fill(cl_lattice* l, U1Args<T>& A, int in, int out)
     A.hubble_limit = l->hubble_limit;
     A.dz = l->u1_dz;
     if (l->u1_staged) {
-        A.pdz = l->u1_pdz;
-        A.pl_n = u1_staged_blocks(l->p.precision, l->N, l->u1_pdz, true);
-        A.pl_partials = l->partials + (size_t)u1_staged_blocks(l->p.precision, l->N, l->u1_dz, false) * kMaxQ;
+        A.tx = l->u1_tile.tx;
+        A.ty = l->u1_tile.ty;
+        A.ptx = l->u1_ptile.tx;
+        A.pty = l->u1_ptile.ty;
+        A.pdz = l->u1_ptile.dz;
+        A.pl_n = u1_staged_blocks(l->u1_ptile, l->N);
+        A.pl_partials = l->partials + (size_t)u1_staged_blocks(l->u1_tile, l->N) * kMaxQ;
     }
 }
 

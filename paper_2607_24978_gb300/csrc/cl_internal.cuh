@@ -250,7 +250,9 @@ struct U1Args {
     double hubble_limit;
     int flags;    // P_EXPANSION, P_FIRST_STAGE, P_COUNT_STEP, P_ENERGY_ONLY, P_HUBBLE_INIT
     int dz;       // planes per block (all three kernels)
-    int pdz;      // staged plaquette launches: planes per block, and where their pl_n partials go
+    int tx, ty;   // staged stage launches: sites of a tile
+    int ptx, pty; // staged plaquette launches: the same, planes per block, and where their pl_n
+    int pdz;      // partials go
     int pl_n;
     double* pl_partials;
     // Leapfrog passes (lf != 0; the stage launch only, the plaquette launch is unchanged).

@@ -8,25 +8,27 @@
 // The gather kernels of u1_stage.cu read 40 to 110 neighbour values per site from L1/L2
 // into registers; a thread can only keep as many loads in flight as it has registers, and
 // both kernels stall on memory latency at a fraction of the HBM bandwidth.  Here a block
-// owns a 32 x TY tile of (x, y) (stage launches: TY = 16 in FP32, 8 in FP64; plaquette
-// launches, which stage fewer arrays: twice that, over z chunks of their own) and marches up its z chunk with planes z-1, z, z+1 of every array that is read at a
-// neighbour in shared memory: rows y0-1 .. y0+TY and columns x0-VE .. x0+31+VE (VE elements
-// per 16 bytes, so that every row is whole 16-byte units; only the first and last columns
-// are read).  Warp roles, synchronised by mbarriers only:
+// owns a tx x ty tile of (x, y) (stage launches: at most 512 sites in FP32, 256 in FP64; plaquette
+// launches, which stage fewer arrays: twice that, over z chunks of their own) and marches up its z
+// chunk with planes z-1, z, z+1 of every array that is read at a neighbour in shared memory: rows
+// y0-1 .. y0+ty and columns x0-VE .. x0+tx-1+VE (VE elements per 16 bytes, so that every row is
+// whole 16-byte units; only the first and last columns are read).  Warp roles, synchronised by mbarriers only:
 //  * six producer warps copy plane after plane into a ring of five slots with 16-byte
 //    asynchronous copies (cp.async; the source of every 16-byte unit of a plane, periodic
 //    wrap included, is tabulated in shared memory once per block), and each lane's copies
 //    arrive on the slot's "full" barrier when they have landed (measured at 192^3 FP32: one
 //    producer warp, 2.5 Gsite-updates/s; two, 4.3; four, 6.3; six, 6.7; eight, 6.4;
 //    single bulk copies of each staged row, 1.1: many small bulk copies are slow);
-//  * TY consumer warps (one row of the tile each) wait for the planes they need, compute the
-//    site, and release a slot once they have read it for the last time (its "empty" barrier
+//  * the consumer warps (a site of the tile a thread, or two) wait for the planes they need, compute
+//    the site, and release a slot once they have read it for the last time (its "empty" barrier
 //    counts one arrival per consumer warp), so no warp waits for another one's work.
 // Arrays read only at the site itself (theta and the Runge-Kutta auxiliaries) are loaded by
 // the consumers straight from global memory, one plane ahead.  Every wait is bounded and
 // reports through the status word.  Needs rows of whole 16-byte units (u1_staged_ok); other sizes
 // use the gather kernels.
 #include <math.h>
+
+#include <algorithm>
 
 #include "cl_internal.cuh"
 #include "kernel_common.cuh"
@@ -35,8 +37,8 @@
 
 namespace clk {
 
-// Tile geometry: TX x TY sites a block, RW tile rows a consumer warp (rows w, w + CW, ...),
-// PWARPS producer warps.
+// Sizes of a block: the sites, staged elements and 16-byte units of a TX x TY tile (other shapes of
+// tile, U1STile, stay within them), RW sites a consumer thread, PWARPS producer warps.
 template <typename T_, int TY_, int PWARPS_, int RW_>
 struct U1SGeomT {
     using T = T_;
@@ -50,7 +52,8 @@ struct U1SGeomT {
     static constexpr int VE = 16 / (int)sizeof(T);
     static constexpr int PW = TX + 2 * VE;     // staged columns x0 - VE .. x0 + TX + VE - 1
     static constexpr int PH = TY + 2;          // staged rows y0 - 1 .. y0 + TY
-    static constexpr int ARR = PH * PW;        // elements of one array plane
+    static constexpr int ARR = PH * PW;        // elements of one array plane (at most, see U1STile)
+    static constexpr int SITES = TX * TY;      // sites of a tile (at most)
     static constexpr int CPR = PW / VE;        // 16-byte units of a staged row
     static constexpr int SLOTS = 5;
     static_assert(TY % RW == 0 && NT <= 1024, "tile rows a warp; threads a block");
@@ -91,31 +94,46 @@ static_assert(u1s_smem_bytes<U1PGeom<double>, PQ_NA>() + 2048 <= (size_t)kPassMa
 static_assert(u1s_smem_bytes<U1SGeom<float>, SG_NA>() + 2048 <= (size_t)kPassMaxSmem, "stage ring (FP32)");
 static_assert(u1s_smem_bytes<U1SGeom<double>, SG_NA>() + 2048 <= (size_t)kPassMaxSmem, "stage ring (FP64)");
 
-// Tile and z range of this block: chunk bz of dz planes (the last one may be shorter).  Where the
-// tiles do not divide N, the last tile of a row or column reaches past it: its copies wrap around
-// (they stage other sites' values, which nothing reads) and the sites past N compute on them
-// without storing or adding anything.
+// Tile and z range of this block: tx x ty sites (at most G::SITES, their halo at most G::ARR; tx of
+// whole 16-byte units), chunk bz of dz planes (the last one may be shorter).  Consumer thread c of
+// the block stands on tile site c, row after row, so a tile fills the warps whatever its width; its
+// staged rows are pw = tx + 2 VE elements.  Where the tiles do not divide N, the last tile of a row
+// or column reaches past it: its copies wrap around (they stage other sites' values, which nothing
+// reads) and the sites past N compute on them without storing or adding anything.
 template <typename G>
 struct U1STile {
-    uint32_t N, x0, y0, z0, nz;
-    __device__ __forceinline__ U1STile(uint32_t N_, uint32_t dz) : N(N_)
+    uint32_t N, tx, ty, pw, x0, y0, z0, nz;
+    __device__ __forceinline__ U1STile(uint32_t N_, uint32_t tx_, uint32_t ty_, uint32_t dz)
+        : N(N_), tx(tx_), ty(ty_), pw(tx_ + 2 * G::VE)
     {
-        const uint32_t ntx = (N + G::TX - 1) / G::TX, nty = (N + G::TY - 1) / G::TY;
+        const uint32_t ntx = (N + tx - 1) / tx, nty = (N + ty - 1) / ty;
         uint32_t b = blockIdx.x;
         const uint32_t bx = b % ntx;
         b /= ntx;
         const uint32_t by = b % nty, bz = b / nty;
-        x0 = bx * G::TX;
-        y0 = by * G::TY;
+        x0 = bx * tx;
+        y0 = by * ty;
         z0 = bz * dz;
         nz = z0 + dz < N ? dz : N - z0;
     }
-    // the site of tile column lx, row ly: whether it exists, and its index in plane 0 (a site past
-    // the lattice stands on the last one of its row or column)
-    __device__ __forceinline__ bool has(int lx, int ly) const { return x0 + lx < N && y0 + ly < N; }
-    __device__ __forceinline__ uint32_t at(int lx, int ly) const
+    // consumer warps that have a site
+    __device__ __forceinline__ int warps() const { return min(G::CW, (int)(tx * ty + 31) / 32); }
+};
+// Tile site c of the block: whether it exists, its index in plane 0 and its element of a staged plane
+// (a site past the tile or the lattice stands on another one).
+template <typename G>
+struct U1SSite {
+    bool has;
+    uint32_t at;
+    int off;
+    __device__ __forceinline__ U1SSite() {}
+    __device__ __forceinline__ U1SSite(const U1STile<G>& t, uint32_t c)
     {
-        return min(y0 + (uint32_t)ly, N - 1) * N + min(x0 + (uint32_t)lx, N - 1);
+        const bool in = c < t.tx * t.ty;
+        const uint32_t ly = in ? c / t.tx : 0, lx = in ? c - ly * t.tx : 0;
+        has = in && t.x0 + lx < t.N && t.y0 + ly < t.N;
+        at = min(t.y0 + ly, t.N - 1) * t.N + min(t.x0 + lx, t.N - 1);
+        off = (int)((ly + 1) * t.pw + lx + G::VE);
     }
 };
 
@@ -126,17 +144,17 @@ template <typename G, int NA>
 __device__ __forceinline__ void u1s_build_units(uint2* table, const U1STile<G>& t, int tid, int nthr)
 {
     using U = U1SUnits<G, NA>;
-    const int N = (int)t.N;
+    const int N = (int)t.N, cpr = (int)t.pw / G::VE, per = ((int)t.ty + 2) * cpr, ch = NA * per;
     for (int e = tid; e < G::PL * U::PER_LANE; e += nthr) {
         const int lane = e % G::PL, i = e / G::PL, c = lane + G::PL * i;
         uint2 v = make_uint2(0xffffffffu, 0u);
-        if (c < U::CH) {
-            const int a = c / (G::PH * G::CPR), rem = c - a * (G::PH * G::CPR);
-            const int r = rem / G::CPR, u = rem - r * G::CPR;
-            int gy = (int)t.y0 - 1 + r, gx = (int)t.x0 - G::VE + u * G::VE;  // in [-1, N + TY) and [-VE, N + TX)
+        if (c < ch) {
+            const int a = c / per, rem = c - a * per;
+            const int r = rem / cpr, u = rem - r * cpr;
+            int gy = (int)t.y0 - 1 + r, gx = (int)t.x0 - G::VE + u * G::VE;  // in [-1, N + ty] and [-VE, N + tx)
             gy = gy < 0 ? gy + N : (gy >= N ? gy - N : gy);
             gx = gx < 0 ? gx + N : (gx >= N ? gx - N : gx);
-            v.x = ((uint32_t)a << 16) | (uint32_t)(a * G::ARR + r * G::PW + u * G::VE);
+            v.x = ((uint32_t)a << 16) | (uint32_t)(a * G::ARR + r * (int)t.pw + u * G::VE);
             v.y = (uint32_t)gy * (uint32_t)N + (uint32_t)gx;
         }
         table[i * G::PL + lane] = v;
@@ -178,9 +196,10 @@ template <typename G>
 struct U1SNb {
     using T = typename G::T;
     const T* p[3];
+    int pw;  // elements of a staged row
     __device__ __forceinline__ T operator()(int a, int ox, int oy, int oz) const
     {
-        return p[oz + 1][a * G::ARR + oy * G::PW + ox];
+        return (p[oz + 1] + oy * pw)[a * G::ARR + ox];
     }
     __device__ __forceinline__ T at(int a, const int (&o)[3]) const { return (*this)(a, o[0], o[1], o[2]); }
     // clover sum of array a (normal k) over the four plaquettes around the site at offset o
@@ -235,13 +254,13 @@ struct U1SRing {
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[q % G::SLOTS]);
     }
-    // the three planes of output plane j at the consumer's site (row ly, column lx)
-    __device__ __forceinline__ U1SNb<G> nb(int j, int lx, int ly) const
+    // the three planes of output plane j at the consumer's site (element `off` of a plane)
+    __device__ __forceinline__ U1SNb<G> nb(int j, int off, int pw) const
     {
-        const int t0 = (ly + 1) * G::PW + lx + G::VE;
         U1SNb<G> n;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) n.p[i] = sm + ((j + i) % G::SLOTS) * SLOT + t0;
+        for (int i = 0; i < 3; ++i) n.p[i] = sm + ((j + i) % G::SLOTS) * SLOT + off;
+        n.pw = pw;
         return n;
     }
 };
@@ -249,7 +268,7 @@ struct U1SRing {
 // unit offset vector along axis d with sign s
 #define U1S_E(d, s) ((d) == 0 ? (s) : 0), ((d) == 1 ? (s) : 0), ((d) == 2 ? (s) : 0)
 
-template <typename T>
+template <typename T, bool W32>
 __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Args<T> A)
 {
     using G = U1PGeom<T>;
@@ -260,6 +279,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
     __shared__ double s_red[G::NT / 32][kMaxQ];  // a row for every warp; the sum takes the consumers'
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const U1STile<G> t((uint32_t)A.N, W32 ? G::TX : (uint32_t)A.ptx, (uint32_t)A.pty, (uint32_t)A.pdz);
     if (tid == 0) {
         s_src[PQ_PHI] = A.phi_in;
 #pragma unroll
@@ -269,13 +289,12 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
         }
         for (int k = 0; k < G::SLOTS; ++k) {
             mbar_init(&s_full[k], G::PL);  // the producer lanes' copies
-            mbar_init(&s_empty[k], G::CW);
+            mbar_init(&s_empty[k], t.warps());
         }
         mbar_fence_init();
         s_fail = 0;
     }
     __syncthreads();
-    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.pdz);
     T* ring_sm = reinterpret_cast<T*>(u1s_dyn);
     uint2* table = reinterpret_cast<uint2*>(ring_sm + G::SLOTS * NA * G::ARR);
     u1s_build_units<G, NA>(table, t, tid, G::NT);
@@ -284,9 +303,12 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
     Acc<T> accGB;
     if (warp >= G::CW) {
         ring.produce(tid - 32 * G::CW, s_src, t);
-    } else {
+    } else if (warp < t.warps()) {
         const uint32_t N = t.N;
         const T dx = (T)A.dx;
+        U1SSite<G> site[G::RW];
+#pragma unroll
+        for (int r = 0; r < G::RW; ++r) site[r] = U1SSite<G>(t, tid + r * 32 * G::CW);
         ring.acquire(0);
         ring.acquire(1);
         for (int j = 0; j < (int)t.nz; ++j) {
@@ -296,7 +318,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
             for (int r = 0; r < G::RW; ++r)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const U1SNb<G> S = ring.nb(j, lane, warp + r * G::CW);
+                const U1SNb<G> S = ring.nb(j, site[r].off, (int)t.pw);
                 const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
                 const T P = S(PQ_TH + k1, 0, 0, 0) + S(PQ_TH + k2, U1S_E(k1, 1)) - S(PQ_TH + k1, U1S_E(k2, 1)) -
                             S(PQ_TH + k2, 0, 0, 0);
@@ -318,13 +340,13 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
                 o_r[r][k] = cp * R;
                 o_z[r][k] = cp * ((T)0.5 * qs);
                 o_c[r][k] = cp;
-                accGB.add(t.has(lane, warp + r * G::CW) ? (T)2 * sh * sh : (T)0);
+                accGB.add(site[r].has ? (T)2 * sh * sh : (T)0);
             }
             ring.release(j, lane);
 #pragma unroll
             for (int r = 0; r < G::RW; ++r) {
-                if (!t.has(lane, warp + r * G::CW)) continue;
-                const uint32_t n = (t.z0 + j) * N * N + t.at(lane, warp + r * G::CW);
+                if (!site[r].has) continue;
+                const uint32_t n = (t.z0 + j) * N * N + site[r].at;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     A.sP[k][n] = o_s[r][k];
@@ -354,7 +376,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquettes(const U1Ar
 // of the previous pass 1, whose plaquette launch saved cos P.
 enum { RQ_PHI = 0, RQ_E = 1, RQ_NA = 4 };
 
-template <typename T>
+template <typename T, bool W32>
 __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const U1Args<T> A)
 {
     using G = U1PGeom<T>;
@@ -364,19 +386,19 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
     __shared__ __align__(8) uint64_t s_full[G::SLOTS], s_empty[G::SLOTS];
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const U1STile<G> t((uint32_t)A.N, W32 ? G::TX : (uint32_t)A.ptx, (uint32_t)A.pty, (uint32_t)A.pdz);
     if (tid == 0) {
         s_src[RQ_PHI] = A.phi_in;
 #pragma unroll
         for (int k = 0; k < 3; ++k) s_src[RQ_E + k] = A.E_in[k];
         for (int k = 0; k < G::SLOTS; ++k) {
             mbar_init(&s_full[k], G::PL);  // the producer lanes' copies
-            mbar_init(&s_empty[k], G::CW);
+            mbar_init(&s_empty[k], t.warps());
         }
         mbar_fence_init();
         s_fail = 0;
     }
     __syncthreads();
-    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.pdz);
     T* ring_sm = reinterpret_cast<T*>(u1s_dyn);
     uint2* table = reinterpret_cast<uint2*>(ring_sm + G::SLOTS * NA * G::ARR);
     u1s_build_units<G, NA>(table, t, tid, G::NT);
@@ -384,19 +406,19 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
     const U1SRing<G, NA> ring{ring_sm, table, s_full, s_empty, &s_fail};
     if (warp >= G::CW) {
         ring.produce(tid - 32 * G::CW, s_src, t);
-    } else {
+    } else if (warp < t.warps()) {
         const uint32_t N = t.N;
         const T dx = (T)A.dx;
+        U1SSite<G> site[G::RW];
+#pragma unroll
+        for (int r = 0; r < G::RW; ++r) site[r] = U1SSite<G>(t, tid + r * 32 * G::CW);
         // cos P of the sites' three plaquettes, loaded one plane ahead
         T cc[G::RW][3];
-        uint32_t at[G::RW];
-#pragma unroll
-        for (int r = 0; r < G::RW; ++r) at[r] = t.at(lane, warp + r * G::CW);
         auto load_c = [&](uint32_t plane) {
 #pragma unroll
             for (int r = 0; r < G::RW; ++r)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) cc[r][k] = A.cP[k][plane + at[r]];
+                for (int k = 0; k < 3; ++k) cc[r][k] = A.cP[k][plane + site[r].at];
         };
         load_c(t.z0 * N * N);
         ring.acquire(0);
@@ -415,7 +437,7 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
             for (int r = 0; r < G::RW; ++r)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const U1SNb<G> S = ring.nb(j, lane, warp + r * G::CW);
+                const U1SNb<G> S = ring.nb(j, site[r].off, (int)t.pw);
                 const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
                 const T R = dx * (S(RQ_E + k1, 0, 0, 0) + S(RQ_E + k2, U1S_E(k1, 1)) - S(RQ_E + k1, U1S_E(k2, 1)) -
                                   S(RQ_E + k2, 0, 0, 0));
@@ -432,11 +454,11 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
             ring.release(j, lane);
 #pragma unroll
             for (int r = 0; r < G::RW; ++r) {
-                if (!t.has(lane, warp + r * G::CW)) continue;
+                if (!site[r].has) continue;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    A.rP[k][plane + at[r]] = o_r[r][k];
-                    A.Z[k][plane + at[r]] = o_z[r][k];
+                    A.rP[k][plane + site[r].at] = o_r[r][k];
+                    A.Z[k][plane + site[r].at] = o_z[r][k];
                 }
             }
         }
@@ -451,7 +473,10 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
 // input state (the state at the step's start), so that the Gauss constraint is tracked each
 // step; a separate instance keeps that work, and its registers, out of the other stages.
 // LF: the passes of the leapfrog (U1Args::lf) instead of a Runge-Kutta stage.
-template <typename T, bool TRACK, bool LF>
+// W32: tiles of 32 columns, the staged rows' length and a thread's row constants (the kernel is at
+// its register limit: with variable ones the stages at 192^3 take 201 and 241 us instead of 198
+// and 231, the plaquettes 105 instead of 101).
+template <typename T, bool TRACK, bool LF, bool W32>
 __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T> A)
 {
     using G = U1SGeom<T>;
@@ -463,6 +488,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     __shared__ double s_red[32][kMaxQ];
     __shared__ int s_last, s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const U1STile<G> t((uint32_t)A.N, W32 ? G::TX : (uint32_t)A.tx, (uint32_t)A.ty, (uint32_t)A.dz);
     const bool first = !LF && (A.flags & P_FIRST_STAGE) != 0;
     const int lf = LF ? A.lf : 0;
     const bool update = (A.flags & P_ENERGY_ONLY) == 0;
@@ -489,13 +515,12 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
         }
         for (int k = 0; k < G::SLOTS; ++k) {
             mbar_init(&s_full[k], G::PL);  // the producer lanes' copies
-            mbar_init(&s_empty[k], G::CW);
+            mbar_init(&s_empty[k], t.warps());
         }
         mbar_fence_init();
         s_fail = 0;
     }
     __syncthreads();
-    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.dz);
     T* ring_sm = reinterpret_cast<T*>(u1s_dyn);
     uint2* table = reinterpret_cast<uint2*>(ring_sm + G::SLOTS * NA * G::ARR);
     u1s_build_units<G, NA>(table, t, tid, G::NT);
@@ -505,7 +530,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     Acc<T> accK, accG, accV, accKE, accGs;
     if (warp >= G::CW) {
         ring.produce(tid - 32 * G::CW, s_src, t);
-    } else {
+    } else if (warp < t.warps()) {
         const T c_dphi = (T)s_coef[0], cL = (T)s_coef[1], cV = (T)s_coef[2], cE = (T)s_coef[3], cfr = (T)s_coef[4];
         const T ca = (T)s_coef[6];
         const T g = (T)A.g, ws2 = (T)A.ws2, dx = (T)A.dx, m2 = (T)A.m2, lam = (T)A.lam;
@@ -534,14 +559,15 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                 for (int q = 0; q < 8; ++q) kc[q] = first ? (T)0 : A.k_in[q][m];
             }
         };
-        const bool has = t.has(lane, warp);
-        const uint32_t at = t.at(lane, warp);
+        const U1SSite<G> site(t, tid);
+        const bool has = site.has;
+        const uint32_t at = site.at;
         if (update) load_site(t.z0 * N * N + at);
         ring.acquire(0);
         ring.acquire(1);
         for (int j = 0; j < (int)t.nz; ++j) {
             ring.acquire(j + 2);
-            const U1SNb<G> S = ring.nb(j, lane, warp);
+            const U1SNb<G> S = ring.nb(j, site.off, (int)t.pw);
             const uint32_t n = (t.z0 + j) * N * N + at;
             T thv[3], kv[8];
 #pragma unroll
@@ -776,6 +802,7 @@ __device__ __forceinline__ U1SNb<U1SGeom<T>> u1f_raw(const T* ring, int c, int l
     U1SNb<U1SGeom<T>> n;
 #pragma unroll
     for (int i = 0; i < 3; ++i) n.p[i] = ring + ((c - 1 + i + G::SLOTS) % G::SLOTS) * SL + t0;
+    n.pw = G::PW;
     return n;
 }
 
@@ -870,6 +897,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1f_stage(const U1Args<T>
     __shared__ double s_red[32][kMaxQ];
     __shared__ int s_last, s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const U1STile<G> t((uint32_t)A.N, G::TX, G::TY, (uint32_t)A.dz);
     const bool first = !LF && (A.flags & P_FIRST_STAGE) != 0;
     const int lf = LF ? A.lf : 0;
     const bool update = (A.flags & P_ENERGY_ONLY) == 0;
@@ -894,13 +922,12 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1f_stage(const U1Args<T>
         }
         for (int k = 0; k < G::SLOTS; ++k) {
             mbar_init(&s_full[k], G::PL);  // the producer lanes' copies
-            mbar_init(&s_empty[k], G::CW);
+            mbar_init(&s_empty[k], t.warps());
         }
         mbar_fence_init();
         s_fail = 0;
     }
     __syncthreads();
-    const U1STile<G> t((uint32_t)A.N, (uint32_t)A.dz);
     T* ring_sm = reinterpret_cast<T*>(u1s_dyn);
     uint2* table = reinterpret_cast<uint2*>(ring_sm + G::SLOTS * NA * G::ARR);
     T* pq = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(u1s_dyn) + u1s_smem_bytes<G, NA>());
@@ -1131,36 +1158,65 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1f_stage(const U1Args<T>
 // one row and unit past the lattice's width.
 bool u1_staged_ok(int precision, int N) { return N >= 32 && N % (precision == CL_PREC_FP64 ? 2 : 4) == 0; }
 
-static int u1s_tiles(int precision, int N, bool plaquettes)
-{
-    const int ty = precision == CL_PREC_FP64 ? (plaquettes ? U1PGeom<double>::TY : U1SGeom<double>::TY)
-                                             : (plaquettes ? U1PGeom<float>::TY : U1SGeom<float>::TY);
-    return ((N + 31) / 32) * ((N + ty - 1) / ty);
-}
+int u1_staged_blocks(const U1Tile& t, int N) { return ((N + t.tx - 1) / t.tx) * ((N + t.ty - 1) / t.ty) * ((N + t.dz - 1) / t.dz); }
 
-int u1_staged_blocks(int precision, int N, int dz, bool plaquettes)
+// The tile and z chunk of a launch: one block per SM at a time, so the busiest SM's
+// waves x (planes + 2 halo planes) x the time of a plane.  That time: a share for each consumer warp
+// that has sites, three such for staging the fullest tile, one for the plane itself; 6% more for
+// widths other than 32, which are not constants of the kernel (128^3 stage with tiles of 128 columns:
+// 99 us against 84); widths that are no multiple of 32 put the end of one row and the start of
+// another, eight banks apart, into one warp: 16% more for each row end in a warp.  Measured (us,
+// stage / plaquettes, tiles of 32 columns against those chosen): 100^3 63.3 / 33.8 against 54.7 /
+// 21.0 (100 columns, FP32 RK3-3), 132^3 110.9 / 56.0 against 96.5 / 43.3 (68 and 132), 200^3
+// leapfrog 243 / 156 against 238 / 136 (100 and 200).
+template <typename G>
+static U1Tile u1s_choose(int N, int nsm, bool fixed)
 {
-    return u1s_tiles(precision, N, plaquettes) * ((N + dz - 1) / dz);
-}
-
-// z chunk of the staged launches: one block per SM at a time, so the chunk count minimises
-// waves x (planes + 2 halo planes) of the busiest SM.
-int u1_staged_dz(int precision, int N, int nsm, bool plaquettes)
-{
-    const long long tiles = u1s_tiles(precision, N, plaquettes);
-    long long best = -1;
-    int best_dz = N;
-    for (int nbz = 1; nbz <= N; ++nbz) {
-        const int dz = (N + nbz - 1) / nbz;
-        if ((N + dz - 1) / dz != nbz) continue;  // same chunks as a smaller count
-        const long long waves = (tiles * nbz + nsm - 1) / nsm;
-        const long long cost = waves * (dz + 2);
-        if (best < 0 || cost < best) {
-            best = cost;
-            best_dz = dz;
+    U1Tile best{G::TX, G::TY, N};
+    double best_cost = -1.0;
+    auto consider = [&](int tx, int ty) {
+        const long long tiles = (long long)((N + tx - 1) / tx) * ((N + ty - 1) / ty);
+        const double staged = 3.0 * (ty + 2) * (tx + 2 * G::VE) / G::ARR;
+        const double plane = ((tx * ty + 31) / 32 + 1.0 + staged) * (tx == G::TX ? 1.0 : 1.06 + (tx % 32 ? 0.16 * 32.0 / tx : 0.0));
+        for (int nbz = 1; nbz <= N; ++nbz) {
+            const int dz = (N + nbz - 1) / nbz;
+            if ((N + dz - 1) / dz != nbz) continue;  // same chunks as a smaller count
+            const long long waves = (tiles * nbz + nsm - 1) / nsm;
+            const double cost = (double)waves * (dz + 2) * plane;
+            if (best_cost < 0.0 || cost < best_cost) {
+                best_cost = cost;
+                best = {tx, ty, dz};
+            }
         }
+    };
+    auto rows = [&](int tx) {  // the most rows, shared evenly among as many tiles
+        const int ty = std::min({G::SITES / tx, G::ARR / (tx + 2 * G::VE) - 2, N});
+        if (ty < 1) return;
+        const int nty = (N + ty - 1) / ty;
+        consider(tx, (N + nty - 1) / nty);
+    };
+    if (fixed) {
+        consider(G::TX, G::TY);
+        return best;
     }
-    return best_dz;
+    rows(G::TX);
+    for (int n = 1; n * G::VE <= N; ++n)  // n tiles across, as even as whole 16-byte units allow
+        rows(((N + n - 1) / n + G::VE - 1) / G::VE * G::VE);
+    return best;
+}
+
+U1Tile u1_staged_tile(int precision, int N, int nsm, bool plaquettes, bool fixed)
+{
+    if (precision == CL_PREC_FP64)
+        return plaquettes ? u1s_choose<U1PGeom<double>>(N, nsm, fixed) : u1s_choose<U1SGeom<double>>(N, nsm, fixed);
+    return plaquettes ? u1s_choose<U1PGeom<float>>(N, nsm, fixed) : u1s_choose<U1SGeom<float>>(N, nsm, fixed);
+}
+
+template <typename G>
+static bool u1s_tile_ok(int N, int tx, int ty, int dz)
+{
+    return tx >= G::VE && tx <= N && tx % G::VE == 0 && ty >= 1 && ty <= N && dz >= 1 && dz <= N &&
+           tx * ty <= G::SITES && (ty + 2) * (tx + 2 * G::VE) <= G::ARR;
 }
 
 template <typename T>
@@ -1168,32 +1224,27 @@ static cudaError_t launch_u1s_t(const U1Args<T>& A, int what, cudaStream_t s)
 {
     using G = U1SGeom<T>;
     const int prec = sizeof(T) == 8 ? CL_PREC_FP64 : CL_PREC_FP32;
-    if (!u1_staged_ok(prec, A.N) || A.dz < 1 || A.dz > A.N) return cudaErrorInvalidValue;
-    if (what != 2 && (A.pdz < 1 || A.pdz > A.N || !A.pl_partials)) return cudaErrorInvalidValue;
-    if (what == 2 && A.N % 32 != 0) return cudaErrorInvalidValue;  // the fused form's tiles divide N
-    const int grid = u1_staged_blocks(prec, A.N, A.dz, false);
-    const int pgrid = what != 2 ? u1_staged_blocks(prec, A.N, A.pdz, true) : 0;
-    static DevFlag attr[5];
-    if (what == 0) {
-        constexpr size_t smem = u1s_smem_bytes<U1PGeom<T>, PQ_NA>();
-        if (!attr[0]) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(k_u1s_plaquettes<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (!u1_staged_ok(prec, A.N) || !u1s_tile_ok<G>(A.N, A.tx, A.ty, A.dz)) return cudaErrorInvalidValue;
+    if (what != 2 && (!u1s_tile_ok<U1PGeom<T>>(A.N, A.ptx, A.pty, A.pdz) || !A.pl_partials))
+        return cudaErrorInvalidValue;
+    if (what == 2 && (A.N % 32 != 0 || A.tx != G::TX || A.ty != G::TY))
+        return cudaErrorInvalidValue;  // the fused form's tiles divide N
+    const int grid = u1_staged_blocks({A.tx, A.ty, A.dz}, A.N);
+    const int pgrid = what != 2 ? u1_staged_blocks({A.ptx, A.pty, A.pdz}, A.N) : 0;
+    if (what == 0 || what == 3) {
+        const size_t smem = what == 0 ? u1s_smem_bytes<U1PGeom<T>, PQ_NA>() : u1s_smem_bytes<U1PGeom<T>, RQ_NA>();
+        if (what == 3 && (!A.cP[0] || !A.cP[1] || !A.cP[2])) return cudaErrorInvalidValue;
+        const bool w32 = A.ptx == U1PGeom<T>::TX;
+        const auto kernel = what == 0 ? (w32 ? k_u1s_plaquettes<T, true> : k_u1s_plaquettes<T, false>)
+                                      : (w32 ? k_u1s_plaquette_rates<T, true> : k_u1s_plaquette_rates<T, false>);
+        static DevFlag attr[2][2];
+        DevFlag& done = attr[what == 0 ? 0 : 1][w32 ? 1 : 0];
+        if (!done) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            attr[0] = true;
+            done = true;
         }
-        k_u1s_plaquettes<T><<<pgrid, U1PGeom<T>::NT, smem, s>>>(A);
-    } else if (what == 3) {
-        constexpr size_t smem = u1s_smem_bytes<U1PGeom<T>, RQ_NA>();
-        if (!A.cP[0] || !A.cP[1] || !A.cP[2]) return cudaErrorInvalidValue;
-        static DevFlag rattr;
-        if (!rattr) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(k_u1s_plaquette_rates<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            rattr = true;
-        }
-        k_u1s_plaquette_rates<T><<<pgrid, U1PGeom<T>::NT, smem, s>>>(A);
+        kernel<<<pgrid, U1PGeom<T>::NT, smem, s>>>(A);
     } else if (what == 2) {
         constexpr size_t smem = u1f_smem_bytes<T>();
         const int form = A.lf ? (A.lf == 2 ? 4 : 3) : ((A.flags & P_FIRST_STAGE) && !(A.flags & P_ENERGY_ONLY) ? 2 : 1);
@@ -1217,20 +1268,22 @@ static cudaError_t launch_u1s_t(const U1Args<T>& A, int what, cudaStream_t s)
         // forms: 1 a Runge-Kutta stage, 2 the first stage of a step (Gauss tracking), 3 a
         // leapfrog pass, 4 the leapfrog's second pass (Gauss tracking)
         const int form = A.lf ? (A.lf == 2 ? 4 : 3) : ((A.flags & P_FIRST_STAGE) && !(A.flags & P_ENERGY_ONLY) ? 2 : 1);
-        if (!attr[form]) {
-            const int sm = (int)smem;
-            const cudaError_t e =
-                form == 4   ? cudaFuncSetAttribute(k_u1s_stage<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                : form == 3 ? cudaFuncSetAttribute(k_u1s_stage<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                : form == 2 ? cudaFuncSetAttribute(k_u1s_stage<T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                            : cudaFuncSetAttribute(k_u1s_stage<T, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        const auto kernel = A.tx == G::TX ? (form == 4   ? k_u1s_stage<T, true, true, true>
+                                             : form == 3 ? k_u1s_stage<T, false, true, true>
+                                             : form == 2 ? k_u1s_stage<T, true, false, true>
+                                                         : k_u1s_stage<T, false, false, true>)
+                                          : (form == 4   ? k_u1s_stage<T, true, true, false>
+                                             : form == 3 ? k_u1s_stage<T, false, true, false>
+                                             : form == 2 ? k_u1s_stage<T, true, false, false>
+                                                         : k_u1s_stage<T, false, false, false>);
+        static DevFlag sattr[2][5];
+        DevFlag& done = sattr[A.tx == G::TX ? 1 : 0][form];
+        if (!done) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            attr[form] = true;
+            done = true;
         }
-        if (form == 4) k_u1s_stage<T, true, true><<<grid, G::NT, smem, s>>>(A);
-        else if (form == 3) k_u1s_stage<T, false, true><<<grid, G::NT, smem, s>>>(A);
-        else if (form == 2) k_u1s_stage<T, true, false><<<grid, G::NT, smem, s>>>(A);
-        else k_u1s_stage<T, false, false><<<grid, G::NT, smem, s>>>(A);
+        kernel<<<grid, G::NT, smem, s>>>(A);
     }
     return cudaGetLastError();
 }

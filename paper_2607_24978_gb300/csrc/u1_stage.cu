@@ -369,7 +369,6 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
         if (mode == 1) gsq_s.add(G);
     }
     const double gsq = gsq_s.value(), e2 = e2_s.value();
-    double gmax = (double)gmx / A.dx, smax = (double)smx / A.dx;
     if (mode == 1) {  // sums in a fixed order, then the last block stores the tracked value
         double v[2] = {gsq, e2};
         block_reduce<2>(v, s_red, tid, nthr);
@@ -395,36 +394,47 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
         }
         return;
     }
-    // block maxima (fixed order), then the last block combines them
-    for (int off = 16; off > 0; off >>= 1) {
-        gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, off));
-        smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, off));
-    }
+    // block maxima, then the last block combines them, a thread's share of the blocks each (by one
+    // thread, 576 blocks of a 48^3 lattice took 90 us)
     const int warp = tid >> 5, lane = tid & 31, nw = (nthr + 31) >> 5;
-    if (lane == 0) {
-        s_red[warp][0] = gmax;
-        s_red[warp][1] = smax;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < nw; ++w) {
-            gmax = fmax(gmax, s_red[w][0]);
-            smax = fmax(smax, s_red[w][1]);
+    auto warp_max = [](T x) {
+        for (int off = 16; off > 0; off >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, off));
+        return x;
+    };
+    T* const s_max = reinterpret_cast<T*>(&s_red[0][0]);  // 2 a warp
+    auto block_max = [&](T& g, T& c) {                   // valid in thread 0
+        g = warp_max(g);
+        c = warp_max(c);
+        if (lane == 0) {
+            s_max[2 * warp] = g;
+            s_max[2 * warp + 1] = c;
         }
-        A.partials[(size_t)blockIdx.x * kMaxQ + 0] = gmax;
-        A.partials[(size_t)blockIdx.x * kMaxQ + 1] = smax;
+        __syncthreads();
+        if (tid == 0)
+            for (int w = 1; w < nw; ++w) {
+                g = fmax(g, s_max[2 * w]);
+                c = fmax(c, s_max[2 * w + 1]);
+            }
+    };
+    block_max(gmx, smx);
+    if (tid == 0) {
+        A.partials[(size_t)blockIdx.x * kMaxQ + 0] = (double)gmx;
+        A.partials[(size_t)blockIdx.x * kMaxQ + 1] = (double)smx;
         __threadfence();
         const unsigned prev = atomicAdd(&A.scal->counter, 1u);
         s_last = (prev + 1u == gridDim.x);
     }
     __syncthreads();
-    if (!s_last || tid != 0) return;
+    if (!s_last) return;
     __threadfence();
-    double G = 0.0, Sc = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) {
-        G = fmax(G, __ldcg(&A.partials[(size_t)b * kMaxQ + 0]));
-        Sc = fmax(Sc, __ldcg(&A.partials[(size_t)b * kMaxQ + 1]));
+    T gall = (T)0, sall = (T)0;
+    for (int b = tid; b < (int)gridDim.x; b += nthr) {
+        gall = fmax(gall, (T)__ldcg(&A.partials[(size_t)b * kMaxQ + 0]));
+        sall = fmax(sall, (T)__ldcg(&A.partials[(size_t)b * kMaxQ + 1]));
     }
+    block_max(gall, sall);
+    if (tid != 0) return;
+    const double G = (double)gall / A.dx, Sc = (double)sall / A.dx;
     A.scal->diag[D_GV] = Sc > 0.0 ? G / Sc : 0.0;
     A.scal->counter = 0u;
 }

@@ -28,10 +28,6 @@ __global__ void __launch_bounds__(480, 1) k_gw_pass_tma(const GwPassArgs<float> 
     float* stage = reinterpret_cast<float*>(gw_smem);
     const int units = A.nby * A.nbz * kGwC;
     if (tid == 0) {
-        const bool expand = (A.flags & P_EXPANSION) != 0;
-        const double a_new = A.scal->a, a_old = expand ? A.scal->a_prev : a_new;
-        s_coef[0] = A.d * apow(0.5 * (a_old + a_new), A.alpha - 3.0);
-        s_coef[1] = apow(a_new, 1.0 + A.alpha);
         for (int s = 0; s < S; ++s) {
             mbar_init(&s_full[s], 1);
             mbar_init(&s_empty[s], CW);
@@ -83,6 +79,13 @@ __global__ void __launch_bounds__(480, 1) k_gw_pass_tma(const GwPassArgs<float> 
     } else {
         using P2 = Two<float>;
         const bool do_drift = (A.flags & P_DRIFT) != 0;
+        if (tid < 2) {  // beside the copies of the first planes
+            const bool expand = (A.flags & P_EXPANSION) != 0;
+            const double a_new = A.scal->a, a_old = expand ? A.scal->a_prev : a_new;
+            const double p = apow(tid == 0 ? 0.5 * (a_old + a_new) : a_new, tid == 0 ? A.alpha - 3.0 : 1.0 + A.alpha);
+            s_coef[tid] = tid == 0 ? A.d * p : p;
+        }
+        named_barrier_sync(3, CT);
         const P2 cd = both((float)s_coef[0]), six = both(-6.f);
         const P2 cL = both((float)(s_coef[1] / (A.dx * A.dx)));
         const P2 cS = both((float)(2.0 * A.kappa * s_coef[1] * 0.25 / (A.dx * A.dx)));  // with the (1/2dx)^2 of the source

@@ -344,14 +344,6 @@ __global__ void __launch_bounds__(480, 1) k_rk_stage_tma(const RkStageArgs<T> A)
     block_units(N, A.nby, A.DZ, u0, u1);
 
     if (tid == 0) {
-        const double a = A.scal->a;
-        const double h = (A.flags & P_DEVICE_H) ? A.scal->h : A.h;  // adaptive steps: the device's h
-        s_coef[0] = h * apow(a, A.alpha - 3.0);
-        s_coef[1] = h * apow(a, 1.0 + A.alpha) / (A.dx * A.dx);
-        s_coef[2] = h * apow(a, 3.0 + A.alpha);
-        s_coef[3] = a;
-        s_coef[5] = h;
-        s_coef[4] = A.nmc ? A.xi * A.scal->rbar : 0.0;  // xi R of the stage's state
 #pragma unroll
         for (int k = 0; k < S; ++k) {
             mbar_init(&s_full[k], 1);
@@ -433,6 +425,21 @@ __global__ void __launch_bounds__(480, 1) k_rk_stage_tma(const RkStageArgs<T> A)
         }
     } else {
         // ---------------------------------------------------------------- consumer warps
+        // the stage's prefactors, lanes side by side, beside the copies of the first planes (before
+        // them, by one thread, they kept the producer waiting)
+        if (tid < 3) {
+            const double a = A.scal->a;
+            const double h = (A.flags & P_DEVICE_H) ? A.scal->h : A.h;  // adaptive steps: the device's h
+            double p = h * apow(a, tid == 0 ? A.alpha - 3.0 : tid == 1 ? 1.0 + A.alpha : 3.0 + A.alpha);
+            if (tid == 1) p = p / (A.dx * A.dx);
+            s_coef[tid] = p;
+            if (tid == 0) {
+                s_coef[3] = a;
+                s_coef[5] = h;
+                s_coef[4] = A.nmc ? A.xi * A.scal->rbar : 0.0;  // xi R of the stage's state
+            }
+        }
+        named_barrier_sync(3, CT);
         const T cphi = (T)s_coef[0], cL = (T)s_coef[1], cV = (T)s_coef[2], xiR = (T)s_coef[4];
         const T cA = (T)A.A, cB = (T)A.B;
         const PotCoef<T> P(A.m2, A.lam, A.g2);

@@ -42,6 +42,27 @@ __device__ __forceinline__ void pass_coefficients_warps(int tid, const double a_
     }
 }
 
+// The same by the consumers of a staged pass (threads 0 .. nthr - 1, whole warps), beside the copies
+// of the first planes: the producer needs none of them, and 2300 cycles of one thread's FP64 work
+// before the block's first load are 1.2 us of every pass.  Lanes 0, 1 and 2 of the first warp raise
+// a to the three powers side by side; all consumers wait for them on named barrier 3.
+__device__ __forceinline__ void consumer_coefficients(int tid, int nthr, const double a_old, const double b_old,
+                                                      const double d, const double alpha, const double dx,
+                                                      const bool expand, double* s_coef)
+{
+    if (tid < 3) {
+        const double a_new = expand ? a_old + d * b_old : a_old;
+        double p = apow(tid == 0 ? 0.5 * (a_old + a_new) : a_new, tid == 0 ? alpha - 3.0 : tid == 1 ? 1.0 + alpha : 3.0 + alpha);
+        if (tid == 0) {
+            p = d * p;
+            s_coef[3] = a_new;
+        }
+        if (tid == 1) p = p / (dx * dx);
+        s_coef[tid] = p;
+    }
+    named_barrier_sync(3, nthr);
+}
+
 // Kick of one own-row vector of a plane.  S*[f] point at row (r+1) of the centre
 // (Sc), lower (Szm) and upper (Szp) planes of field f; rows r and r+2 of the
 // centre plane are Sc -/+ N.  Writes pi_out and accumulates K, G, V.

@@ -46,7 +46,6 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
     block_units(N, A.nby, A.DZ, u0, u1);
 
     if (tid == 0) {
-        pass_coefficients(A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             mbar_init(&s_full[s], 1);
@@ -103,6 +102,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
         }
     } else {
         constexpr int CP = CH / 2;  // pairs of sites (k = 2 i, 2 i + 1)
+        consumer_coefficients(tid, CT, A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);
         const T cd = (T)s_coef[0];
         const Two<T> cd2 = both(cd), ncd2 = both(-cd), six = both((T)-6);
         const bool do_drift = (A.flags & P_DRIFT) != 0;

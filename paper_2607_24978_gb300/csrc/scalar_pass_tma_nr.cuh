@@ -35,7 +35,6 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_nr(const ScalarPassA
     block_units(N, A.nby, A.DZ, u0, u1);
 
     if (tid == 0) {
-        pass_coefficients(A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             mbar_init(&s_full[s], 1);
@@ -90,6 +89,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_nr(const ScalarPassA
         }
     } else {
         // ---------------------------------------------------------------- consumer warps
+        consumer_coefficients(tid, CT, A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);
         const T cd = (T)s_coef[0], cL = (T)s_coef[1], cV = (T)s_coef[2];
         const T ce = (T)A.e, ck = (T)A.k;
         const bool do_drift = (A.flags & P_DRIFT) != 0;

@@ -495,15 +495,6 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     constexpr bool track = TRACK;
     const bool expand = (A.flags & P_EXPANSION) != 0;
     if (tid == 0) {
-        const double a = A.scal->a, b = expand ? A.scal->b : 0.0;
-        s_coef[0] = apow(a, A.alpha - 3.0);                 // phi' = c0 pi
-        s_coef[1] = apow(a, 1.0 + A.alpha) / (A.dx * A.dx);  // Laplacian
-        s_coef[2] = apow(a, 3.0 + A.alpha);                 // potential
-        s_coef[3] = apow(a, A.alpha - 1.0);                 // E' prefactor
-        s_coef[4] = (1.0 - A.alpha) * b / a;               // electric friction
-        s_coef[5] = a;
-        s_coef[6] = apow(a, 1.0 - A.alpha);                 // a^(1-alpha) E in the Gauss charge
-        s_coef[7] = LF && A.lf == 3 ? u1_lf_drift(a, b, A.h, A.alpha) : 0.0;  // leapfrog drift of phi
         s_src[SG_PHI] = A.phi_in;
         s_src[SG_PI] = A.pi_in;
 #pragma unroll
@@ -531,6 +522,21 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     if (warp >= G::CW) {
         ring.produce(tid - 32 * G::CW, s_src, t);
     } else if (warp < t.warps()) {
+        // the prefactors, lanes side by side, beside the copies of the first planes
+        if (tid < 5) {
+            const double a = A.scal->a, b = expand ? A.scal->b : 0.0;
+            const double e = tid == 0 ? A.alpha - 3.0 : tid == 1 ? 1.0 + A.alpha : tid == 2 ? 3.0 + A.alpha
+                             : tid == 3 ? A.alpha - 1.0 : 1.0 - A.alpha;
+            double p = apow(a, e);
+            // phi' = c0 pi; Laplacian (c1); potential (c2); E' prefactor (c3); a^(1-alpha) E in the
+            // Gauss charge (c6); electric friction (c4)
+            if (tid == 1) p = p / (A.dx * A.dx);
+            s_coef[tid == 4 ? 6 : tid] = p;
+            if (tid == 2) s_coef[4] = (1.0 - A.alpha) * b / a;
+            if (tid == 3) s_coef[7] = LF && A.lf == 3 ? u1_lf_drift(a, b, A.h, A.alpha) : 0.0;  // leapfrog drift of phi
+            if (tid == 0) s_coef[5] = a;
+        }
+        named_barrier_sync(3, 32 * t.warps());
         const T c_dphi = (T)s_coef[0], cL = (T)s_coef[1], cV = (T)s_coef[2], cE = (T)s_coef[3], cfr = (T)s_coef[4];
         const T ca = (T)s_coef[6];
         const T g = (T)A.g, ws2 = (T)A.ws2, dx = (T)A.dx, m2 = (T)A.m2, lam = (T)A.lam;

@@ -337,7 +337,8 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * the same z chunks so that one wave of blocks covers the lattice; -1 = a persistent grid
  * of one wave, each block a balanced contiguous range of planes; for the axion-U(1)
  * kernels, the planes of the z chunk each (x, y) tile marches through, half as many in the staged
- * plaquette launches, whose tiles are twice as tall).  CL_OPT_STAGES: TMA stage buffers
+ * plaquette launches, whose tiles have twice the sites; ensembles: planes per work item, 0 = the
+ * members' columns cut into blocks of equal work).  CL_OPT_STAGES: TMA stage buffers
  * of the fused pass, 2..6, or -1 for the loader without TMA staging (0 = library choice;
  * FP32 rows that are not a multiple of 16 bytes run their own staged kernel with 3 or 4
  * buffers, reported as variant 0, unless variant 0 or stages -1 is asked for; FP64 ones always

@@ -659,8 +659,8 @@ cl_status choose_tiles(cl_lattice* l)
         // the fused stage only on request: measured slower than the two launches at 192^3
         // (3.96 against 5.12 Gsite-updates/s; both latency-bound)
         l->u1_fused = l->opt_variant == 1 && u1_fused_ok(N) && !is_u1_lf(l);
-        // the staged launches (neighbourhoods in shared memory) are the library's choice
-        // where the tiles divide N
+        // the staged launches (neighbourhoods in shared memory) are the library's choice where
+        // rows are whole 16-byte units, from the size on where they pay (u1_staged_pays)
         l->u1_staged = u1_staged_ok(prec, N) && (l->opt_variant == 2 || (l->opt_variant == 3 && N % 32 == 0) ||
                                                  (l->opt_variant == -1 && u1_staged_pays(N)));
         l->u1_sfused = l->u1_staged && l->opt_variant == 3;

@@ -570,7 +570,8 @@ cl_status choose_tiles(cl_lattice* l)
         if (!l->ps_barrier && cudaMalloc(&l->ps_barrier, 256) != cudaSuccess)
             return fail(l, CL_ENOMEM, "cannot allocate the grid barrier");
         l->ps_grid = ((N + l->ps_BY - 1) / l->ps_BY) * ((N + l->ps_BZ - 1) / l->ps_BZ);
-        if (3 * l->ps_grid > nblocks) nblocks = 3 * l->ps_grid;  // 2 (kMaxQ + 1) numbers a block
+        static_assert(3 * (kMaxQ + 1) <= 4 * kMaxQ, "three buffers of kMaxQ + 1 numbers a block");
+        if (4 * l->ps_grid > nblocks) nblocks = 4 * l->ps_grid;
     }
     l->rk_stages = 0;
     if (is_rk(l->p.integrator) && l->VW * l->es == 16 && N % l->VW == 0 && l->opt_stages != -1) {

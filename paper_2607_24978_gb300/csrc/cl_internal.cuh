@@ -153,7 +153,7 @@ struct PersistArgs {
     T* pi[2][2];
     T* c[2][2];
     DevScal* scal;
-    double* partials;   // [2][kMaxQ + 1][grid]
+    double* partials;   // [3][kMaxQ + 1][grid]
     unsigned* barrier;  // zero at the launch
     int N, BY, BZ, nby; // box of rows of a block
     int in0;            // buffer read by the first pass

@@ -104,7 +104,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
     const int by0 = (int)(blockIdx.x % A.nby) * A.BY, bz0 = (int)(blockIdx.x / A.nby) * A.BZ;
     const int ry = min(A.BY, N - by0), rz = min(A.BZ, N - bz0);
     const bool expand = (A.flags & P_EXPANSION) != 0;
-    // partials of a pass: the blocks' a'' terms, then their five sums (written when needed)
+    // partials of a pass: the blocks' a'' terms, then their five sums (written when needed), in
+    // three buffers in turn.  Block 0's scalar warp reads the sums of pass p (with a Hubble limit)
+    // after it has let its own block go on; the blocks that write that buffer again, for pass
+    // p + 3, have passed grid barrier p + 2, where block 0 arrives after its scalar warp has
+    // worked out the factors that follow pass p + 1, hence after those reads.  (With two buffers
+    // they would need barrier p + 1 only, where block 0 arrives without that warp.)
     double* const part0 = A.partials;
     const size_t part_stride = (size_t)G * (kMaxQ + 1);
 
@@ -126,7 +131,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
             if (expand) beta *= a * spow(a, e2a);
             const bool full = p + 1 == A.passes || A.hubble_limit > 0.0;
             bar_sync(2, 32 * (kMaxQ + 1));
-            double* part = part0 + (p & 1) * part_stride;
+            double* part = part0 + (p % 3) * part_stride;
             double w = 0.0, term;
             if constexpr (sizeof(T) == 4) {
                 const float2 v = lane < kMaxQ ? s_q[lane] : make_float2(0.f, 0.f);
@@ -189,7 +194,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
             const double dl = half * A.d[cn], ka = A.k[c];
             double r0 = 0.0;
             if (ex.n >= 0 && ex.neg) r0 = 1.0 / ipow(expand ? __fma_rn(dl, b, a1) : a1, ex.n);
-            const double* part = part0 + (p & 1) * part_stride;
+            const double* part = part0 + (p % 3) * part_stride;
             int ok = 1;
             if (lane == 0) {
                 const unsigned want = (unsigned)(p + 1) * G;

@@ -366,7 +366,7 @@ cl_status ens_tiles(cl_lattice* l)
 bool u1_staged_pays(int N) { return N % 32 == 0 || N >= 36; }
 
 // Lattices up to this many sites take their steps in the resident multi-pass kernel, whose pass
-// starts sooner (3.9 us against 16.4 at 32^3) but reads a site's neighbours through L1 and L2
+// starts sooner (4.0 us against 16.4 at 32^3) but reads a site's neighbours through L1 and L2
 // instead of staging them, and drifts them once per reader.  The lines lie where the two cross
 // (us a pass, per-pass kernel / resident).  FP32 + Kahan, one field: 24.4 / 22.1 at 128^3, 26.0 / 28.0
 // at 136^3; two fields: 31.8 / 30.2 at 120^3, 32.3 / 34.4 at 124^3; rows of other alignment, whose

@@ -19,8 +19,8 @@
 //    works.  An FP64 instruction occupies its scheduler for 64 cycles whether one lane or 32 take
 //    part (measured), so independent scalars sit in different lanes and warps;
 //  * block 0 keeps the status and, for the last pass (and a Hubble limit), the energies.
-// Measured (us a pass, one launch a pass before): 16.4 -> 3.9 at 32^3 one field FP32 + Kahan, 21.9 ->
-// 7.9 at 64^3 two fields, 22.5 -> 11.4 at 96^3 one field; FP64 22.5 -> 6.2 at 32^3.  Of the 3.9, about
+// Measured (us a pass, one launch a pass before): 16.4 -> 4.0 at 32^3 one field FP32 + Kahan, 21.9 ->
+// 7.9 at 64^3 two fields, 22.5 -> 11.4 at 96^3 one field; FP64 22.5 -> 6.2 at 32^3.  Of the 4.0, about
 // 1.0 is the barrier (release, arrival, poll), 1.0 FP64 instructions of the scalar warp.
 // Waits are bounded: a barrier that does not complete within two seconds sets ST_TIMEOUT and
 // every block leaves.
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
 {
     using Pair = typename std::conditional<sizeof(T) == 4, float2, double>::type;
     __shared__ Pair s_acc[kMaxQ][kCT];
-    __shared__ Pair s_q[8];      // the block's sums
+    __shared__ double s_q[8];    // the block's sums
     __shared__ double s_a;       // the pass's a
     __shared__ T s_coef[4];      // drift and kick prefactors
     __shared__ int s_stop;
@@ -132,16 +132,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
             const bool full = p + 1 == A.passes || A.hubble_limit > 0.0;
             bar_sync(2, 32 * (kMaxQ + 1));
             double* part = part0 + (p % 3) * part_stride;
-            double w = 0.0, term;
-            if constexpr (sizeof(T) == 4) {
-                const float2 v = lane < kMaxQ ? s_q[lane] : make_float2(0.f, 0.f);
-                const double hi = (double)v.x, lo = (double)v.y;
-                term = __fma_rn(beta, lo, beta * hi);
-                if (full) w = hi + lo;
-            } else {
-                w = lane < kMaxQ ? s_q[lane] : 0.0;
-                term = beta * w;
-            }
+            const double w = lane < kMaxQ ? s_q[lane] : 0.0;
+            double term = beta * w;
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) term += __shfl_xor_sync(0xffffffffu, term, off);
             if (full && lane < kMaxQ) __stcg(&part[(size_t)(lane + 1) * G + blockIdx.x], w);
@@ -367,8 +359,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
             }
             advance(spot);
         }
-        // block sums: warp q adds quantity q over the threads (compensated FP32 sums as float
-        // pairs, converted once; FP64 as it is)
+        // block sums: warp q adds quantity q over the threads -- compensated FP32 sums as float
+        // pairs over each warp's lanes, then in FP64 over the warps, as the other passes do; FP64
+        // as it is
         const Acc<T>* const acc[kMaxQ] = {&accK[0], NF > 1 ? &accK[NF - 1] : nullptr, &accG[0],
                                           NF > 1 ? &accG[NF - 1] : nullptr, &accV};
 #pragma unroll
@@ -378,7 +371,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
         }
         bar_sync(1, kCT);
         if (warp < kMaxQ) {
-            const int nw = min(kNW, (ry * rz * N + 31) / 32);  // warps with sites
             if constexpr (sizeof(T) == 4) {
                 F2 x[kNW];
 #pragma unroll
@@ -386,16 +378,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_scalar_persist(const PersistArg
                     const float2 o = s_acc[warp][32 * i + lane];
                     x[i] = F2{o.x, o.y};
                 }
-#pragma unroll
-                for (int h = kNW / 2; h > 0; h /= 2)
-#pragma unroll
-                    for (int i = 0; i < h; ++i) x[i] = f2_add(x[i], x[i + h]);
-                for (int off = 16; off > 0; off >>= 1)
-                    x[0] = f2_add(x[0], F2{__shfl_xor_sync(0xffffffffu, x[0].hi, off), __shfl_xor_sync(0xffffffffu, x[0].lo, off)});
-                if (lane == 0) s_q[warp] = make_float2(x[0].hi, x[0].lo);
+                // a pair of lanes holds a warp's sum: one takes the high part, the other the low
+                const F2 w = warp_sums<kNW>(x, lane);
+                double d = (double)(lane & 1 ? w.lo : w.hi);
+                for (int off = 1; off < 32; off *= 2) d += __shfl_xor_sync(0xffffffffu, d, off);
+                if (lane == 0) s_q[warp] = d;
             } else {
                 double x = 0.0;
                 if (NF == 2 || (warp != 1 && warp != 3)) {
+                    const int nw = min(kNW, (ry * rz * N + 31) / 32);  // warps with sites
                     for (int i = 0; i < nw; ++i) x += s_acc[warp][32 * i + lane];
                     for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
                 }

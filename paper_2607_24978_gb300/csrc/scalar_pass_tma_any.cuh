@@ -18,9 +18,11 @@
 //
 // The arithmetic runs on pairs of sites (Two<T>): the kernel is bound by issue and the latency
 // behind it (14 consumer warps an SM, 56 % of the issue slots at 251^3, two fields), and packed
-// instructions take half the slots of the scalar ones: 213 -> 177 us a pass.  Copying every row
-// with scalar loads through the direct loader took 619 us there (363 -> 91 with one field; 125^3
-// two fields 94 -> 39; 250^3, 8-byte vectors, 263 -> 176); HBM alone would need 113 us.
+// instructions take half the slots of the scalar ones: 213 -> 174 us a pass.  The energy sums stay
+// scalar, every site added to the thread's compensated sum by itself: pairs of sums take twice the
+// registers of the sums and spill (227 us with them; sums of the two fields in pairs 192).  Copying every row
+// with scalar loads through the direct loader took 619 us there (363 -> 92 with one field; 125^3
+// two fields 94 -> 36; 250^3, 8-byte vectors, 263 -> 174); HBM alone would need 113 us.
 template <typename T, int NF, bool KAHAN, int CH, int S>
 __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPassArgs<T> A)
 {
@@ -194,7 +196,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                 }
                 if (j >= 2) {
                     const T* sp = stage + st_prev * stage_stride;
-                    Two<T> lap[NF][CP], ks[NF], vs = both((T)0);
+                    Two<T> lap[NF][CP];
 #pragma unroll
                     for (int f = 0; f < NF; ++f) {
                         const T* sa = sp + f * KPF * arr_stride;
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
 #pragma unroll
                             for (int i = 0; i < CP; ++i) y2[i] = Two<T>(y[2 * i], y[2 * i + 1]);
                         };
-                        Two<T> ysum[CP], g = both((T)0);
+                        Two<T> ysum[CP];
                         if (warp_lo) load_halo(lo_row, own - N, sh_prev[0] + first);
                         else load_row(sa + own - N);
 #pragma unroll
@@ -259,11 +261,9 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                             lap[f][i] = fma2(six, c, add2(add2(add2(xp, xm), ysum[i]), add2(znew[f][i], zlo[f][i])));
                             const Two<T> gx = sub2(xp, c), gz = sub2(znew[f][i], c);
                             gs[i] = fma2(gx, gx, fma2(gz, gz, gs[i]));
-                            g = add2(g, Two<T>(valid >> (2 * i) & 1u ? gs[i].lo() : (T)0,
-                                               valid >> (2 * i + 1) & 1u ? gs[i].hi() : (T)0));
+                            accG[f].add(valid >> (2 * i) & 1u ? gs[i].lo() : (T)0);
+                            accG[f].add(valid >> (2 * i + 1) & 1u ? gs[i].hi() : (T)0);
                         }
-                        accG[f].add(g.lo() + g.hi());
-                        ks[f] = both((T)0);
                     }
                     const size_t base = (size_t)(z0 + j - 2) * plane + row_off + first;
 #pragma unroll
@@ -282,13 +282,12 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                         for (int f = 0; f < NF; ++f) {
                             if (va) A.pi_out[f][base + 64 * i] = q[f].lo();
                             if (vb) A.pi_out[f][base + 64 * i + 32] = q[f].hi();
-                            ks[f] = add2(ks[f], Two<T>(va ? k1[f].lo() : (T)0, vb ? k1[f].hi() : (T)0));
+                            accK[f].add(va ? k1[f].lo() : (T)0);
+                            accK[f].add(vb ? k1[f].hi() : (T)0);
                         }
-                        vs = add2(vs, Two<T>(va ? v1.lo() : (T)0, vb ? v1.hi() : (T)0));
+                        accV.add(va ? v1.lo() : (T)0);
+                        accV.add(vb ? v1.hi() : (T)0);
                     }
-#pragma unroll
-                    for (int f = 0; f < NF; ++f) accK[f].add(ks[f].lo() + ks[f].hi());
-                    accV.add(vs.lo() + vs.hi());
                 }
                 if (j >= 1) release(st_prev);
 #pragma unroll

@@ -41,3 +41,15 @@ def test_resident_launches_add_warps_in_fp64(cl, prec):
     (a pair of floats holds 2^26 and 1 and loses the rest)."""
     K0 = kinetic(cl, 32, prec, {(0, 0, 0): 2.0**13, (0, 1, 0): 1.0, (0, 2, 0): 2.0**-13})
     assert K0 == (2.0**26 + 1.0 + 2.0**-26) / 2.0**16
+
+
+# sites of one thread: 0, 32, 64 and 96 along the tile's rows (N = 33: x = 0 and 32 of row 0, 31 of
+# row 1, 30 of row 2)
+@pytest.mark.parametrize("small", [(0, 0, 32), (0, 1, 31), (0, 2, 30)])
+@pytest.mark.parametrize("prec", [1, 2])
+def test_rows_of_any_alignment_add_every_site_compensated(cl, prec, small):
+    """1 + 2^-26 needs 27 bits, more than FP32 has: lost (1.5e-8 relative) where two sites are added
+    before the compensated sum, kept to 1e-14 where each is added to it."""
+    N = 33
+    K0 = kinetic(cl, N, prec, {(0, 0, 0): 1.0, small: 2.0**-13}, ((cl.CL_OPT_STAGES, 4),))
+    assert K0 == pytest.approx((1.0 + 2.0**-26) / (2.0 * N**3), rel=1e-12, abs=0.0)

@@ -310,23 +310,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_u1_stage(const 
     }
 }
 
-// A thread's sum of squares: FP32 values as float pairs of the exact square, FP64 as they are.
-template <typename T> struct GaussSum;
-template <> struct GaussSum<float> {
-    F2 s{0.f, 0.f};
-    __device__ __forceinline__ void add(float x)
-    {
-        const float q = __fmul_rn(x, x);
-        s = f2_add(s, F2{q, __fmaf_rn(x, x, -q)});
-    }
-    __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
-};
-template <> struct GaussSum<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double x) { s = fma(x, x, s); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-
 // Lattice Gauss charge G(n) = sum_i [P_i(n) - P_i(n - i)] / dx, P = a^(1-alpha) E + g W.
 // mode 0 writes diag[D_GV] = max_n |G(n)| / max_n sum_i (|P_i(n)| + |P_i(n - i)|) / dx;
 // mode 1 (per-step tracking, for the launch forms whose stage does not sum it itself) the
@@ -338,19 +321,20 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
     __shared__ int s_last;
     const uint32_t N = (uint32_t)A.N;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    // per-site arithmetic and maxima in the field precision, FP32 sums of exact squares (square
-    // plus its rounding error) as float pairs: the two FP64 divisions, conversions and additions
-    // a site took before made 440 us at 192^3 and 92 us at 100^3 of this launch on GB300's FP64 pipe
+    // per-site arithmetic and maxima in the field precision (two FP64 divisions, conversions and
+    // additions a site made 440 us at 192^3 and 92 us at 100^3 of this launch on GB300's FP64 pipe);
+    // the squares and sums of mode 1 in FP64: G is what cancellation leaves of E, and its FP32
+    // square vanishes where that of E does not
     const T ca = (T)apow(A.scal->a, 1.0 - A.alpha);
     const T b4 = (T)(0.25 / (A.dx * A.dx)), gh = (T)(0.5 * A.g);
     T gmx = (T)0, smx = (T)0;
-    GaussSum<T> gsq_s, e2_s;
+    double gsq = 0.0, e2 = 0.0;
     const U1Tile tile(N, (uint32_t)A.dz);
     for (uint32_t z = tile.z0; z < tile.z1; ++z) {
         if (!tile.active) break;
         const uint32_t n = (z * N + tile.y) * N + tile.x;
         const Nbhd s(tile.x, tile.y, z, N);
-        T G = (T)0, sc = (T)0;
+        T G = (T)0, sc = (T)0, ee = (T)0;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const Off op(i, 1), om(i, -1);
@@ -362,13 +346,15 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
             const T Pm = ca * A.E_in[i][nm] + gh * (A.phi_in[nm] * Bm + A.phi_in[n] * Bn);
             G += Pn - Pm;
             sc += fabs(Pn) + fabs(Pm);
-            if (mode == 1) e2_s.add(A.E_in[i][n]);
+            ee += A.E_in[i][n] * A.E_in[i][n];
         }
         gmx = fmax(gmx, fabs(G));
         smx = fmax(smx, sc);
-        if (mode == 1) gsq_s.add(G);
+        if (mode == 1) {
+            gsq = fma((double)G, (double)G, gsq);
+            e2 += (double)ee;
+        }
     }
-    const double gsq = gsq_s.value(), e2 = e2_s.value();
     if (mode == 1) {  // sums in a fixed order, then the last block stores the tracked value
         double v[2] = {gsq, e2};
         block_reduce<2>(v, s_red, tid, nthr);

@@ -509,6 +509,10 @@ __global__ void __launch_bounds__(U1PGeom<T>::NT, 1) k_u1s_plaquette_rates(const
 // W32: tiles of 32 columns, the staged rows' length and a thread's row constants (the kernel is at
 // its register limit: with variable ones the stages at 192^3 take 201 and 241 us instead of 198
 // and 231, the plaquettes 105 instead of 101).
+// The tracked squares of the Gauss charge are summed in FP64 except in the W32 instance, which takes
+// that launch only where 32 divides N: the gather launches that the staged ones replaced on other
+// sizes sum them so, and what cancellation leaves of E has squares below FP32's range first (FP64
+// for all sizes costs 1 to 2% of a step at 192^3).
 template <typename T, bool TRACK, bool LF, bool W32>
 __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T> A)
 {
@@ -525,7 +529,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     const bool first = !LF && (A.flags & P_FIRST_STAGE) != 0;
     const int lf = LF ? A.lf : 0;
     const bool update = (A.flags & P_ENERGY_ONLY) == 0;
-    constexpr bool track = TRACK;
+    constexpr bool track = TRACK, GSQ64 = TRACK && !W32;
     const bool expand = (A.flags & P_EXPANSION) != 0;
     if (tid == 0) {
         s_src[SG_PHI] = A.phi_in;
@@ -553,6 +557,7 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     const U1SRing<G, NA> ring{ring_sm, table, s_full, s_empty, &s_fail};
     const uint32_t N = t.N, V = N * N * N;
     Acc<T> accK, accG, accV, accKE, accGs;
+    double gsq = 0.0;
     if (warp >= G::CW) {
         ring.produce(tid - 32 * G::CW, s_src, t);
     } else if (warp < t.warps()) {
@@ -689,7 +694,10 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
                         gd += ca * (ec[i] - em[i]) +
                               (T)0.5 * g * (S(SG_PHI, U1S_E(i, 1)) * Bpi - S(SG_PHI, U1S_E(i, -1)) * Bmi);
                     }
-                    if (has) accGs.add(gd * gd);
+                    if (has) {
+                        if constexpr (GSQ64) gsq = fma((double)gd, (double)gd, gsq);
+                        else accGs.add(gd * gd);
+                    }
                 }
                 // link forces
                 T F_E[3];
@@ -770,8 +778,13 @@ __global__ void __launch_bounds__(U1SGeom<T>::NT, 1) k_u1s_stage(const U1Args<T>
     // slot 4 of the stage's partials carries the Gauss sum (the magnetic energy's partials
     // follow in the plaquette launch's region)
     double v[kMaxQ];
-    const Acc<T>* av[kMaxQ] = {&accK, &accG, &accV, &accKE, &accGs};
+    const Acc<T>* av[kMaxQ] = {&accK, &accG, &accV, &accKE, GSQ64 ? nullptr : &accGs};
     block_reduce_acc<T, kMaxQ>(av, v, s_red, tid, G::NT);
+    if constexpr (GSQ64) {
+        double g1[1] = {gsq};
+        block_reduce<1>(g1, s_red, tid, G::NT);
+        v[kMaxQ - 1] = g1[0];
+    }
     if (tid == 0) {
         if (s_fail) atomicOr(&A.scal->status, ST_TIMEOUT);
 #pragma unroll
@@ -1308,16 +1321,17 @@ static cudaError_t launch_u1s_t(const U1Args<T>& A, int what, cudaStream_t s)
         // forms: 1 a Runge-Kutta stage, 2 the first stage of a step (Gauss tracking), 3 a
         // leapfrog pass, 4 the leapfrog's second pass (Gauss tracking)
         const int form = A.lf ? (A.lf == 2 ? 4 : 3) : ((A.flags & P_FIRST_STAGE) && !(A.flags & P_ENERGY_ONLY) ? 2 : 1);
-        const auto kernel = A.tx == G::TX ? (form == 4   ? k_u1s_stage<T, true, true, true>
-                                             : form == 3 ? k_u1s_stage<T, false, true, true>
-                                             : form == 2 ? k_u1s_stage<T, true, false, true>
-                                                         : k_u1s_stage<T, false, false, true>)
-                                          : (form == 4   ? k_u1s_stage<T, true, true, false>
-                                             : form == 3 ? k_u1s_stage<T, false, true, false>
-                                             : form == 2 ? k_u1s_stage<T, true, false, false>
-                                                         : k_u1s_stage<T, false, false, false>);
+        const bool w32 = A.tx == G::TX && (A.N % 32 == 0 || form == 1 || form == 3);
+        const auto kernel = w32 ? (form == 4   ? k_u1s_stage<T, true, true, true>
+                                   : form == 3 ? k_u1s_stage<T, false, true, true>
+                                   : form == 2 ? k_u1s_stage<T, true, false, true>
+                                               : k_u1s_stage<T, false, false, true>)
+                                : (form == 4   ? k_u1s_stage<T, true, true, false>
+                                   : form == 3 ? k_u1s_stage<T, false, true, false>
+                                   : form == 2 ? k_u1s_stage<T, true, false, false>
+                                               : k_u1s_stage<T, false, false, false>);
         static DevFlag sattr[2][5];
-        DevFlag& done = sattr[A.tx == G::TX ? 1 : 0][form];
+        DevFlag& done = sattr[w32 ? 1 : 0][form];
         if (!done) {
             const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;

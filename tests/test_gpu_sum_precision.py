@@ -53,3 +53,27 @@ def test_rows_of_any_alignment_add_every_site_compensated(cl, prec, small):
     N = 33
     K0 = kinetic(cl, N, prec, {(0, 0, 0): 1.0, small: 2.0**-13}, ((cl.CL_OPT_STAGES, 4),))
     assert K0 == pytest.approx((1.0 + 2.0**-26) / (2.0 * N**3), rel=1e-12, abs=0.0)
+
+
+# the gather launches, and the staged ones on a size that is no multiple of their 32-column tiles
+@pytest.mark.parametrize("N", [16, 36])
+@pytest.mark.parametrize("integ", ["CL_INT_RK3_3", "CL_INT_VV2"])
+def test_gauss_tracking_of_weak_fields(cl, N, integ):
+    """E = 2^-60 but for one link, a unit in the last place (2^-83) larger: the charge is 2^-83 on two
+    sites, its square 2^-166 below FP32's range, E^2 = 2^-120 within it."""
+    E = np.full((N, N, N), 2.0**-60, np.float32)
+    E[3, 5, 7] = np.float32(2.0**-60 * (1.0 + 2.0**-23))
+    zero = np.zeros_like(E)
+    with cl.Lattice(N, 1.0 * N, 1, cl.CL_PREC_FP32, getattr(cl, integ), gauge=cl.CL_GAUGE_U1_AXION, expansion=False,
+                    alpha=1.0, dt=1e-6) as g:
+        g.cl_set_potential(cl.CL_POT_LPHI4, [1.0])
+        g.cl_set_gauge_coupling(1.0, 1.0)
+        for f in (cl.CL_FIELD_PHI0, cl.CL_FIELD_PI0):
+            g.cl_set_state(f, zero)
+        for i in range(3):
+            g.cl_set_state(cl.CL_FIELD_THETA1 + i, zero)
+            g.cl_set_state(cl.CL_FIELD_E1 + i, E if i == 0 else zero)
+        g.cl_set_scalars(1.0)
+        g.cl_step(1)
+        r = g.cl_energies()["gauss_rms_step"]
+    assert r == pytest.approx(2.0**0.5 * 2.0**-23 / N**1.5, rel=1e-6, abs=0.0)

@@ -234,6 +234,10 @@ cl_status cl_energies(cl_lattice* l, cl_energy* out, int32_t count);
  * normalisation):  type 1: Delta = n_l S_l / (N^6 dn);  type 2: Delta = 4 pi n_l^3 (S_l/#_l) / N^6.
  * k_out[l] = (2 pi / L) n_l, count_out[l] = #_l (number of modes), delta_out[0] = 0.
  * Writes min(cap, bins) host values and sets *nbins to the number of bins of the lattice.
+ * Between calls (this one, cl_gauge_spectrum, cl_gw_spectrum) the handle keeps up to 512 MB of
+ * device memory in all, scratch and transform plans with their work areas; what needs more is
+ * allocated and released by the call.  cl_free gives it back, and so does any later call on the
+ * handle whose allocations would otherwise fail.
  * Uses cuFFT; synchronising.  Errors: CL_EINVAL, CL_ECUDA, CL_ENOMEM. */
 cl_status cl_spectrum(cl_lattice* l, int32_t member, int32_t field, double dn, int32_t type,
                       double* k_out, double* delta_out, double* count_out, int32_t cap, int32_t* nbins);

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "cl_internal.cuh"
+#include "kept_scratch.cuh"
 #include "surrogate_train.cuh"
 #include "rk_tma.cuh"
 #include "u1_staged.cuh"
@@ -44,6 +45,29 @@ bool is_rk(int integrator)
 {
     return integrator == CL_INT_RK3_3 || integrator == CL_INT_RK4_5 || integrator == CL_INT_RK3_4;
 }
+
+// Scratch and D2Z plans of the spectra (see KeptScratch).  A measurement every few steps paid three
+// cudaMalloc / cudaFree pairs and a plan each time (1.0 of 3.4 ms at 256^3, whose scratch is 270 MB).
+// What takes more than kSpecKeep bytes, long against that, is allocated and released by its call.
+struct SpecApi {
+    using Plan = cufftHandle;
+    static bool alloc(void** p, size_t bytes)
+    {
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+        cudaGetLastError();  // not the next launch's error
+        *p = nullptr;
+        return false;
+    }
+    static void free(void* p) { cudaFree(p); }
+    static bool plan(int N, Plan* plan, size_t* work)
+    {
+        if (cufftPlan3d(plan, N, N, N, CUFFT_D2Z) != CUFFT_SUCCESS) return false;
+        if (cufftGetSize(*plan, work) != CUFFT_SUCCESS) *work = (size_t)-1 / 2;  // not kept
+        return true;
+    }
+    static void destroy(Plan plan) { cufftDestroy(plan); }
+};
+constexpr size_t kSpecKeep = (size_t)512 << 20;
 
 }  // namespace
 
@@ -124,9 +148,7 @@ struct cl_lattice {
     int nitems = 0, ens_grid = 0, ens_stages = 0, ens_stage_stride = 0, ens_ring_slot = 0, ens_variant = 0;
     float* sg_buf = nullptr;        // surrogate jumps: packed input (3 V), output (2 V), snapshot (3 V)
     size_t ens_smem = 0;
-    void* sp_mem = nullptr;         // spectra: scratch kept between calls (see spec_acquire)
-    size_t sp_bytes = 0;
-    std::vector<std::pair<int, cufftHandle>> sp_plans;  // D2Z plans by lattice size
+    KeptScratch<SpecApi> spec{kSpecKeep};
     char err[512] = {0};
 };
 
@@ -177,12 +199,19 @@ void invalidate_graphs(cl_lattice* l)
 
 cl_status query_blocks_per_sm(cl_lattice* l, int* per_sm);
 
+// Device memory for a handle in use: what it keeps for its spectra gives way.
+template <typename P>
+bool dev_alloc(cl_lattice* l, P** p, size_t bytes)
+{
+    return l->spec.retry([&] { return SpecApi::alloc((void**)p, bytes); });
+}
+
 cl_status grow_partials(cl_lattice* l, int nblocks)
 {
     if (nblocks > l->partials_cap) {
         if (l->partials) cudaFree(l->partials);
         l->partials = nullptr;
-        if (cudaMalloc(&l->partials, sizeof(double) * kMaxQ * (size_t)nblocks) != cudaSuccess)
+        if (!dev_alloc(l, &l->partials, sizeof(double) * kMaxQ * (size_t)nblocks))
             return fail(l, CL_ENOMEM, "cannot allocate %d reduction partials", nblocks);
         l->partials_cap = nblocks;
     }
@@ -346,12 +375,12 @@ cl_status ens_tiles(cl_lattice* l)
     l->d_items = nullptr;
     if (l->d_first) cudaFree(l->d_first);
     l->d_first = nullptr;
-    if (!l->d_members && cudaMalloc(&l->d_members, sizeof(EnsMember) * B) != cudaSuccess)
+    if (!l->d_members && !dev_alloc(l, &l->d_members, sizeof(EnsMember) * B))
         return fail(l, CL_ENOMEM, "cannot allocate the member table");
-    if (cudaMalloc(&l->d_items, sizeof(EnsItem) * l->hitems.size()) != cudaSuccess)
+    if (!dev_alloc(l, &l->d_items, sizeof(EnsItem) * l->hitems.size()))
         return fail(l, CL_ENOMEM, "cannot allocate the item table");
     CUDA_TRY(l, cudaMemcpy(l->d_items, l->hitems.data(), sizeof(EnsItem) * l->hitems.size(), cudaMemcpyHostToDevice));
-    if (cudaMalloc(&l->d_first, sizeof(int) * first.size()) != cudaSuccess)
+    if (!dev_alloc(l, &l->d_first, sizeof(int) * first.size()))
         return fail(l, CL_ENOMEM, "cannot allocate the item schedule");
     CUDA_TRY(l, cudaMemcpy(l->d_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
     cl_status s = upload_members(l);
@@ -567,7 +596,7 @@ cl_status choose_tiles(cl_lattice* l)
     if (!is_rk(l->p.integrator) && !l->gauge && !l->gw && !l->user_tiles && l->V <= persist_max_sites(l) &&
         persist_tiles(prec, N, nsm, &l->ps_BY, &l->ps_BZ)) {
         // small lattices: cl_step runs its passes in the resident kernel
-        if (!l->ps_barrier && cudaMalloc(&l->ps_barrier, 256) != cudaSuccess)
+        if (!l->ps_barrier && !dev_alloc(l, &l->ps_barrier, 256))
             return fail(l, CL_ENOMEM, "cannot allocate the grid barrier");
         l->ps_grid = ((N + l->ps_BY - 1) / l->ps_BY) * ((N + l->ps_BZ - 1) / l->ps_BZ);
         static_assert(3 * (kMaxQ + 1) <= 4 * kMaxQ, "three buffers of kMaxQ + 1 numbers a block");
@@ -1426,72 +1455,29 @@ namespace {
 
 // Scratch and plan of one spectrum call.
 struct SpecWork {
+    KeptScratch<SpecApi>::Use use;
     double* real = nullptr;  // transform input
     double2* F = nullptr;    // half spectra
     double* bins = nullptr;  // S[nb], C[nb], k[nb], delta[nb]
     int* table = nullptr;    // bin of every squared mode number
-    cufftHandle plan = 0;
-    void* temp = nullptr;    // scratch to free after the call
-    bool temp_plan = false;
 };
-
-// Bytes of scratch, and of a plan's work area, that a handle keeps from one spectrum call to the
-// next: a measurement every few steps paid three cudaMalloc / cudaFree pairs and a plan each time
-// (1.0 of 3.4 ms at 256^3, whose scratch is 270 MB).  Larger calls, long against that, allocate
-// and release their own, as all did, so that a lattice that fills the device leaves it the room.
-constexpr size_t kSpecKeep = (size_t)512 << 20;
-constexpr size_t kSpecPlans = 8;  // an ensemble's sizes
 
 cl_status spec_acquire(cl_lattice* l, int N, size_t nreal, size_t nF, int nb, SpecWork* w)
 {
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t b_real = up(nreal * sizeof(double)), b_F = up(nF * sizeof(double2)), b_bins = up(4 * (size_t)nb * sizeof(double));
-    const size_t bytes = b_real + b_F + b_bins + up(spectrum_table_bytes(N));
-    char* base = nullptr;
-    if (bytes <= kSpecKeep) {
-        if (l->sp_bytes < bytes) {
-            if (l->sp_mem) cudaFree(l->sp_mem);
-            l->sp_mem = nullptr;
-            l->sp_bytes = 0;
-            if (cudaMalloc(&l->sp_mem, bytes) != cudaSuccess) {
-                l->sp_mem = nullptr;
-                return fail(l, CL_ENOMEM, "spectrum scratch allocation failed");
-            }
-            l->sp_bytes = bytes;
-        }
-        base = (char*)l->sp_mem;
-    } else {
-        if (cudaMalloc(&w->temp, bytes) != cudaSuccess) {
-            w->temp = nullptr;
-            return fail(l, CL_ENOMEM, "spectrum scratch allocation failed");
-        }
-        base = (char*)w->temp;
+    switch (l->spec.acquire(N, b_real + b_F + b_bins + up(spectrum_table_bytes(N)), &w->use)) {
+    case KeptScratch<SpecApi>::NO_MEMORY: return fail(l, CL_ENOMEM, "spectrum scratch allocation failed");
+    case KeptScratch<SpecApi>::NO_PLAN: return fail(l, CL_ECUDA, "cufftPlan3d failed");
+    default: break;
     }
+    char* base = (char*)w->use.mem;
     w->real = (double*)base;
     w->F = (double2*)(base + b_real);
     w->bins = (double*)(base + b_real + b_F);
     w->table = (int*)(base + b_real + b_F + b_bins);
-    for (const auto& pp : l->sp_plans)
-        if (pp.first == N) w->plan = pp.second;
-    if (!w->plan) {
-        if (cufftPlan3d(&w->plan, N, N, N, CUFFT_D2Z) != CUFFT_SUCCESS) {
-            w->plan = 0;
-            return fail(l, CL_ECUDA, "cufftPlan3d failed");
-        }
-        size_t ws = 0;
-        if (l->sp_plans.size() < kSpecPlans && cufftGetSize(w->plan, &ws) == CUFFT_SUCCESS && ws <= kSpecKeep)
-            l->sp_plans.push_back({N, w->plan});
-        else
-            w->temp_plan = true;
-    }
-    if (cufftSetStream(w->plan, l->stream) != CUFFT_SUCCESS) return fail(l, CL_ECUDA, "cufftSetStream failed");
+    if (cufftSetStream(w->use.plan, l->stream) != CUFFT_SUCCESS) return fail(l, CL_ECUDA, "cufftSetStream failed");
     return CL_OK;
-}
-
-void spec_release(SpecWork* w)
-{
-    if (w->temp_plan) cufftDestroy(w->plan);
-    if (w->temp) cudaFree(w->temp);
 }
 
 }  // namespace
@@ -1550,8 +1536,7 @@ void cl_free(cl_lattice* l)
     if (l->partials) cudaFree(l->partials);
     if (l->ps_barrier) cudaFree(l->ps_barrier);
     if (l->sg_buf) cudaFree(l->sg_buf);
-    if (l->sp_mem) cudaFree(l->sp_mem);
-    for (const auto& pp : l->sp_plans) cufftDestroy(pp.second);
+    l->spec.release();
     if (l->d_members) cudaFree(l->d_members);
     if (l->d_items) cudaFree(l->d_items);
     if (l->d_first) cudaFree(l->d_first);
@@ -1921,7 +1906,7 @@ cl_status cl_enable_gw(cl_lattice* l)
     const size_t bytes = (size_t)l->N * l->N * l->N * l->es;
     for (int c = 0; c < 5; ++c)
         for (int b = 0; b < 2; ++b) {
-            if (cudaMalloc(&l->gv[c][b], bytes) != cudaSuccess || cudaMalloc(&l->gpv[c][b], bytes) != cudaSuccess)
+            if (!dev_alloc(l, &l->gv[c][b], bytes) || !dev_alloc(l, &l->gpv[c][b], bytes))
                 return fail(l, CL_ENOMEM, "GW field allocation failed");
             CUDA_TRY(l, cudaMemsetAsync(l->gv[c][b], 0, bytes, l->stream));
             CUDA_TRY(l, cudaMemsetAsync(l->gpv[c][b], 0, bytes, l->stream));
@@ -1961,7 +1946,7 @@ cl_status cl_gw_spectrum(cl_lattice* l, double dn, int32_t type, double* k_out, 
     st = spec_acquire(l, N, (size_t)V, 5 * nh, nb, &sw);
     double *real = sw.real, *bins = sw.bins;
     double2* F = sw.F;
-    const cufftHandle plan = sw.plan;
+    const cufftHandle plan = sw.use.plan;
     for (int c = 0; c < 5 && st == CL_OK; ++c) {
         // h' = a^(alpha-3) pi_v: the factor is applied to the binned sums below
         if (launch_field_to_double(l->p.precision, l->gpv[c][buf], real, V, l->stream) != cudaSuccess)
@@ -1990,7 +1975,7 @@ cl_status cl_gw_spectrum(cl_lattice* l, double dn, int32_t type, double* k_out, 
             delta_out[i] = ca * h[3 * nb + i];
         }
     }
-    spec_release(&sw);
+    l->spec.release(sw.use);
     return st;
 }
 
@@ -2355,8 +2340,8 @@ cl_status cl_init_vacuum(cl_lattice* l, int32_t member, const cl_vacuum_params* 
     double* real = nullptr;
     std::vector<std::pair<int, cufftHandle>> plans;  // one Z2D plan per member size
     cl_status st = CL_OK;
-    if (cudaMalloc(&fk, nh_max * sizeof(double2)) != cudaSuccess || cudaMalloc(&pk, nh_max * sizeof(double2)) != cudaSuccess ||
-        cudaMalloc(&real, (size_t)nmax * nmax * nmax * sizeof(double)) != cudaSuccess) {
+    if (!dev_alloc(l, &fk, nh_max * sizeof(double2)) || !dev_alloc(l, &pk, nh_max * sizeof(double2)) ||
+        !dev_alloc(l, &real, (size_t)nmax * nmax * nmax * sizeof(double))) {
         st = fail(l, CL_ENOMEM, "vacuum scratch allocation failed");
     }
     if (st == CL_OK) st = close_leapfrog(l, true);
@@ -2377,7 +2362,7 @@ cl_status cl_init_vacuum(cl_lattice* l, int32_t member, const cl_vacuum_params* 
         for (const auto& pp : plans)
             if (pp.first == N) plan = pp.second;
         if (!plan) {
-            if (cufftPlan3d(&plan, N, N, N, CUFFT_Z2D) != CUFFT_SUCCESS) { st = fail(l, CL_ECUDA, "cufftPlan3d failed"); break; }
+            if (!l->spec.retry([&] { return cufftPlan3d(&plan, N, N, N, CUFFT_Z2D) == CUFFT_SUCCESS; })) { st = fail(l, CL_ECUDA, "cufftPlan3d failed"); break; }
             plans.push_back({N, plan});
             if (cufftSetStream(plan, l->stream) != CUFFT_SUCCESS) { st = fail(l, CL_ECUDA, "cufftSetStream failed"); break; }
         }
@@ -2461,7 +2446,7 @@ cl_status cl_spectrum(cl_lattice* l, int32_t member, int32_t field, double dn, i
     cl_status st = spec_acquire(l, N, (size_t)V, nh, nb, &w);
     double *real = w.real, *bins = w.bins;
     double2* F = w.F;
-    const cufftHandle plan = w.plan;
+    const cufftHandle plan = w.use.plan;
     if (st == CL_OK && launch_field_to_double(l->p.precision, src, real, V, l->stream) != cudaSuccess)
         st = fail(l, CL_ECUDA, "field conversion failed");
     if (st == CL_OK && cufftExecD2Z(plan, real, (cufftDoubleComplex*)F) != CUFFT_SUCCESS) st = fail(l, CL_ECUDA, "D2Z failed");
@@ -2484,7 +2469,7 @@ cl_status cl_spectrum(cl_lattice* l, int32_t member, int32_t field, double dn, i
             delta_out[i] = h[3 * nb + i];
         }
     }
-    spec_release(&w);
+    l->spec.release(w.use);
     return st;
 }
 
@@ -2506,7 +2491,7 @@ cl_status cl_gauge_spectrum(cl_lattice* l, int32_t which, double dn, int32_t typ
     cl_status st = spec_acquire(l, N, 3 * (size_t)V, 3 * nh, nb, &sw);
     double *real = sw.real, *bins = sw.bins;
     double2* F = sw.F;
-    const cufftHandle plan = sw.plan;
+    const cufftHandle plan = sw.use.plan;
     if (st == CL_OK) {
         const cudaError_t e = is_fp64(l) ? gauge_fields_t<double>(l, which, real) : gauge_fields_t<float>(l, which, real);
         if (e != cudaSuccess) st = fail(l, CL_ECUDA, "gauge field conversion failed");
@@ -2533,7 +2518,7 @@ cl_status cl_gauge_spectrum(cl_lattice* l, int32_t which, double dn, int32_t typ
             delta_out[i] = h[3 * nb + i];
         }
     }
-    spec_release(&sw);
+    l->spec.release(sw.use);
     return st;
 }
 
@@ -2603,7 +2588,7 @@ cl_status cl_surrogate_jump(cl_surrogate* s, cl_lattice* l, int32_t steps, const
     if (st != CL_OK) return st;
     const DevScal h0 = h[0];
     const size_t V = (size_t)l->V;
-    if (!l->sg_buf && cudaMalloc(&l->sg_buf, 8 * V * sizeof(float)) != cudaSuccess)
+    if (!l->sg_buf && !dev_alloc(l, &l->sg_buf, 8 * V * sizeof(float)))
         return fail(l, CL_ENOMEM, "jump: scratch allocation failed");
     float* x = l->sg_buf;
     float* y = x + 3 * V;

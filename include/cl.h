@@ -345,7 +345,7 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * members' columns cut into blocks of equal work).  CL_OPT_STAGES: TMA stage buffers
  * of the fused pass, 2..6, or -1 for the loader without TMA staging (0 = library choice;
  * FP32 rows that are not a multiple of 16 bytes run their own staged kernel with 3 or 4
- * buffers, reported as variant 0, unless variant 0 or stages -1 is asked for; FP64 ones always
+ * buffers, whatever the variant (reported as 0), unless stages -1 is asked for; FP64 ones always
  * use the loader without TMA; ensembles clamp to 2..4 with the ring kernel and 3..6 ringless).  On a Runge-Kutta scalar lattice
  * the three options tile the stage kernel instead: CL_OPT_STAGES 3..6 stage buffers of the
  * TMA-staged stage kernel (2 counts as 3; -1 = the direct-load kernel), CL_OPT_TILE_BY its
@@ -353,8 +353,8 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * same chunks, one wave of blocks; -1 = balanced persistent ranges).
  * CL_OPT_PASS_VARIANT (-1 = library choice, the default): TMA-staged pass kernel, 1 =
  * ringless (the library's choice: each warp drifts the neighbour rows it needs from the
- * stage buffers, no consumer barrier; 16-byte vectors, 2..5 stages (ensembles 3..6), FP32 rows
- * of any alignment 3 or 4, other rows fall back to 0), 0 = drifted rows shared through a ring in shared memory with one
+ * stage buffers, no consumer barrier; 16-byte vectors, 2..5 stages (ensembles 3..6), other
+ * rows fall back to 0), 0 = drifted rows shared through a ring in shared memory with one
  * consumer barrier per plane.  Both give bit-identical fields on the same tiles.  For an
  * axion-U(1) lattice, two launches per Runge-Kutta stage (plaquette fields through global
  * memory, then the stage) unless 1: 0 = every neighbour gathered from L1/L2, 2 = the
@@ -374,7 +374,8 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * A small scalar lattice (up to about 2e6 sites in FP32, 4e5 to 1e6 in FP64) takes the leapfrog
  * steps of a cl_step call in resident launches of many passes each, unless the caller set one of
  * the tiling options (the library's choices that cl_get_option reports then still serve the
- * passes outside cl_step).
+ * passes outside cl_step).  Setting an option back to its library choice, or cl_autotune, ends the
+ * caller's choice.
  * Errors: CL_EINVAL, CL_EUNSUPPORTED. */
 enum { CL_OPT_GRAPH = 0, CL_OPT_TILE_BY = 1, CL_OPT_TILE_DZ = 2, CL_OPT_STAGES = 3, CL_OPT_PASS_VARIANT = 4 };
 cl_status cl_set_option(cl_lattice* l, int32_t option, int64_t value);
@@ -388,9 +389,11 @@ cl_status cl_get_option(cl_lattice* l, int32_t option, int64_t* value);
 /* Autotuner of the fused leapfrog pass (single lattices and ensembles, no gauge field):
  * times trial passes of candidate tilings -- TMA stage buffers (CL_OPT_STAGES), rows per tile
  * (CL_OPT_TILE_BY), planes per work unit or z chunk (CL_OPT_TILE_DZ) and, for single
- * lattices, the pass kernel (CL_OPT_PASS_VARIANT) -- and keeps the fastest.  A trial pass does the full work of a pass (drift while loading, stencil kick,
- * energies) but writes into the spare buffers and commits nothing: the state, a, a' and t are
- * unchanged.  cache_path (may be NULL): a text file of earlier choices, one JSON object per
+ * lattices, the pass kernel (CL_OPT_PASS_VARIANT) -- and keeps the fastest.  A trial pass does the
+ * full work of a pass (drift while loading, stencil kick, energies) but writes into the spare
+ * buffers and commits nothing: the state, a, a' and t are unchanged.  On a small lattice, whose
+ * steps run in resident launches (see the options), those are timed too, on the state, which is
+ * put back, and are kept unless the best tiling is faster; the microseconds are then theirs.  cache_path (may be NULL): a text file of earlier choices, one JSON object per
  * line, keyed by the lattice's shape, precision and field count; a hit applies the cached
  * choice without trials, a miss appends the new one.  best (may be NULL, else 5 doubles)
  * receives the tiling then in effect (as cl_get_option reports it: stages, 0 for the loader

@@ -105,7 +105,8 @@ struct cl_lattice {
                                     //   integer-time state of the last uncommitted close
     double hubble_limit = 0.0;
     bool use_graph = true;
-    bool user_tiles = false;        // a tiling option was set by the caller (not by the autotuner)
+    unsigned user_opts = 0;         // tiling options set by the caller (1 << option; not by the autotuner)
+    bool no_resident = false;       // the autotuner measured a launch per pass to be faster
     int ps_BY = 0, ps_BZ = 0, ps_grid = 0;  // resident multi-pass kernel: box of rows, blocks (0: not used)
     unsigned* ps_barrier = nullptr;
     int opt_BY = 0, opt_DZ = 0, opt_stages = 0, opt_variant = -1;  // -1: library choice
@@ -494,7 +495,7 @@ cl_status choose_tiles(cl_lattice* l)
     int var_eff = stages > 0 ? var : 0;
     // FP32 rows that are no multiple of 16 bytes: the staged pass for rows of any alignment
     l->any_rows = false;
-    if (prec != CL_PREC_FP64 && l->VW * l->es != 16 && l->opt_stages != -1 && l->opt_variant != 0) {
+    if (prec != CL_PREC_FP64 && l->VW * l->es != 16 && l->opt_stages != -1) {
         auto fits = [&](int by, int st) {
             return by >= 1 && scalar_pass_any_threads(N, by) <= 448 &&
                    scalar_pass_smem_bytes(prec, l->nf, N, by, st, 2) <= (size_t)kPassMaxSmem;
@@ -593,7 +594,7 @@ cl_status choose_tiles(cl_lattice* l)
         l->gw_nbz = (N + l->gw_DZ - 1) / l->gw_DZ;
     }
     l->ps_grid = 0;
-    if (!is_rk(l->p.integrator) && !l->gauge && !l->gw && !l->user_tiles && l->V <= persist_max_sites(l) &&
+    if (!is_rk(l->p.integrator) && !l->gauge && !l->gw && !l->user_opts && !l->no_resident && l->V <= persist_max_sites(l) &&
         persist_tiles(prec, N, nsm, &l->ps_BY, &l->ps_BZ)) {
         // small lattices: cl_step runs its passes in the resident kernel
         if (!l->ps_barrier && !dev_alloc(l, &l->ps_barrier, 256))
@@ -2009,9 +2010,9 @@ cl_status cl_get_option(cl_lattice* l, int32_t option, int64_t* value)
     return fail(l, CL_EINVAL, "unknown option %d", option);
 }
 
-static cl_status retile(cl_lattice* l)
+static cl_status retile(cl_lattice* l, int32_t option, bool set)
 {
-    l->user_tiles = l->opt_BY != 0 || l->opt_DZ != 0 || l->opt_stages != 0 || l->opt_variant != -1;
+    l->user_opts = set ? l->user_opts | 1u << option : l->user_opts & ~(1u << option);
     return choose_tiles(l);
 }
 
@@ -2023,22 +2024,22 @@ cl_status cl_set_option(cl_lattice* l, int32_t option, int64_t value)
     case CL_OPT_TILE_BY:
         if (value < 0 || value > l->N) return fail(l, CL_EINVAL, "tile BY out of range");
         l->opt_BY = (int)value;
-        return retile(l);
+        return retile(l, option, value != 0);
     case CL_OPT_TILE_DZ:
         if (value < -1 || value > l->N) return fail(l, CL_EINVAL, "tile DZ out of range");
         l->opt_DZ = (int)value;
-        return retile(l);
+        return retile(l, option, value != 0);
     case CL_OPT_PASS_VARIANT:
         if (value < -1 || value > (l->gauge ? 3 : 1))
             return fail(l, CL_EINVAL, "pass variant must be -1, 0 or 1 (2, 3 on an axion-U(1) lattice)");
         if (value == 1 && is_u1_lf(l))
             return fail(l, CL_EUNSUPPORTED, "the axion-U(1) leapfrog has no fused pass form");
         l->opt_variant = (int)value;
-        return retile(l);
+        return retile(l, option, value != -1);
     case CL_OPT_STAGES:
         if (value < -1 || value == 1 || value > 6) return fail(l, CL_EINVAL, "stages must be -1, 0 or 2..6");
         l->opt_stages = (int)value;
-        return retile(l);
+        return retile(l, option, value != 0);
     }
     return fail(l, CL_EINVAL, "unknown option %d", option);
 }
@@ -2076,7 +2077,7 @@ static std::string tune_key(const cl_lattice* l)
 
 static cl_status apply_tiles(cl_lattice* l, int stages, int by, int dz, int variant)
 {
-    l->user_tiles = false;
+    l->user_opts = 0;
     l->opt_stages = stages;
     l->opt_BY = by;
     l->opt_DZ = dz;
@@ -2108,6 +2109,55 @@ static cl_status time_trials(cl_lattice* l, int warm, int n, double* us)
     return s;
 }
 
+// The same for the passes of resident launches.  These advance the state, which is put back from a
+// copy.  *us = 0: no memory for one, not timed.
+static cl_status time_resident(cl_lattice* l, double* us)
+{
+    const std::vector<PassCoef> sched = {{l->p.dt, 0.5 * l->p.dt, l->p.dt, P_DRIFT | P_COMMIT}};
+    const size_t bytes = (size_t)l->V * l->es;
+    void* state[3 * 2];
+    int n = 0;
+    for (int f = 0; f < l->nf; ++f) {
+        state[n++] = l->phi[f][l->cur];
+        state[n++] = l->pi[f][l->cur];
+        if (has_kahan(l)) state[n++] = l->cc[f][l->cur];
+    }
+    char* copy = nullptr;
+    *us = 0.0;
+    if (!dev_alloc(l, &copy, n * bytes + sizeof(DevScal))) return CL_OK;
+    auto saved = [&](bool back) {
+        for (int i = 0; i <= n; ++i) {
+            void* p = i < n ? state[i] : (void*)l->scal;
+            char* c = copy + i * bytes;
+            const cudaError_t e = cudaMemcpyAsync(back ? p : c, back ? c : p, i < n ? bytes : sizeof(DevScal),
+                                                  cudaMemcpyDeviceToDevice, l->stream);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
+    cudaEvent_t a = nullptr, b = nullptr;
+    cl_status s = CL_OK;
+    const bool have_copy = saved(false) == cudaSuccess;
+    if (!have_copy || cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess)
+        s = fail(l, CL_ECUDA, "resident trial: set-up failed");
+    l->sync_valid = false;
+    for (int warm = 1; s == CL_OK && warm >= 0; --warm) {  // even counts: the state's buffer stays
+        const int passes = warm ? 16 : 128;
+        cudaEventRecord(a, l->stream);
+        s = is_fp64(l) ? run_persist_t<double>(l, sched, passes) : run_persist_t<float>(l, sched, passes);
+        cudaEventRecord(b, l->stream);
+        float ms = 0.f;
+        if (s == CL_OK && (cudaEventSynchronize(b) != cudaSuccess || cudaEventElapsedTime(&ms, a, b) != cudaSuccess))
+            s = fail(l, CL_ECUDA, "resident trial failed");
+        *us = 1e3 * ms / passes;
+    }
+    if (have_copy && saved(true) != cudaSuccess && s == CL_OK) s = fail(l, CL_ECUDA, "resident trial: copy failed");
+    if (a) cudaEventDestroy(a);
+    if (b) cudaEventDestroy(b);
+    cudaFree(copy);
+    return s;
+}
+
 cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
 {
     if (!l) return CL_EINVAL;
@@ -2119,6 +2169,7 @@ cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
         if (FILE* f = fopen(cache_path, "r")) {
             char line[512];
             int hit = 0, st = 0, by = 0, dz = 0, var = 1;
+            bool launches = false;  // a launch per pass was faster than the resident kernel
             double us = 0.0;
             while (fgets(line, sizeof(line), f)) {
                 const char* k = strstr(line, "\"key\": \"");
@@ -2127,10 +2178,13 @@ cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
                 const char* e = strchr(k, '"');
                 if (!e || std::string(k, e - k) != key) continue;
                 if (sscanf(e, "\", \"stages\": %d, \"by\": %d, \"dz\": %d, \"variant\": %d, \"us\": %lf", &st, &by, &dz,
-                           &var, &us) == 5)
+                           &var, &us) == 5) {
                     hit = 1;
+                    launches = strstr(e, "\"resident\": 0") != nullptr;
+                }
             }
             fclose(f);
+            if (hit) l->no_resident = launches;
             if (hit && apply_tiles(l, st, by, dz, var) == CL_OK) {
                 report_tiles(l, us, best);
                 l->diag_valid = false;
@@ -2139,8 +2193,8 @@ cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
             }
         }
     }
-    // candidates
     // candidates {stages, BY, DZ, pass variant}
+    l->no_resident = false;
     std::vector<std::array<int, 4>> cand;
     if (is_ens(l)) {
         // {stages, variant}: the direct loader, the ring kernel and the ringless kernel
@@ -2153,8 +2207,7 @@ cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
         cl_status s0 = apply_tiles(l, 0, 0, 0, 1);
         if (s0 != CL_OK) return s0;
         const int by_auto = l->BY;
-        // the ringless kernels take 16-byte vectors, or FP32 rows of any alignment
-        const bool nr_ok = l->VW * l->es == 16 || l->any_rows;
+        const bool nr_ok = l->VW * l->es == 16;  // the ringless kernel takes 16-byte vectors
         std::vector<int> st_list = {-1, 0};
         if (scalar_pass_tma_ok(l->p.precision, l->N))
             for (int st = 2; st <= 6; ++st) st_list.push_back(st);
@@ -2181,13 +2234,25 @@ cl_status cl_autotune(cl_lattice* l, const char* cache_path, double* best)
     }
     cl_status s = apply_tiles(l, best_c[0], best_c[1], best_c[2], best_c[3]);
     if (s != CL_OK) return s;
+    if (l->ps_grid > 0) {  // a small lattice: the steps' resident launches against the best tiling
+        double us = 0.0;
+        s = time_resident(l, &us);
+        if (s != CL_OK) return s;
+        if (us > best_us) {
+            l->no_resident = true;
+            s = choose_tiles(l);
+            if (s != CL_OK) return s;
+        } else if (us > 0.0) {
+            best_us = us;
+        }
+    }
     CUDA_TRY(l, cudaStreamSynchronize(l->stream));
     l->diag_valid = false;
     l->rbar_valid = false;
     if (cache_path && best_us < 1e300) {
         if (FILE* f = fopen(cache_path, "a")) {
-            fprintf(f, "{\"key\": \"%s\", \"stages\": %d, \"by\": %d, \"dz\": %d, \"variant\": %d, \"us\": %.3f}\n",
-                    key.c_str(), best_c[0], best_c[1], best_c[2], best_c[3], best_us);
+            fprintf(f, "{\"key\": \"%s\", \"stages\": %d, \"by\": %d, \"dz\": %d, \"variant\": %d, \"us\": %.3f, \"resident\": %d}\n",
+                    key.c_str(), best_c[0], best_c[1], best_c[2], best_c[3], best_us, l->ps_grid > 0 ? 1 : 0);
             fclose(f);
         }
     }

@@ -106,7 +106,8 @@ struct cl_lattice {
     double hubble_limit = 0.0;
     bool use_graph = true;
     unsigned user_opts = 0;         // tiling options set by the caller (1 << option; not by the autotuner)
-    bool no_resident = false;       // the autotuner measured a launch per pass to be faster
+    bool no_resident = false;       // no resident launches: the autotuner measured a launch per pass to be
+                                    //   faster, or one did not fit the SMs that the stream may use
     int ps_BY = 0, ps_BZ = 0, ps_grid = 0;  // resident multi-pass kernel: box of rows, blocks (0: not used)
     unsigned* ps_barrier = nullptr;
     int opt_BY = 0, opt_DZ = 0, opt_stages = 0, opt_variant = -1;  // -1: library choice
@@ -597,9 +598,8 @@ cl_status choose_tiles(cl_lattice* l)
     if (!is_rk(l->p.integrator) && !l->gauge && !l->gw && !l->user_opts && !l->no_resident && l->V <= persist_max_sites(l) &&
         persist_tiles(prec, N, nsm, &l->ps_BY, &l->ps_BZ)) {
         // small lattices: cl_step runs its passes in the resident kernel
-        if (!l->ps_barrier && !dev_alloc(l, &l->ps_barrier, 256))
-            return fail(l, CL_ENOMEM, "cannot allocate the grid barrier");
-        l->ps_grid = ((N + l->ps_BY - 1) / l->ps_BY) * ((N + l->ps_BZ - 1) / l->ps_BZ);
+        if (l->ps_barrier || dev_alloc(l, &l->ps_barrier, 256))
+            l->ps_grid = ((N + l->ps_BY - 1) / l->ps_BY) * ((N + l->ps_BZ - 1) / l->ps_BZ);
         static_assert(3 * (kMaxQ + 1) <= 4 * kMaxQ, "three buffers of kMaxQ + 1 numbers a block");
         if (4 * l->ps_grid > nblocks) nblocks = 4 * l->ps_grid;
     }
@@ -1058,9 +1058,11 @@ double open_kick(const cl_lattice* l)
     return 0.5 * w[0] * l->p.dt;
 }
 
-// nsteps steps of a small lattice in launches of the resident kernel (open leapfrog).
+// nsteps steps of a small lattice in launches of the resident kernel (open leapfrog).  *done: the steps
+// taken -- fewer (and the handle launches every pass from then on) where not all of its blocks can be
+// resident at once: a stream or process limited to some of the SMs.
 template <typename T>
-cl_status run_persist_t(cl_lattice* l, const std::vector<PassCoef>& sched, int nsteps)
+cl_status run_persist_t(cl_lattice* l, const std::vector<PassCoef>& sched, int nsteps, int* done)
 {
     PersistArgs<T> A{};
     for (int f = 0; f < l->nf; ++f)
@@ -1085,15 +1087,21 @@ cl_status run_persist_t(cl_lattice* l, const std::vector<PassCoef>& sched, int n
     A.hubble_limit = l->hubble_limit;
     A.flags = l->p.expansion ? P_EXPANSION : 0;
     const int most = kPersistPasses / A.pps;  // steps of one launch
-    for (int done = 0; done < nsteps;) {
-        const int n = std::min(most, nsteps - done);
+    for (*done = 0; *done < nsteps;) {
+        const int n = std::min(most, nsteps - *done);
         A.in0 = l->cur;
         A.passes = n * A.pps;
         CUDA_TRY(l, cudaMemsetAsync(l->ps_barrier, 0, sizeof(unsigned), l->stream));
         const cudaError_t e = launch_scalar_persist(l->p.precision, l->nf, &A, l->ps_grid, l->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+            cudaGetLastError();
+            l->no_resident = true;
+            l->ps_grid = 0;
+            return CL_OK;
+        }
         if (e != cudaSuccess) return fail(l, CL_ECUDA, "resident pass launch failed: %s", cudaGetErrorString(e));
         l->cur = (l->cur + A.passes) & 1;
-        done += n;
+        *done += n;
     }
     return CL_OK;
 }
@@ -2110,7 +2118,7 @@ static cl_status time_trials(cl_lattice* l, int warm, int n, double* us)
 }
 
 // The same for the passes of resident launches.  These advance the state, which is put back from a
-// copy.  *us = 0: no memory for one, not timed.
+// copy.  *us = 0: no memory for one, or no such launches: not timed.
 static cl_status time_resident(cl_lattice* l, double* us)
 {
     const std::vector<PassCoef> sched = {{l->p.dt, 0.5 * l->p.dt, l->p.dt, P_DRIFT | P_COMMIT}};
@@ -2144,7 +2152,9 @@ static cl_status time_resident(cl_lattice* l, double* us)
     for (int warm = 1; s == CL_OK && warm >= 0; --warm) {  // even counts: the state's buffer stays
         const int passes = warm ? 16 : 128;
         cudaEventRecord(a, l->stream);
-        s = is_fp64(l) ? run_persist_t<double>(l, sched, passes) : run_persist_t<float>(l, sched, passes);
+        int done = 0;
+        s = is_fp64(l) ? run_persist_t<double>(l, sched, passes, &done) : run_persist_t<float>(l, sched, passes, &done);
+        if (done < passes) break;  // none of them fits: *us stays 0
         cudaEventRecord(b, l->stream);
         float ms = 0.f;
         if (s == CL_OK && (cudaEventSynchronize(b) != cudaSuccess || cudaEventElapsedTime(&ms, a, b) != cudaSuccess))
@@ -2292,11 +2302,13 @@ cl_status cl_step(cl_lattice* l, int32_t nsteps)
     // that of their last input state
     l->rbar_valid = nmc_f;
     if (l->ps_grid > 0) {
-        cl_status s = is_fp64(l) ? run_persist_t<double>(l, sched, nsteps) : run_persist_t<float>(l, sched, nsteps);
+        int done = 0;
+        cl_status s = is_fp64(l) ? run_persist_t<double>(l, sched, nsteps, &done) : run_persist_t<float>(l, sched, nsteps, &done);
         if (s != CL_OK) return s;
-        l->last_launches += (int64_t)pps * nsteps;  // the passes that ran, as everywhere
+        l->last_launches += (int64_t)pps * done;  // the passes that ran, as everywhere
         l->diag_valid = true;
-        return CL_OK;
+        nsteps -= done;
+        if (nsteps == 0) return CL_OK;
     }
     for (int i = 0; i < nsteps; ++i) {
         if (l->use_graph) {

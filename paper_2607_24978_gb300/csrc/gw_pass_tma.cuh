@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(480, 1) k_gw_pass_tma(const GwPassArgs<float> 
             }
         }
     } else {
-        using P2 = Two<float>;
+        using P2 = Two;
         const bool do_drift = (A.flags & P_DRIFT) != 0;
         if (tid < 2) {  // beside the copies of the first planes
             const bool expand = (A.flags & P_EXPANSION) != 0;

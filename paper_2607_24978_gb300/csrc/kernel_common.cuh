@@ -100,13 +100,11 @@ __device__ __forceinline__ void drift(T& phi, T& c, T pi, T cd)
     }
 }
 
-// Two values of the element type handled together.  FP32: one 64-bit register pair and the
-// packed instructions of Blackwell (add, mul and fma on both halves in one issue slot, each
-// half rounded as the scalar instruction; the lanes per cycle are the same, so what they save is
-// issue slots -- measured: 1.9 packed against 3.6 scalar instructions per cycle and SM).
-// FP64: two scalars.
-template <typename T> struct Two;
-template <> struct Two<float> {
+// Two FP32 values handled together: one 64-bit register pair and the packed instructions of
+// Blackwell (add, mul and fma on both halves in one issue slot, each half rounded as the scalar
+// instruction; the lanes per cycle are the same, so what they save is issue slots -- measured: 1.9
+// packed against 3.6 scalar instructions per cycle and SM).
+struct Two {
     unsigned long long v;
     __device__ __forceinline__ Two() {}
     __device__ __forceinline__ Two(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
@@ -123,58 +121,43 @@ template <> struct Two<float> {
         return b;
     }
 };
-template <> struct Two<double> {
-    double a, b;
-    __device__ __forceinline__ Two() {}
-    __device__ __forceinline__ Two(double x, double y) : a(x), b(y) {}
-    __device__ __forceinline__ double lo() const { return a; }
-    __device__ __forceinline__ double hi() const { return b; }
-};
-__device__ __forceinline__ Two<float> fma2(Two<float> a, Two<float> b, Two<float> c)
+__device__ __forceinline__ Two fma2(Two a, Two b, Two c)
 {
-    Two<float> d;
+    Two d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return d;
 }
-__device__ __forceinline__ Two<float> add2(Two<float> a, Two<float> b)
+__device__ __forceinline__ Two add2(Two a, Two b)
 {
-    Two<float> d;
+    Two d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
     return d;
 }
-__device__ __forceinline__ Two<float> sub2(Two<float> a, Two<float> b)
+__device__ __forceinline__ Two sub2(Two a, Two b)
 {
-    Two<float> d;
+    Two d;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
     return d;
 }
-__device__ __forceinline__ Two<float> mul2(Two<float> a, Two<float> b)
+__device__ __forceinline__ Two mul2(Two a, Two b)
 {
-    Two<float> d;
+    Two d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
     return d;
 }
-__device__ __forceinline__ Two<double> fma2(Two<double> a, Two<double> b, Two<double> c)
-{
-    return {__fma_rn(a.a, b.a, c.a), __fma_rn(a.b, b.b, c.b)};
-}
-__device__ __forceinline__ Two<double> add2(Two<double> a, Two<double> b) { return {__dadd_rn(a.a, b.a), __dadd_rn(a.b, b.b)}; }
-__device__ __forceinline__ Two<double> sub2(Two<double> a, Two<double> b) { return {__dsub_rn(a.a, b.a), __dsub_rn(a.b, b.b)}; }
-__device__ __forceinline__ Two<double> mul2(Two<double> a, Two<double> b) { return {__dmul_rn(a.a, b.a), __dmul_rn(a.b, b.b)}; }
-template <typename T>
-__device__ __forceinline__ Two<T> both(T x)
+__device__ __forceinline__ Two both(float x)
 {
     return {x, x};
 }
 
 // drift of two values; ncd = -cd.  The same rounded values as drift(): y' = fma(-cd, pi, c) is
 // -y, so phi + y = phi - y' and (t - phi) - y = (t - phi) + y'.
-template <typename T, bool KAHAN>
-__device__ __forceinline__ void drift2(Two<T>& phi, Two<T>& c, Two<T> pi, Two<T> cd, Two<T> ncd)
+template <bool KAHAN>
+__device__ __forceinline__ void drift2(Two& phi, Two& c, Two pi, Two cd, Two ncd)
 {
     if (KAHAN) {
-        const Two<T> y = fma2(ncd, pi, c);
-        const Two<T> t = sub2(phi, y);
+        const Two y = fma2(ncd, pi, c);
+        const Two t = sub2(phi, y);
         c = add2(sub2(t, phi), y);
         phi = t;
     } else {

@@ -481,8 +481,8 @@ static cudaError_t launch_any(const ScalarPassArgs<T>& A, dim3 grid, cudaStream_
         const int block = scalar_pass_any_threads(A.N, A.BY) + 32;
         const size_t smem = scalar_pass_smem_bytes(prec, NF, A.N, A.BY, A.stages, 2);
         if (block > 480 || smem > (size_t)kPassMaxSmem || (A.stages != 3 && A.stages != 4)) return cudaErrorInvalidValue;
-        auto* k3 = k_scalar_pass_tma_any<T, NF, KAHAN, kAnySites, 3>;
-        auto* k4 = k_scalar_pass_tma_any<T, NF, KAHAN, kAnySites, 4>;
+        auto* k3 = k_scalar_pass_tma_any<NF, KAHAN, kAnySites, 3>;
+        auto* k4 = k_scalar_pass_tma_any<NF, KAHAN, kAnySites, 4>;
         auto* k = A.stages == 3 ? k3 : k4;
         static DevFlag attr[2];
         DevFlag& set = attr[A.stages - 3];

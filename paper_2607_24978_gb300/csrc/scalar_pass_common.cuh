@@ -187,10 +187,9 @@ __device__ __forceinline__ void kick_vector(const T* const (&Sc)[NF], const T* c
 }
 
 // Coefficients of the kick of two sites at a time (each constant twice).
-template <typename T>
 struct KickCoef2 {
-    Two<T> cL, cV, ce, ck, m20, m21, l0, l1, g2, h_m20, h_m21, q_l0, q_l1, h_g2;
-    __device__ __forceinline__ KickCoef2(T cL_, T cV_, T ce_, T ck_, const PotCoef<T>& P)
+    Two cL, cV, ce, ck, m20, m21, l0, l1, g2, h_m20, h_m21, q_l0, q_l1, h_g2;
+    __device__ __forceinline__ KickCoef2(float cL_, float cV_, float ce_, float ck_, const PotCoef<float>& P)
         : cL(both(cL_)), cV(both(-cV_)), ce(both(ce_)), ck(both(ck_)), m20(both(P.m20)), m21(both(P.m21)),
           l0(both(P.l0)), l1(both(P.l1)), g2(both(P.g2)), h_m20(both(P.h_m20)), h_m21(both(P.h_m21)),
           q_l0(both(P.q_l0)), q_l1(both(P.q_l1)), h_g2(both(P.h_g2))
@@ -200,28 +199,28 @@ struct KickCoef2 {
 
 // Kick of two sites: fields p[f], Laplacians lap[f] and momenta pin[f] (times dx^2 as in
 // kick_vector).  Returns the kicked momenta in pin and adds pi_int^2 to ks[f] and V to vs.
-template <typename T, int NF>
-__device__ __forceinline__ void kick_two(const Two<T> (&p)[NF], const Two<T> (&lap)[NF], Two<T> (&pin)[NF],
-                                         const KickCoef2<T>& C, Two<T> (&ks)[NF], Two<T>& vs)
+template <int NF>
+__device__ __forceinline__ void kick_two(const Two (&p)[NF], const Two (&lap)[NF], Two (&pin)[NF],
+                                         const KickCoef2& C, Two (&ks)[NF], Two& vs)
 {
-    const Two<T> p0 = p[0];
-    Two<T> s0 = fma2(mul2(C.l0, p0), p0, C.m20), v = fma2(mul2(C.q_l0, p0), p0, C.h_m20);
-    const Two<T> P0 = mul2(p0, p0);
+    const Two p0 = p[0];
+    Two s0 = fma2(mul2(C.l0, p0), p0, C.m20), v = fma2(mul2(C.q_l0, p0), p0, C.h_m20);
+    const Two P0 = mul2(p0, p0);
     vs = fma2(P0, v, vs);
     if constexpr (NF > 1) {
-        const Two<T> p1 = p[NF - 1], P1 = mul2(p1, p1);
+        const Two p1 = p[NF - 1], P1 = mul2(p1, p1);
         s0 = fma2(mul2(C.g2, p1), p1, s0);
-        Two<T> s1 = fma2(mul2(C.l1, p1), p1, C.m21);
+        Two s1 = fma2(mul2(C.l1, p1), p1, C.m21);
         s1 = fma2(mul2(C.g2, p0), p0, s1);
         v = fma2(C.h_g2, P0, fma2(C.q_l1, P1, C.h_m21));
         vs = fma2(P1, v, vs);
-        const Two<T> F1 = fma2(C.cL, lap[NF - 1], mul2(C.cV, mul2(p1, s1)));
-        const Two<T> pe = fma2(C.ce, F1, pin[NF - 1]);
+        const Two F1 = fma2(C.cL, lap[NF - 1], mul2(C.cV, mul2(p1, s1)));
+        const Two pe = fma2(C.ce, F1, pin[NF - 1]);
         pin[NF - 1] = fma2(C.ck, F1, pin[NF - 1]);
         ks[NF - 1] = fma2(pe, pe, ks[NF - 1]);
     }
-    const Two<T> F0 = fma2(C.cL, lap[0], mul2(C.cV, mul2(p0, s0)));
-    const Two<T> pe = fma2(C.ce, F0, pin[0]);
+    const Two F0 = fma2(C.cL, lap[0], mul2(C.cV, mul2(p0, s0)));
+    const Two pe = fma2(C.ce, F0, pin[0]);
     pin[0] = fma2(C.ck, F0, pin[0]);
     ks[0] = fma2(pe, pe, ks[0]);
 }

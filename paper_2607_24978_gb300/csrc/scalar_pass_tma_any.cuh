@@ -16,16 +16,17 @@
 // threads whatever N is.  x neighbours come from the warp's registers by shuffles; the first
 // and last site of a row or of a warp's sites drift their neighbour again from the stage.
 //
-// The arithmetic runs on pairs of sites (Two<T>): the kernel is bound by issue and the latency
+// The arithmetic runs on pairs of sites (Two): the kernel is bound by issue and the latency
 // behind it (14 consumer warps an SM, 56 % of the issue slots at 251^3, two fields), and packed
 // instructions take half the slots of the scalar ones: 213 -> 174 us a pass.  The energy sums stay
 // scalar, every site added to the thread's compensated sum by itself: pairs of sums take twice the
 // registers of the sums and spill (227 us with them; sums of the two fields in pairs 192).  Copying every row
 // with scalar loads through the direct loader took 619 us there (363 -> 92 with one field; 125^3
 // two fields 94 -> 36; 250^3, 8-byte vectors, 263 -> 174); HBM alone would need 113 us.
-template <typename T, int NF, bool KAHAN, int CH, int S>
-__global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPassArgs<T> A)
+template <int NF, bool KAHAN, int CH, int S>
+__global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPassArgs<float> A)
 {
+    using T = float;
     constexpr int KPF = KAHAN ? 3 : 2;
     constexpr int NARR = NF * KPF;
     constexpr int E = 16 / (int)sizeof(T);
@@ -106,14 +107,14 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
         constexpr int CP = CH / 2;  // pairs of sites (k = 2 i, 2 i + 1)
         consumer_coefficients(tid, CT, A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);
         const T cd = (T)s_coef[0];
-        const Two<T> cd2 = both(cd), ncd2 = both(-cd), six = both((T)-6);
+        const Two cd2 = both(cd), ncd2 = both(-cd), six = both((T)-6);
         const bool do_drift = (A.flags & P_DRIFT) != 0;
         const PotCoef<T> P(A.m2, A.lam, A.g2);
-        const KickCoef2<T> KC((T)s_coef[1], (T)s_coef[2], (T)A.e, (T)A.k, P);
+        const KickCoef2 KC((T)s_coef[1], (T)s_coef[2], (T)A.e, (T)A.k, P);
         const int lane = tid & 31;
         const int first = (tid >> 5) * 32 * CH + lane;  // the lane's first site of the tile
-        Two<T> pcur[NF][CP], pnext[NF][CP];
-        Two<T> zlo[NF][CP], zmid[NF][CP], znew[NF][CP];
+        Two pcur[NF][CP], pnext[NF][CP];
+        Two zlo[NF][CP], zmid[NF][CP], znew[NF][CP];
         int st = 0, st_prev = 0;
         uint32_t full_phase = 0;
         const size_t plane = (size_t)N * N;
@@ -170,13 +171,13 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                     for (int f = 0; f < NF; ++f) {
                         const T* sa = sb + f * KPF * arr_stride + HN + sh[1] + first;
                         const T *sv = sa + arr_stride, *sc = sv + arr_stride;
-                        Two<T> cv[CP];
+                        Two cv[CP];
 #pragma unroll
                         for (int i = 0; i < CP; ++i) {
-                            znew[f][i] = Two<T>(sa[64 * i], sa[64 * i + 32]);
-                            pnext[f][i] = Two<T>(sv[64 * i], sv[64 * i + 32]);
-                            if (KAHAN) cv[i] = Two<T>(sc[64 * i], sc[64 * i + 32]);
-                            if (do_drift) drift2<T, KAHAN>(znew[f][i], cv[i], pnext[f][i], cd2, ncd2);
+                            znew[f][i] = Two(sa[64 * i], sa[64 * i + 32]);
+                            pnext[f][i] = Two(sv[64 * i], sv[64 * i + 32]);
+                            if (KAHAN) cv[i] = Two(sc[64 * i], sc[64 * i + 32]);
+                            if (do_drift) drift2<KAHAN>(znew[f][i], cv[i], pnext[f][i], cd2, ncd2);
                         }
                         if (write_out) {
                             T *po = A.phi_out[f] + base, *co = A.c_out[f] + base;
@@ -196,24 +197,24 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                 }
                 if (j >= 2) {
                     const T* sp = stage + st_prev * stage_stride;
-                    Two<T> lap[NF][CP];
+                    Two lap[NF][CP];
 #pragma unroll
                     for (int f = 0; f < NF; ++f) {
                         const T* sa = sp + f * KPF * arr_stride;
                         const int own = HN + sh_prev[1] + first;
                         // y neighbours (y2): a row down or up in the own region -- one unbroken
                         // stretch, 32 elements between a lane's sites -- or the halo row
-                        Two<T> y2[CP];
+                        Two y2[CP];
                         auto load_row = [&](const T* s0) {
                             const T *s1 = s0 + arr_stride, *s2 = s1 + arr_stride;
 #pragma unroll
                             for (int i = 0; i < CP; ++i) {
-                                y2[i] = Two<T>(s0[64 * i], s0[64 * i + 32]);
+                                y2[i] = Two(s0[64 * i], s0[64 * i + 32]);
                                 if (do_drift) {
-                                    const Two<T> m(s1[64 * i], s1[64 * i + 32]);
-                                    Two<T> c;
-                                    if (KAHAN) c = Two<T>(s2[64 * i], s2[64 * i + 32]);
-                                    drift2<T, KAHAN>(y2[i], c, m, cd2, ncd2);
+                                    const Two m(s1[64 * i], s1[64 * i + 32]);
+                                    Two c;
+                                    if (KAHAN) c = Two(s2[64 * i], s2[64 * i + 32]);
+                                    drift2<KAHAN>(y2[i], c, m, cd2, ncd2);
                                 }
                             }
                         };
@@ -223,19 +224,19 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                             for (int k = 0; k < CH; ++k)
                                 y[k] = drifted1(sa, (in_halo >> k & 1u ? halo_off : own_off) + 32 * k);
 #pragma unroll
-                            for (int i = 0; i < CP; ++i) y2[i] = Two<T>(y[2 * i], y[2 * i + 1]);
+                            for (int i = 0; i < CP; ++i) y2[i] = Two(y[2 * i], y[2 * i + 1]);
                         };
-                        Two<T> ysum[CP];
+                        Two ysum[CP];
                         if (warp_lo) load_halo(lo_row, own - N, sh_prev[0] + first);
                         else load_row(sa + own - N);
 #pragma unroll
                         for (int i = 0; i < CP; ++i) ysum[i] = y2[i];
                         if (warp_hi) load_halo(hi_row, own + N, HN + ON + sh_prev[2] + first - (R - 1) * N);
                         else load_row(sa + own + N);
-                        Two<T> gs[CP];
+                        Two gs[CP];
 #pragma unroll
                         for (int i = 0; i < CP; ++i) {
-                            const Two<T> gy = sub2(y2[i], zmid[f][i]);
+                            const Two gy = sub2(y2[i], zmid[f][i]);
                             gs[i] = mul2(gy, gy);
                             ysum[i] = add2(y2[i], ysum[i]);
                         }
@@ -257,9 +258,9 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                         }
 #pragma unroll
                         for (int i = 0; i < CP; ++i) {
-                            const Two<T> c = zmid[f][i], xm(xmv[2 * i], xmv[2 * i + 1]), xp(xpv[2 * i], xpv[2 * i + 1]);
+                            const Two c = zmid[f][i], xm(xmv[2 * i], xmv[2 * i + 1]), xp(xpv[2 * i], xpv[2 * i + 1]);
                             lap[f][i] = fma2(six, c, add2(add2(add2(xp, xm), ysum[i]), add2(znew[f][i], zlo[f][i])));
-                            const Two<T> gx = sub2(xp, c), gz = sub2(znew[f][i], c);
+                            const Two gx = sub2(xp, c), gz = sub2(znew[f][i], c);
                             gs[i] = fma2(gx, gx, fma2(gz, gz, gs[i]));
                             accG[f].add(valid >> (2 * i) & 1u ? gs[i].lo() : (T)0);
                             accG[f].add(valid >> (2 * i + 1) & 1u ? gs[i].hi() : (T)0);
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                     const size_t base = (size_t)(z0 + j - 2) * plane + row_off + first;
 #pragma unroll
                     for (int i = 0; i < CP; ++i) {
-                        Two<T> p[NF], l[NF], q[NF], k1[NF], v1 = both((T)0);
+                        Two p[NF], l[NF], q[NF], k1[NF], v1 = both((T)0);
 #pragma unroll
                         for (int f = 0; f < NF; ++f) {
                             p[f] = zmid[f][i];
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                             q[f] = pcur[f][i];
                             k1[f] = both((T)0);
                         }
-                        kick_two<T, NF>(p, l, q, KC, k1, v1);
+                        kick_two<NF>(p, l, q, KC, k1, v1);
                         const bool va = valid >> (2 * i) & 1u, vb = valid >> (2 * i + 1) & 1u;
 #pragma unroll
                         for (int f = 0; f < NF; ++f) {

@@ -109,7 +109,10 @@ enum {
  * count, advanced together by one launch per pass (N and L are then ignored).  They share
  * nfields, precision, integrator (VV-2 or a Yoshida composition), alpha, kappa and dt;
  * gauge must be CL_GAUGE_NONE.  Every call that takes a member addresses one of them; the
- * fields of member m hold member_N[m]^3 elements.  Errors at creation: CL_EINVAL (sizes),
+ * fields of member m hold member_N[m]^3 elements.  A member evolves bit for bit as it would beside
+ * any other members with which the library takes the same pass kernel (CL_OPT_STAGES and
+ * CL_OPT_PASS_VARIANT report it; the vector width of a row is the largest that divides all
+ * members' rows).  Errors at creation: CL_EINVAL (sizes),
  * CL_EUNSUPPORTED (Runge-Kutta or gauge ensembles). */
 typedef struct {
     int32_t N;            /* sites per side, 2 <= N <= 1536 (single lattice; reduced      */
@@ -342,7 +345,8 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * of one wave, each block a balanced contiguous range of planes; for the axion-U(1)
  * kernels, the planes of the z chunk each (x, y) tile marches through, half as many in the staged
  * plaquette launches, whose tiles have twice the sites; ensembles: planes per work item, 0 = the
- * members' columns cut into blocks of equal work).  CL_OPT_STAGES: TMA stage buffers
+ * members' columns of planes, whole or cut into blocks of equal work where that is estimated to be
+ * faster).  CL_OPT_STAGES: TMA stage buffers
  * of the fused pass, 2..6, or -1 for the loader without TMA staging (0 = library choice;
  * FP32 rows that are not a multiple of 16 bytes run their own staged kernel with 3 or 4
  * buffers, whatever the variant (reported as 0), unless stages -1 is asked for; FP64 ones always

@@ -146,7 +146,7 @@ struct cl_lattice {
     EnsMember* d_members = nullptr;
     EnsItem* d_items = nullptr;
     int* h_status = nullptr;        // page-locked: the members' status words, joined (check_status)
-    int* d_first = nullptr;         // first item of each block of a whole pass (library's cuts)
+    int* d_sched = nullptr;         // a whole pass's lists of items: where each block's begins, then the items
     int nitems = 0, ens_grid = 0, ens_stages = 0, ens_stage_stride = 0, ens_ring_slot = 0, ens_variant = 0;
     float* sg_buf = nullptr;        // surrogate jumps: packed input (3 V), output (2 V), snapshot (3 V)
     size_t ens_smem = 0;
@@ -232,57 +232,129 @@ cl_status upload_members(cl_lattice* l)
     return CL_OK;
 }
 
-// One column of an ensemble: BY full rows of a member, the planes from z0.
+// One column of an ensemble: BY full rows of a member, the planes from z0; items of it begin at
+// multiples of cz planes.
 struct EnsColumn {
-    int member, y0, z0, planes;
+    int member, y0, z0, planes, cz;
     int64_t row;  // work of one plane of it
+};
+// Items in member order, and the blocks' lists of them: block b runs sched[first[b] .. first[b + 1]).
+struct EnsPlan {
+    std::vector<EnsItem> items;
+    std::vector<int64_t> work;  // of each item
+    std::vector<int> sched, first;
+    int blocks() const { return (int)first.size() - 1; }
 };
 
 // Work of an item, in units of one site's bandwidth share: a plane of it takes the time of its sites
 // or, where the block waits rather than copies, about that of kEnsPlane sites (1550 cycles); the two
-// halo planes and the start and the end of an item (prefactors, partial sums, the member's epilogue:
-// 15000 to 25000 cycles) that of kEnsExtra planes.  Measured (us a pass; one field, FP32 with
-// compensated sums; members of 32, 48, 64 sites in turn / 16, 32 / 27, 33, 50 / 24, 40, 56): whole
-// columns dealt out by decreasing size 184 (256 members), 33 (8), 146 (100), 50 (40); cut by sites
-// alone with kEnsExtra = 8 177, 40, 119, 35; so 162, 22, 101, 32.
-constexpr int kEnsPlane = 1024, kEnsExtra = 18;
-constexpr int kEnsMinPlanes = 8;  // (16: 165, 23, 113, 35)
+// halo planes and the start and the end of an item (prefactors, the member's sums and epilogue)
+// that of kEnsExtra planes.
+constexpr int kEnsPlane = 1024, kEnsExtra = 12;
+// The most planes of a chunk of the sums (EnsMember), which is the least that an item has.  Adding a
+// warp's sums takes 0.5 us a chunk (64 members of 64^3, whole columns, us a pass: 78.8 with one chunk
+// a column, 80.3 at 22 planes, 82.0 at 16, 86 at 8), and short chunks let few members spread over more
+// SMs (two of 64^3: 57, 29, 26, 22).
+constexpr int kEnsChunk = 16;
+int64_t ens_work(int planes, int64_t row) { return (int64_t)(planes + kEnsExtra) * row; }
 
-// Cut the columns, one after the other, into blocks of at most `target` work each; an item keeps at
-// least min_planes planes (columns no longer than that stay whole).  Returns the number of blocks
-// (0: no block can hold the shortest item); with `items`, also the items and each block's first one.
-int ens_cut(const std::vector<EnsColumn>& cols, double target, int min_planes, std::vector<EnsItem>* items,
-            std::vector<int>* first)
+// Cut the columns, one after the other, into blocks of at most `target` work each, at chunk
+// boundaries.  Returns the number of blocks (0: no block can hold the shortest item); with `plan`,
+// also the items and the blocks' lists.
+int ens_cut(const std::vector<EnsColumn>& cols, int64_t target, EnsPlan* plan)
 {
     int blocks = 1, n = 0;
-    double load = 0.0;
-    if (first) first->assign(1, 0);
+    int64_t load = 0;
+    if (plan) *plan = EnsPlan{{}, {}, {}, {0}};
     for (const EnsColumn& c : cols)
         for (int z = 0; z < c.planes;) {
             const int left = c.planes - z;
-            const double room = (target - load) / (double)c.row - kEnsExtra;
-            int p = room >= left ? left : (int)room;
-            if (p < left && left - p < min_planes) p = left - min_planes;
-            if (p < (left < min_planes ? left : min_planes)) {
-                if (load == 0.0) return 0;
+            const int64_t room = (target - load) / c.row - kEnsExtra;
+            const int p = room >= left ? left : room < 0 ? 0 : (int)room / c.cz * c.cz;
+            if (p < 1) {
+                if (load == 0) return 0;
                 ++blocks;
-                load = 0.0;
-                if (first) first->push_back(n);
+                load = 0;
+                if (plan) plan->first.push_back(n);
                 continue;
             }
-            if (items) items->push_back({c.member, c.y0, c.z0 + z, p});
+            if (plan) {
+                plan->items.push_back({c.member, c.y0, c.z0 + z, p});
+                plan->work.push_back(ens_work(p, c.row));
+                plan->sched.push_back(n);
+            }
             ++n;
-            load += ((double)p + kEnsExtra) * (double)c.row;
+            load += ens_work(p, c.row);
             z += p;
         }
-    if (first) first->push_back(n);
+    if (plan) plan->first.push_back(n);
     return blocks;
 }
 
+// Whole columns dealt out to at most `blocks` blocks in turn, by decreasing work.
+EnsPlan ens_deal(const std::vector<EnsColumn>& cols, int blocks)
+{
+    EnsPlan P;
+    const int n = (int)cols.size();
+    if (blocks > n) blocks = n;
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) {
+        order[i] = i;
+        P.items.push_back({cols[i].member, cols[i].y0, cols[i].z0, cols[i].planes});
+        P.work.push_back(ens_work(cols[i].planes, cols[i].row));
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return P.work[a] > P.work[b]; });
+    for (int b = 0; b < blocks; ++b) {
+        P.first.push_back((int)P.sched.size());
+        for (int i = b; i < n; i += blocks) P.sched.push_back(order[i]);
+    }
+    P.first.push_back(n);
+    return P;
+}
+
+// Time of a plan: that of the slowest SM, whose blocks are b, b + nsm, ...: its longest block, and
+// the share `beside` of the others (two 64^3 columns on an SM take 1.45 times the time of one; the
+// direct loader's FP32 blocks wait, and four take little longer than one).
+double ens_time(const EnsPlan& P, int nsm, double beside)
+{
+    double worst = 0.0;
+    for (int s = 0; s < nsm && s < P.blocks(); ++s) {
+        int64_t longest = 0, sum = 0;
+        for (int b = s; b < P.blocks(); b += nsm) {
+            int64_t w = 0;
+            for (int i = P.first[b]; i < P.first[b + 1]; ++i) w += P.work[P.sched[i]];
+            longest = std::max(longest, w);
+            sum += w;
+        }
+        worst = std::max(worst, (double)longest + beside * (double)(sum - longest));
+    }
+    return worst;
+}
+
+// The ensemble's items and the blocks that run them: whole columns, or cut into one wave of blocks of
+// equal work where that is faster by the estimate above -- with columns for few of the SMs, or for
+// more than a wave of blocks.  Measured (us a pass, FP32 with compensated sums, one field, members of
+// these sizes in turn; whole columns / cut): 256 of 32, 48, 64 186 / 165; 8 of 16, 32 37 / 26; 40 of
+// 24, 40, 56 55 / 37; and kept whole: 256 of 16, 32 41 / 47; 100 of 27, 33, 50 100 / 103.
+EnsPlan ens_plan(const std::vector<EnsColumn>& cols, int wave, int nsm, double beside, bool may_cut)
+{
+    EnsPlan best = ens_deal(cols, wave);
+    if (!may_cut) return best;
+    int64_t lo = 0, hi = 0;  // hi: one block takes everything
+    for (const EnsColumn& c : cols) hi += (c.planes + kEnsExtra) * c.row;
+    while (hi - lo > 1) {
+        const int64_t mid = lo + (hi - lo) / 2;
+        const int n = ens_cut(cols, mid, nullptr);
+        if (n > 0 && n <= wave) hi = mid;
+        else lo = mid;
+    }
+    EnsPlan cut;
+    ens_cut(cols, hi, &cut);
+    return ens_time(cut, nsm, beside) < 0.99 * ens_time(best, nsm, beside) ? cut : best;
+}
+
 // Ensemble work items.  Per member: columns of BY full rows (as many as one block's threads
-// cover, balanced within the member).  The columns of all members, one after the other, are cut
-// into one wave of resident blocks of equal work, each a run of consecutive items (whole columns
-// and at most two parts), by the smallest target that a wave holds.
+// cover, balanced within the member), cut and dealt out by ens_plan.
 cl_status ens_tiles(cl_lattice* l)
 {
     const int B = l->members, prec = l->p.precision;
@@ -292,6 +364,7 @@ cl_status ens_tiles(cl_lattice* l)
     int64_t stage_max = 0, ring_max = 0;
     const int narr = l->nf * (has_kahan(l) ? 3 : 2);
     std::vector<EnsColumn> cols;
+    int units = 0;
     for (int m = 0; m < B; ++m) {
         const int N = l->mN[m], TX = N / l->VW;
         int BY = kEnsThreads / TX;
@@ -313,10 +386,16 @@ cl_status ens_tiles(cl_lattice* l)
         M.dx = l->mL[m] / N;
         if ((nby - 1) * BY >= N || (nbz - 1) * DZ >= N) return fail(l, CL_EINVAL, "ensemble tiling error");
         M.item0 = M.nitems = 0;
+        const int chunks = (N + kEnsChunk - 1) / kEnsChunk;
+        M.CZ = l->opt_DZ > 0 ? DZ : (N + chunks - 1) / chunks;  // CL_OPT_TILE_DZ's chunks are items
+        M.nkz = (N + M.CZ - 1) / M.CZ;
+        M.unit0 = units;
+        M.nunits = nby * M.nkz * (kEnsThreads / 32);
+        units += M.nunits;
         for (int bz = 0; bz < nbz; ++bz)
             for (int by = 0; by < nby; ++by) {
                 const int R = BY < N - by * BY ? BY : N - by * BY, nz = DZ < N - bz * DZ ? DZ : N - bz * DZ;
-                cols.push_back({m, by * BY, bz * DZ, nz, (int64_t)R * N + kEnsPlane});
+                cols.push_back({m, by * BY, bz * DZ, nz, M.CZ, (int64_t)R * N + kEnsPlane});
             }
         const size_t sm = (size_t)l->nf * 3 * (BY + 2) * N * l->es;
         if (sm > smem) smem = sm;
@@ -354,19 +433,10 @@ cl_status ens_tiles(cl_lattice* l)
         return fail(l, CL_ECUDA, "cannot query the SM count");
     CUDA_TRY(l, ensemble_pass_blocks_per_sm(prec, l->nf, l->VW, stages, var, smem, &per_sm));
     if (per_sm < 1) return fail(l, CL_EINVAL, "ensemble pass does not fit on an SM");
-    const int wave = per_sm * nsm;
-    std::vector<int> first;
-    const int min_planes = l->opt_DZ > 0 ? kEnsMaxN : kEnsMinPlanes;  // CL_OPT_TILE_DZ's chunks stay as they are
-    double lo = 0.0, hi = 0.0;  // hi: one block takes everything
-    for (const EnsColumn& c : cols) hi += ((double)c.planes + kEnsExtra + 1.0) * (double)c.row;
-    for (int i = 0; i < 60 && hi - lo > 1.0; ++i) {
-        const double mid = 0.5 * (lo + hi);
-        const int n = ens_cut(cols, mid, min_planes, nullptr, nullptr);
-        if (n > 0 && n <= wave) hi = mid;
-        else lo = mid;
-    }
-    ens_cut(cols, hi, min_planes, &l->hitems, &first);
-    l->ens_grid = (int)first.size() - 1;
+    const double beside = stages == 0 && prec != CL_PREC_FP64 ? 0.1 : 0.45;
+    EnsPlan plan = ens_plan(cols, per_sm * nsm, nsm, beside, l->opt_DZ <= 0);
+    l->hitems = std::move(plan.items);
+    l->ens_grid = plan.blocks();
     l->nitems = (int)l->hitems.size();
     for (int i = l->nitems - 1; i >= 0; --i) {  // a member's items are consecutive
         EnsMember& M = l->hmem[l->hitems[i].member];
@@ -375,19 +445,22 @@ cl_status ens_tiles(cl_lattice* l)
     }
     if (l->d_items) cudaFree(l->d_items);
     l->d_items = nullptr;
-    if (l->d_first) cudaFree(l->d_first);
-    l->d_first = nullptr;
+    if (l->d_sched) cudaFree(l->d_sched);
+    l->d_sched = nullptr;
     if (!l->d_members && !dev_alloc(l, &l->d_members, sizeof(EnsMember) * B))
         return fail(l, CL_ENOMEM, "cannot allocate the member table");
     if (!dev_alloc(l, &l->d_items, sizeof(EnsItem) * l->hitems.size()))
         return fail(l, CL_ENOMEM, "cannot allocate the item table");
     CUDA_TRY(l, cudaMemcpy(l->d_items, l->hitems.data(), sizeof(EnsItem) * l->hitems.size(), cudaMemcpyHostToDevice));
-    if (!dev_alloc(l, &l->d_first, sizeof(int) * first.size()))
+    // the blocks' lists: where each begins (ens_grid + 1 numbers), then the items
+    std::vector<int> lists = std::move(plan.first);
+    lists.insert(lists.end(), plan.sched.begin(), plan.sched.end());
+    if (!dev_alloc(l, &l->d_sched, sizeof(int) * lists.size()))
         return fail(l, CL_ENOMEM, "cannot allocate the item schedule");
-    CUDA_TRY(l, cudaMemcpy(l->d_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(l, cudaMemcpy(l->d_sched, lists.data(), sizeof(int) * lists.size(), cudaMemcpyHostToDevice));
     cl_status s = upload_members(l);
     if (s != CL_OK) return s;
-    s = grow_partials(l, l->nitems);
+    s = grow_partials(l, units);
     if (s != CL_OK) return s;
     invalidate_graphs(l);
     return CL_OK;
@@ -907,7 +980,8 @@ cl_status run_ens_pass_t(cl_lattice* l, const PassCoef& pc, int in, int out, int
     }
     A.members = l->d_members;
     A.items = l->d_items;
-    A.first = (m0 == 0 && m1 == l->members) ? l->d_first : nullptr;  // whole passes: the blocks' runs
+    A.first = (m0 == 0 && m1 == l->members) ? l->d_sched : nullptr;  // whole passes: the blocks' lists
+    A.sched = A.first ? A.first + l->ens_grid + 1 : nullptr;
     A.scal = l->scal;
     A.partials = l->partials;
     A.item_begin = l->hmem[m0].item0;
@@ -1548,7 +1622,7 @@ void cl_free(cl_lattice* l)
     l->spec.release();
     if (l->d_members) cudaFree(l->d_members);
     if (l->d_items) cudaFree(l->d_items);
-    if (l->d_first) cudaFree(l->d_first);
+    if (l->d_sched) cudaFree(l->d_sched);
     if (l->own_stream && l->stream) cudaStreamDestroy(l->stream);
     delete l;
 }

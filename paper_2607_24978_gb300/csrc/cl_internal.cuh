@@ -286,13 +286,19 @@ cudaError_t u1_fused_blocks_per_sm(int precision, int* blocks);
 
 // Batched ensemble of independent lattices (ensemble_pass.cu).  Every array class (phi,
 // pi, compensation, per field and buffer) is one arena holding the members back to back,
-// each starting on a 256-byte boundary.  A work item is BY full x rows times DZ planes of
+// each starting on a 256-byte boundary.  A work item is BY full x rows times some planes of
 // one member; items of a member are consecutive in the item table.
+// A member's sums are made of units: what one warp's threads add over one chunk of CZ planes of one
+// tile of rows.  Items begin and end at chunk boundaries, and tiles, chunks, units and the order in
+// which a member's units are added follow from its own N, so how items are cut and dealt out to
+// blocks, which depends on all members, changes no bit of a member's a, a' and energies.
 constexpr int kEnsThreads = 256;
 struct EnsMember {
     long long off;       // element offset of the member's arrays in every arena
-    int N, BY, DZ;       // sites per side and the tile of one work item
+    int N, BY, DZ;       // sites per side, the rows of a tile, the most planes of a work item
     int item0, nitems;   // the member's work items [item0, item0 + nitems)
+    int CZ, nkz;         // planes of a chunk, chunks of a tile
+    int unit0, nunits;   // the member's units: tile, chunk, warp
     double dx;
     double m2[2], lam[2], g2;
 };
@@ -309,10 +315,10 @@ struct EnsPassArgs {
     T* c_out[2];
     const EnsMember* members;
     const EnsItem* items;
-    const int* first;     // block b takes items first[b] .. first[b + 1] - 1 (nullptr: the items
-                          // item_begin + b, + grid, ... below item_end)
+    const int* sched;     // block b takes items sched[first[b]] .. sched[first[b + 1] - 1] (first
+    const int* first;     // nullptr: the items item_begin + b, + grid, ... below item_end)
     DevScal* scal;        // one per member
-    double* partials;     // [items][kMaxQ]
+    double* partials;     // [units][kMaxQ]
     int item_begin, item_end;
     double alpha, kappa;
     double d, e, k;       // pass coefficients (already x dt), as in ScalarPassArgs

@@ -2,15 +2,16 @@
 //
 // Many small lattices (each with its own size, box, couplings, a and a') advance by one
 // pass of the staggered kick-drift scheme in a single persistent launch.  The work is a
-// table of items, each BY full x rows times some planes of one member; block b takes a run of
-// consecutive items (the library cuts the members' columns of planes so that every block has the
-// same work) and runs the same per-site arithmetic as the single-lattice direct loader on it
-// (drift while loading, stencil kick, energies).
-// Reductions: every item writes its FP64 partial sums; the block that completes the last
-// item of a member (an arrival counter per member) sums that member's partials in a fixed
-// order and runs the member's scale-factor epilogue.  Reading a, a' happens at item
+// table of items, each BY full x rows times some planes of one member; block b takes a list of
+// items (see ens_tiles) and runs the same per-site arithmetic as the single-lattice direct loader
+// on them (drift while loading, stencil kick, energies).
+// Reductions: every warp writes its FP64 sums of each chunk of planes (EnsMember); the block that
+// completes the last item of a member (an arrival counter per member) adds that member's sums in a
+// fixed order and runs the member's scale-factor epilogue.  Reading a, a' happens at item
 // start, before the item's arrival, so the epilogue never races a reader.
 #include <math.h>
+
+#include <type_traits>
 
 #include "cl_internal.cuh"
 #include "kernel_common.cuh"
@@ -19,16 +20,91 @@
 
 namespace clk {
 
-// Items of this block: it, it + step, ... below end.
+// Items of this block: item(k), k = it, it + step, ... below end.
 struct EnsRange {
+    const int* sched;
     int it, end, step;
     template <typename A_>
     __device__ __forceinline__ explicit EnsRange(const A_& A)
-        : it(A.first ? A.first[blockIdx.x] : A.item_begin + (int)blockIdx.x),
+        : sched(A.first ? A.sched : nullptr), it(A.first ? A.first[blockIdx.x] : A.item_begin + (int)blockIdx.x),
           end(A.first ? A.first[blockIdx.x + 1] : A.item_end), step(A.first ? 1 : (int)gridDim.x)
     {
     }
+    __device__ __forceinline__ int item(int k) const { return sched ? sched[k] : k; }
 };
+
+// The sums of this warp's chunks of an item: one unit a chunk, written when the chunk's last plane
+// has been kicked (all lanes call chunk_done()).
+template <typename T, int NF>
+struct EnsSums {
+    Acc<T> K[NF], G[NF], V;
+    double* row;           // the warp's unit of the current chunk
+    __device__ __forceinline__ EnsSums(double* partials, const EnsMember& M, const EnsItem& I, int warp)
+        : row(partials + (size_t)kMaxQ * (M.unit0 + (I.y0 / M.BY * M.nkz + I.z0 / M.CZ) * (kEnsThreads / 32) + warp))
+    {
+    }
+    __device__ __forceinline__ void chunk_done(int lane)
+    {
+        typename std::conditional<sizeof(T) == 4, F2, double>::type v[kMaxQ];
+        const Acc<T>* const acc[kMaxQ] = {&K[0], NF > 1 ? &K[NF - 1] : nullptr, &G[0], NF > 1 ? &G[NF - 1] : nullptr, &V};
+#pragma unroll
+        for (int q = 0; q < kMaxQ; ++q) {
+            if constexpr (sizeof(T) == 4) v[q] = acc[q] ? F2{acc[q]->s, -acc[q]->c} : F2{0.f, 0.f};
+            else v[q] = acc[q] ? acc[q]->value() : 0.0;
+        }
+        const auto x = warp_sums<kMaxQ>(v, lane);
+#pragma unroll
+        for (int q = 0; q < kMaxQ; ++q)
+            if (lane == warp_sum_lane<kMaxQ>(q)) {
+                if constexpr (sizeof(T) == 4) *reinterpret_cast<float2*>(&row[q]) = make_float2(x.hi, x.lo);
+                else row[q] = x;
+            }
+        row += (kEnsThreads / 32) * kMaxQ;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) K[f] = G[f] = Acc<T>();
+        V = Acc<T>();
+    }
+};
+
+// End of an item, by the kEnsThreads consumers, whose barrier is sync(): the block that finds every
+// item of the member done adds its units and runs its epilogue.
+template <typename T, typename Sync>
+__device__ __forceinline__ void ens_item_done(const EnsPassArgs<T>& A, const EnsMember& M, DevScal* S, double a,
+                                              double (*s_red)[kMaxQ], int* s_last, int tid, Sync sync)
+{
+    sync();  // every warp has written its units
+    if (tid == 0) {
+        __threadfence();
+        const unsigned prev = atomicAdd(&S->counter, 1u);
+        *s_last = (prev + 1u == (unsigned)M.nitems);
+    }
+    sync();
+    if (*s_last) {
+        __threadfence();
+        double w[kMaxQ] = {};
+        for (int u = tid; u < M.nunits; u += kEnsThreads) {
+            const double* row = A.partials + (size_t)kMaxQ * (M.unit0 + u);
+#pragma unroll
+            for (int q = 0; q < kMaxQ; ++q) {
+                if constexpr (sizeof(T) == 4) {
+                    const float2 x = __ldcg(reinterpret_cast<const float2*>(row + q));
+                    w[q] += (double)x.x + (double)x.y;
+                } else {
+                    w[q] += __ldcg(row + q);
+                }
+            }
+        }
+        warp_sums_to<kMaxQ>(w, s_red, tid >> 5, tid & 31);
+        sync();
+        if (tid < 32) {
+            sum_rows<kMaxQ>(w, s_red, kEnsThreads / 32, tid);
+            if (tid == 0)
+                scalar_epilogue(S, w, (double)M.N * M.N * M.N, M.dx, a, A.alpha, A.kappa, A.d, A.e, A.k, A.flags,
+                                A.hubble_limit);
+        }
+    }
+    sync();  // the prefactors, s_red and s_last are rewritten by the next item
+}
 
 template <typename T, int NF, bool KAHAN, int VW>
 __global__ void __launch_bounds__(kEnsThreads) k_ensemble_pass(const EnsPassArgs<T> A)
@@ -43,8 +119,8 @@ __global__ void __launch_bounds__(kEnsThreads) k_ensemble_pass(const EnsPassArgs
     const bool expand = (A.flags & P_EXPANSION) != 0;
 
     const EnsRange W(A);
-    for (int it = W.it; it < W.end; it += W.step) {
-        const EnsItem I = A.items[it];
+    for (int k = W.it; k < W.end; k += W.step) {
+        const EnsItem I = A.items[W.item(k)];
         const EnsMember& M = A.members[I.member];
         const int N = M.N, BY = M.BY;
         const double dx = M.dx;
@@ -64,31 +140,11 @@ __global__ void __launch_bounds__(kEnsThreads) k_ensemble_pass(const EnsPassArgs
             F.pi_out[f] = A.pi_out[f] + off;
             F.c_out[f] = KAHAN ? A.c_out[f] + off : nullptr;
         }
-        Acc<T> accK[NF], accG[NF], accV;
-        const int R = min(BY, N - I.y0), NZ = I.nz;
-        march_tile<T, NF, KAHAN, VW>(F, N, BY, I.y0, R, I.z0, NZ, sm, tid, nthr, do_drift, C, P, accK, accG, accV);
-
-        double v[kMaxQ];
-        const Acc<T>* av[kMaxQ] = {&accK[0], NF > 1 ? &accK[NF - 1] : nullptr, &accG[0],
-                                   NF > 1 ? &accG[NF - 1] : nullptr, &accV};
-        block_reduce_acc<T, kMaxQ>(av, v, s_red, tid, nthr);
-        if (tid == 0) {
-#pragma unroll
-            for (int q = 0; q < kMaxQ; ++q) A.partials[(size_t)it * kMaxQ + q] = v[q];
-            __threadfence();
-            const unsigned prev = atomicAdd(&S->counter, 1u);
-            s_last = (prev + 1u == (unsigned)M.nitems);
-        }
-        __syncthreads();
-        if (s_last && tid < 32) {  // block-uniform; one warp sums the member's item partials
-            __threadfence();
-            double w[kMaxQ];
-            warp_sum_partials<kMaxQ>(A.partials + (size_t)M.item0 * kMaxQ, M.nitems, tid, w);
-            if (tid == 0)
-                scalar_epilogue(S, w, (double)N * N * N, dx, s_coef[3], A.alpha, A.kappa, A.d, A.e, A.k, A.flags,
-                                A.hubble_limit);
-        }
-        __syncthreads();  // s_coef and s_last are rewritten by the next item
+        EnsSums<T, NF> sums(A.partials, M, I, tid >> 5);
+        const int R = min(BY, N - I.y0);
+        march_tile<T, NF, KAHAN, VW>(F, N, BY, I.y0, R, I.z0, I.nz, sm, tid, nthr, do_drift, C, P, sums.K, sums.G, sums.V,
+                                     nullptr, M.CZ, [&] { sums.chunk_done(tid & 31); });
+        ens_item_done(A, M, S, s_coef[3], s_red, &s_last, tid, [] { __syncthreads(); });
     }
 }
 
@@ -142,8 +198,8 @@ __global__ void __launch_bounds__(kEnsTmaThreads, NF == 1 ? 2 : 1) k_ensemble_pa
         uint32_t empty_phase = 0;
         int issued = 0;
         const EnsRange W(A);
-        for (int it = W.it; it < W.end; it += W.step) {
-            const EnsItem I = A.items[it];
+        for (int k = W.it; k < W.end; k += W.step) {
+            const EnsItem I = A.items[W.item(k)];
             const EnsMember& M = A.members[I.member];
             const int N = M.N, BY = M.BY, y0 = I.y0, z0 = I.z0;
             const int R = min(BY, N - y0), NZ = I.nz;
@@ -188,8 +244,8 @@ __global__ void __launch_bounds__(kEnsTmaThreads, NF == 1 ? 2 : 1) k_ensemble_pa
         };
         ZMarch<T, NF, VW> Z;
         const EnsRange W(A);
-        for (int it = W.it; it < W.end; it += W.step) {
-            const EnsItem I = A.items[it];
+        for (int k = W.it; k < W.end; k += W.step) {
+            const EnsItem I = A.items[W.item(k)];
             const EnsMember& M = A.members[I.member];
             const int N = M.N, BY = M.BY, y0 = I.y0, z0 = I.z0;
             const int R = min(BY, N - y0), NZ = I.nz;
@@ -203,55 +259,38 @@ __global__ void __launch_bounds__(kEnsTmaThreads, NF == 1 ? 2 : 1) k_ensemble_pa
             const TileGeom G(N, VW, BY, R, tid);
             const size_t plane = (size_t)N * N;
             const size_t row_off = (size_t)(y0 + G.r) * N + G.x0;
-            Acc<T> accK[NF], accG[NF], accV;
+            EnsSums<T, NF> sums(A.partials, M, I, tid >> 5);
             int zz = z0 == 0 ? N - 1 : z0 - 1;
-            for (int j = 0; j < NZ + 2; ++j) {
-                if (!mbar_wait_bounded(&s_full[st], (full_phase >> st) & 1u, s_timeout ? 1000000ull : 2000000000ull))
-                    s_timeout = 1;
-                full_phase ^= 1u << st;
-                if constexpr (NR) {
-                    tma_consume_plane_nr<T, NF, KAHAN, VW>(G, stage + st * A.stage_stride,
-                                                           stage + st_prev * A.stage_stride, do_drift,
-                                                           j >= 1 && j <= NZ, j >= 2, (size_t)zz * plane + row_off,
-                                                           (size_t)(z0 + j - 2) * plane + row_off, Out, C, P, Z, accK,
-                                                           accG, accV);
-                    if (j >= 1) release(st_prev);  // plane j-1: kicked (or the lower z halo, never kicked)
-                } else {
-                    tma_consume_plane<T, NF, KAHAN, VW>(G, stage + st * A.stage_stride, ring + rnew * A.ring_slot,
-                                                        ring + rmid * A.ring_slot, tid, CT, do_drift,
-                                                        j >= 1 && j <= NZ, j >= 2, (size_t)zz * plane + row_off,
-                                                        (size_t)(z0 + j - 2) * plane + row_off, Out, C, P, Z, accK,
-                                                        accG, accV, &s_empty[st]);
-                    rmid = rnew;
-                    rnew = rnew + 1 == RING ? 0 : rnew + 1;
+            // plane j - 2 of the item is kicked in turn j: a chunk's last one in turn end - 1
+            for (int j = 0, end = min(NZ, M.CZ) + 2; j < NZ + 2; end = min(NZ + 2, end + M.CZ)) {
+                for (; j < end; ++j) {
+                    if (!mbar_wait_bounded(&s_full[st], (full_phase >> st) & 1u, s_timeout ? 1000000ull : 2000000000ull))
+                        s_timeout = 1;
+                    full_phase ^= 1u << st;
+                    if constexpr (NR) {
+                        tma_consume_plane_nr<T, NF, KAHAN, VW>(G, stage + st * A.stage_stride,
+                                                               stage + st_prev * A.stage_stride, do_drift,
+                                                               j >= 1 && j <= NZ, j >= 2, (size_t)zz * plane + row_off,
+                                                               (size_t)(z0 + j - 2) * plane + row_off, Out, C, P, Z, sums.K,
+                                                               sums.G, sums.V);
+                        if (j >= 1) release(st_prev);  // plane j-1: kicked (or the lower z halo, never kicked)
+                    } else {
+                        tma_consume_plane<T, NF, KAHAN, VW>(G, stage + st * A.stage_stride, ring + rnew * A.ring_slot,
+                                                            ring + rmid * A.ring_slot, tid, CT, do_drift,
+                                                            j >= 1 && j <= NZ, j >= 2, (size_t)zz * plane + row_off,
+                                                            (size_t)(z0 + j - 2) * plane + row_off, Out, C, P, Z, sums.K,
+                                                            sums.G, sums.V, &s_empty[st]);
+                        rmid = rnew;
+                        rnew = rnew + 1 == RING ? 0 : rnew + 1;
+                    }
+                    st_prev = st;
+                    st = st + 1 == S ? 0 : st + 1;
+                    zz = zz + 1 == N ? 0 : zz + 1;
                 }
-                st_prev = st;
-                st = st + 1 == S ? 0 : st + 1;
-                zz = zz + 1 == N ? 0 : zz + 1;
+                sums.chunk_done(lane);
             }
             if constexpr (NR) release(st_prev);  // the upper z halo of the item is never kicked
-            // item partials; the member's last item reduces them in a fixed order
-            double v[kMaxQ];
-            const Acc<T>* av[kMaxQ] = {&accK[0], NF > 1 ? &accK[NF - 1] : nullptr, &accG[0],
-                                       NF > 1 ? &accG[NF - 1] : nullptr, &accV};
-            group_reduce_acc<T, kMaxQ>(av, v, s_red, tid, CT, 2);
-            if (tid == 0) {
-#pragma unroll
-                for (int q = 0; q < kMaxQ; ++q) A.partials[(size_t)it * kMaxQ + q] = v[q];
-                __threadfence();
-                const unsigned prev = atomicAdd(&Sm->counter, 1u);
-                s_last = (prev + 1u == (unsigned)M.nitems);
-            }
-            named_barrier_sync(2, CT);
-            if (s_last && tid < 32) {  // uniform over the consumers; one warp sums the item partials
-                __threadfence();
-                double w[kMaxQ];
-                warp_sum_partials<kMaxQ>(A.partials + (size_t)M.item0 * kMaxQ, M.nitems, tid, w);
-                if (tid == 0)
-                    scalar_epilogue(Sm, w, (double)N * N * N, dx, s_coef[3], A.alpha, A.kappa, A.d, A.e, A.k, A.flags,
-                                    A.hubble_limit);
-            }
-            named_barrier_sync(2, CT);  // s_coef, s_red and s_last are rewritten by the next item
+            ens_item_done(A, M, Sm, s_coef[3], s_red, &s_last, tid, [] { named_barrier_sync(2, CT); });
         }
     }
     __syncthreads();  // producer and consumers meet; no copy is in flight past this point

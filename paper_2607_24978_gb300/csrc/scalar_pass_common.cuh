@@ -6,6 +6,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "cl_internal.cuh"
 #include "kernel_common.cuh"
 
@@ -247,12 +249,15 @@ struct TileCoef {
 // x 3 slots x (BY+2) rows x N) holds the drifted field of the planes below, at and above
 // the plane being kicked; thread tid < BY*(N/VW) owns one row vector.  Every output is
 // written once; loads of the halo rows (and planes) are the only re-reads.  Ends with a
-// block barrier, so the ring may be refilled at once.
-template <typename T, int NF, bool KAHAN, int VW, bool SBP = false>
+// block barrier, so the ring may be refilled at once.  All threads call done() after every `chunk`
+// planes and the last one (if Done is not NoChunks).
+struct NoChunks {
+};
+template <typename T, int NF, bool KAHAN, int VW, bool SBP = false, typename Done = NoChunks>
 __device__ __forceinline__ void march_tile(const FieldSet<T>& F, int N, int BY, int y0, int R, int z0, int NZ,
                                            T* sm, int tid, int nthr, bool do_drift, const TileCoef<T>& C,
                                            const PotCoef<T>& P, Acc<T> (&accK)[NF], Acc<T> (&accG)[NF],
-                                           Acc<T>& accV, const T* gC = nullptr)
+                                           Acc<T>& accV, const T* gC = nullptr, int chunk = 0, Done done = Done())
 {
     const int TX = N / VW;
     const int r = tid < BY * TX ? tid / TX : BY, tx = tid < BY * TX ? tid % TX : 0;
@@ -307,7 +312,7 @@ __device__ __forceinline__ void march_tile(const FieldSet<T>& F, int N, int BY, 
     T pcur[NF][VW], pnext[NF][VW];
     fill(-1, 0, false, pnext);
     fill(0, 1, true, pcur);
-    for (int zr = 0; zr < NZ; ++zr) {
+    auto plane = [&](int zr) {
         const int sl = zr % 3, sc = (zr + 1) % 3, su = (zr + 2) % 3;
         fill(zr + 1, su, zr + 1 < NZ, pnext);
         __syncthreads();
@@ -330,6 +335,14 @@ __device__ __forceinline__ void march_tile(const FieldSet<T>& F, int N, int BY, 
 #pragma unroll
             for (int i = 0; i < VW; ++i) pcur[f][i] = pnext[f][i];
         __syncthreads();
+    };
+    if constexpr (std::is_same<Done, NoChunks>::value) {
+        for (int zr = 0; zr < NZ; ++zr) plane(zr);
+    } else {
+        for (int zr = 0; zr < NZ;) {
+            for (const int end = min(NZ, zr + chunk); zr < end; ++zr) plane(zr);
+            done();
+        }
     }
 }
 

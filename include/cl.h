@@ -375,11 +375,13 @@ cl_status cl_set_hubble_limit(cl_lattice* l, double limit);
  * drifted rows in registers; CL_OPT_TILE_DZ its rows per chunk, CL_OPT_TILE_BY how many rows
  * ahead it prefetches into L2, 0 = library choice) or 0 = one thread per site; both agree to
  * rounding.
- * A small scalar lattice (up to 1.75e6 to 3e6 sites in FP32, 4e5 to 1e6 in FP64, by fields, compensation
+ * A small scalar lattice (up to 1.75e6 to 3e6 sites in FP32, 3e5 to 9e5 in FP64, by fields, compensation
  * and alignment) takes the leapfrog steps of a cl_step call in resident launches of many passes
  * each, unless the caller set one of the tiling options (the library's choices that cl_get_option
- * reports then still serve the passes outside cl_step).  Such steps replay no graph: CL_OPT_GRAPH has
- * no effect on them.  Setting an option back to its library choice, or cl_autotune, ends the
+ * reports then still serve the passes outside cl_step) or the call has too few passes to gain by it
+ * (one; up to three on the larger of these lattices).  Such steps replay no graph: CL_OPT_GRAPH has
+ * no effect on them.  Both forms agree to rounding, so above 40^3 sites, as among tilings, how a run
+ * is divided into calls of so few steps can change its last bits.  Setting an option back to its library choice, or cl_autotune, ends the
  * caller's choice.
  * Errors: CL_EINVAL, CL_EUNSUPPORTED. */
 enum { CL_OPT_GRAPH = 0, CL_OPT_TILE_BY = 1, CL_OPT_TILE_DZ = 2, CL_OPT_STAGES = 3, CL_OPT_PASS_VARIANT = 4 };

@@ -476,13 +476,24 @@ bool u1_staged_pays(int N) { return N % 32 == 0 || N >= 36; }
 // at 136^3; two fields: 31.8 / 30.2 at 120^3, 32.3 / 34.4 at 124^3; rows of other alignment, whose
 // staged kernel is slower: 45.1 / 43.8 at 131^3 and 46.6 / 48.4 at 135^3 (two fields).  Plain FP32:
 // 24.9 / 22.1 at 144^3 (one field), 40.5 / 30.3 at 131^3 (two).  FP64, where both are bound by the
-// FP64 pipe and the repeated drifts count: 67.8 / 66.5 at 100^3 (one field), 63.5 / 62.3 at 72^3 (two).
+// FP64 pipe and the repeated drifts count: 65.7 / 60.0 at 96^3 and 65.7 / 66.5 at 100^3 (one field),
+// 47.2 / 45.9 at 64^3 and 61.6 / 62.3 at 72^3 (two).
 int64_t persist_max_sites(const cl_lattice* l)
 {
-    if (is_fp64(l)) return l->nf == 1 ? 1000000 : 400000;
+    if (is_fp64(l)) return l->nf == 1 ? 900000 : 300000;
     if (!has_kahan(l)) return l->nf == 1 ? 3000000 : 2300000;
     if (l->VW * l->es != 16) return 2250000;
     return l->nf == 1 ? 2150000 : 1750000;
+}
+
+// The fewest passes of a cl_step call that go to resident launches: these take 12 to 16 us more than
+// their passes (prefactors before the first, energies after the last), and gain the less on each the
+// nearer a lattice is to the sizes above.  Measured (us a call, per-pass kernel / resident, FP32 +
+// Kahan): one pass 16.5 / 16.8 at 40^3, 16.5 / 20.7 at 48^3, 24.7 / 37 at 128^3; two 41.2 / 39.3 at
+// 100^3; two and three at 128^3 49.4 / 55.6 and 74 / 76; two fields at 100^3 49.4 / 53.8 and 74 / 73.
+int persist_min_passes(const cl_lattice* l)
+{
+    return l->V <= 64000 ? 1 : 2 + (int)(2 * l->V / persist_max_sites(l));
 }
 
 cl_status choose_tiles(cl_lattice* l)
@@ -2375,7 +2386,7 @@ cl_status cl_step(cl_lattice* l, int32_t nsteps)
     // the fused stages leave R of the final state behind; stages with a reduction launch leave
     // that of their last input state
     l->rbar_valid = nmc_f;
-    if (l->ps_grid > 0) {
+    if (l->ps_grid > 0 && (int64_t)pps * nsteps >= persist_min_passes(l)) {
         int done = 0;
         cl_status s = is_fp64(l) ? run_persist_t<double>(l, sched, nsteps, &done) : run_persist_t<float>(l, sched, nsteps, &done);
         if (s != CL_OK) return s;

@@ -71,3 +71,28 @@ def test_the_librarys_tiling_matches_the_oracle(cl, N, prec, tol):
 def test_resident_launches_at_their_largest_sizes(cl, N, nf, prec):
     a, b = (run(cl, N, nf, prec, cl.CL_INT_YOSHIDA4, (2, 1), r) for r in (True, False))
     check(a, b, prec)
+
+
+# calls of one and of a few passes on lattices that take longer ones in resident launches: the same
+# bits as with a tiling option set, where the call launches every pass
+@pytest.mark.parametrize("N,nf,prec,passes", [(41, 1, 1, 1), (64, 2, 1, 1), (96, 1, 0, 1), (100, 2, 1, 2), (125, 1, 1, 2)])
+def test_calls_of_few_passes_are_launched_one_by_one(cl, N, nf, prec, passes):
+    phi, pi = inputs.scalar_state(N, nf, seed=5, fbar=(1.0, 0.1), amp=0.05, pamp=0.05)
+    dtype = np.float64 if prec == 0 else np.float32
+    outs = []
+    for tiled, calls in ((False, [passes] * 4), (True, [passes] * 4), (False, [4 * passes])):
+        with cl.Lattice(N, 0.4 * N, nf, prec, cl.CL_INT_VV2, expansion=True, alpha=0.3, kappa=0.2, dt=0.01) as g:
+            g.cl_set_potential(cl.CL_POT_POLY, [0.5, 1.0] + ([0.2, 0.4, 3.0] if nf == 2 else [0.0] * 3))
+            if tiled:
+                g.cl_set_option(cl.CL_OPT_TILE_BY, g.cl_get_option(cl.CL_OPT_TILE_BY))
+            for f in range(nf):
+                g.cl_set_state(cl.CL_FIELD_PHI0 + f, phi[f].astype(dtype))
+                g.cl_set_state(cl.CL_FIELD_PI0 + f, pi[f].astype(dtype))
+            g.cl_set_scalars(1.0)
+            for n in calls:
+                g.cl_step(n)
+            outs.append(g.cl_energies())
+    assert outs[0] == outs[1]
+    for k in ("a", "adot", "rho"):
+        assert outs[0][k] == pytest.approx(outs[2][k], rel=1e-7 if prec else 1e-11)
+    assert outs[0] != outs[2]  # the longer call is a resident one: its sums have another order

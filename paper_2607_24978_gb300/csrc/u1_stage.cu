@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
             const T Pm = ca * A.E_in[i][nm] + gh * (A.phi_in[nm] * Bm + A.phi_in[n] * Bn);
             G += Pn - Pm;
             sc += fabs(Pn) + fabs(Pm);
-            ee += A.E_in[i][n] * A.E_in[i][n];
+            if (mode == 1) ee += A.E_in[i][n] * A.E_in[i][n];
         }
         gmx = fmax(gmx, fabs(G));
         smx = fmax(smx, sc);

@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(kEnsTmaThreads, NF == 1 ? 2 : 1) k_ensemble_pa
                 zz = zz + 1 == N ? 0 : zz + 1;
             }
         }
+        if (!copies_landed(s_full, S, issued, s_timeout != 0)) s_timeout = 1;
     } else {
         int st = 0, st_prev = 0;
         uint32_t full_phase = 0;

@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(480, 1) k_gw_pass_tma(const GwPassArgs<float> 
                 zz = zz + 1 == N ? 0 : zz + 1;
             }
         }
+        if (!copies_landed(s_full, S, issued, s_timeout != 0)) s_timeout = 1;
     } else {
         using P2 = Two;
         const bool do_drift = (A.flags & P_DRIFT) != 0;

@@ -490,4 +490,17 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     }
 }
 
+// Whether the copies of a producer's `issued` planes, into S stages in turn, have landed: those still
+// under way when it has issued the last one, each waited for within the limit (hurry: a wait of the
+// block has given up before).  A block must not end before they have, whatever its consumers did.
+__device__ __forceinline__ bool copies_landed(uint64_t* full, int S, int issued, bool hurry)
+{
+    bool ok = true;
+    for (int s = 0; s < S && s < issued; ++s) {
+        const int uses = (issued - s + S - 1) / S;
+        ok = mbar_wait_bounded(&full[s], (uint32_t)(uses - 1) & 1u, hurry ? 1000000ull : 2000000000ull) && ok;
+    }
+    return ok;
+}
+
 }  // namespace clk

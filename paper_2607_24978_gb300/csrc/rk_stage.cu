@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(480, 1) k_rk_stage_tma(const RkStageArgs<T> A)
                 zz = zz + 1 == N ? 0 : zz + 1;
             }
         }
+        if (!copies_landed(s_full, S, issued, s_timeout != 0)) s_timeout = 1;
     } else {
         // ---------------------------------------------------------------- consumer warps
         // the stage's prefactors, lanes side by side, beside the copies of the first planes (before

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(512, 1) k_scalar_pass_tma(const ScalarPassArgs
                 zz = zz + 1 == N ? 0 : zz + 1;
             }
         }
+        if (!copies_landed(s_full, S, issued, s_timeout != 0)) s_timeout = 1;
     } else {
         // ---------------------------------------------------------------- consumer warps
         const T cd = (T)s_coef[0], cL = (T)s_coef[1], cV = (T)s_coef[2];

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_any(const ScalarPass
                 zz = zz + 1 == N ? 0 : zz + 1;
             }
         }
+        if (!copies_landed(s_full, S, issued, s_timeout != 0)) s_timeout = 1;
     } else {
         constexpr int CP = CH / 2;  // pairs of sites (k = 2 i, 2 i + 1)
         consumer_coefficients(tid, CT, A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);

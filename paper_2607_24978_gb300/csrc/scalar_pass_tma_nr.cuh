@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(480, 1) k_scalar_pass_tma_nr(const ScalarPassA
                 zz = zz + 1 == N ? 0 : zz + 1;
             }
         }
+        if (!copies_landed(s_full, S, issued, s_timeout != 0)) s_timeout = 1;
     } else {
         // ---------------------------------------------------------------- consumer warps
         consumer_coefficients(tid, CT, A.scal->a, A.scal->b, A.d, A.alpha, A.dx, (A.flags & P_EXPANSION) != 0, s_coef);

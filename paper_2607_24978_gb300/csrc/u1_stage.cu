@@ -311,11 +311,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_u1_stage(const 
 }
 
 // Lattice Gauss charge G(n) = sum_i [P_i(n) - P_i(n - i)] / dx, P = a^(1-alpha) E + g W.
-// mode 0 writes diag[D_GV] = max_n |G(n)| / max_n sum_i (|P_i(n)| + |P_i(n - i)|) / dx;
-// mode 1 (per-step tracking, for the launch forms whose stage does not sum it itself) the
+// MODE 0 writes diag[D_GV] = max_n |G(n)| / max_n sum_i (|P_i(n)| + |P_i(n - i)|) / dx;
+// MODE 1 (per-step tracking, for the launch forms whose stage does not sum it itself) the
 // rms violation sqrt(sum_n (dx G)^2) / (a^(1-alpha) sqrt(sum_n E^2)) into DevScal::gauss.
-template <typename T>
-__global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
+// Bound by the latency of its gathers: 64 registers (four blocks an SM) keep more loads in flight than
+// the compiler's own 40 (192^3 98 against 161 us, 125^3 36 and 44; 80 registers 36 at 125^3).
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256, 4) k_u1_gauss(const U1Args<T> A)
 {
     __shared__ double s_red[32][kMaxQ];
     __shared__ int s_last;
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
     const int tid = threadIdx.x, nthr = blockDim.x;
     // per-site arithmetic and maxima in the field precision (two FP64 divisions, conversions and
     // additions a site made 440 us at 192^3 and 92 us at 100^3 of this launch on GB300's FP64 pipe);
-    // the squares and sums of mode 1 in FP64: G is what cancellation leaves of E, and its FP32
+    // the squares and sums of MODE 1 in FP64: G is what cancellation leaves of E, and its FP32
     // square vanishes where that of E does not
     const T ca = (T)apow(A.scal->a, 1.0 - A.alpha);
     const T b4 = (T)(0.25 / (A.dx * A.dx)), gh = (T)(0.5 * A.g);
@@ -346,16 +348,16 @@ __global__ void __launch_bounds__(256) k_u1_gauss(const U1Args<T> A, int mode)
             const T Pm = ca * A.E_in[i][nm] + gh * (A.phi_in[nm] * Bm + A.phi_in[n] * Bn);
             G += Pn - Pm;
             sc += fabs(Pn) + fabs(Pm);
-            if (mode == 1) ee += A.E_in[i][n] * A.E_in[i][n];
+            if (MODE == 1) ee += A.E_in[i][n] * A.E_in[i][n];
         }
         gmx = fmax(gmx, fabs(G));
         smx = fmax(smx, sc);
-        if (mode == 1) {
+        if (MODE == 1) {
             gsq = fma((double)G, (double)G, gsq);
             e2 += (double)ee;
         }
     }
-    if (mode == 1) {  // sums in a fixed order, then the last block stores the tracked value
+    if constexpr (MODE == 1) {  // sums in a fixed order, then the last block stores the tracked value
         double v[2] = {gsq, e2};
         block_reduce<2>(v, s_red, tid, nthr);
         if (tid == 0) {
@@ -439,7 +441,8 @@ static cudaError_t launch_u1_t(const U1Args<T>& A, int what, cudaStream_t s)
     const int grid = u1_grid(A.N, A.dz);
     if (what == 0) k_u1_plaquettes<T><<<grid, 256, 0, s>>>(A);
     else if (what == 1) k_u1_stage<T><<<grid, 256, 0, s>>>(A);
-    else k_u1_gauss<T><<<grid, 256, 0, s>>>(A, what == 3 ? 1 : 0);
+    else if (what == 3) k_u1_gauss<T, 1><<<grid, 256, 0, s>>>(A);
+    else k_u1_gauss<T, 0><<<grid, 256, 0, s>>>(A);
     return cudaGetLastError();
 }
 

@@ -146,7 +146,7 @@ __host__ __device__ constexpr int any_own_region(int N, int BY)
 
 // Many fused passes in one cooperative launch, for small lattices (scalar_persist.cu).
 constexpr int kPersistSched = 81;      // passes of the longest composition's step (Yoshida-10)
-constexpr int kPersistPasses = 2048;   // passes a launch runs at most (about 10 ms)
+constexpr int kPersistPasses = 2048;   // passes a launch runs at most (8 ms at 32^3, 72 ms at 125^3, two fields)
 template <typename T>
 struct PersistArgs {
     T* phi[2][2];  // [field][buffer]

@@ -22,6 +22,8 @@
 // Measured (us a pass, one launch a pass before): 16.4 -> 4.0 at 32^3 one field FP32 + Kahan, 21.9 ->
 // 7.9 at 64^3 two fields, 22.5 -> 11.4 at 96^3 one field; FP64 22.5 -> 6.2 at 32^3.  Of the 4.0, about
 // 1.0 is the barrier (release, arrival, poll), 1.0 FP64 instructions of the scalar warp.
+// Over a launch of one pass that is 12 us more than the pass: calls of few passes go to the kernels
+// launched per pass (persist_min_passes).
 // Waits are bounded: a barrier that does not complete within two seconds sets ST_TIMEOUT and
 // every block leaves.
 #include <type_traits>

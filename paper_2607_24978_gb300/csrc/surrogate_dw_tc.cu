@@ -29,7 +29,7 @@
 // Staging all three rows with every unit moved 4.5 GB through L2 for a 48-channel layer at 128^3,
 // 9 TB/s in 500 us.
 //
-// Warp roles, synchronised by mbarriers only: warp 0, lane 0 issues the MMAs; warps 1-6 stage
+// Warp roles, synchronised by mbarriers only: an elected lane of warp 0 issues the MMAs; warps 1-6 stage
 // units with cp.async, whose arrivals on the slot's barrier come when they land, as many units
 // ahead as there are slots (FP32 operands: loaded into registers a unit ahead, converted and
 // stored); warps 7-10 read the accumulators back at the end.  All

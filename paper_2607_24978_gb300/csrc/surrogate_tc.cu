@@ -16,7 +16,7 @@
 //
 // A block owns tiles of z-columns and marches up z through a ring of five staged input
 // planes, with three warp roles synchronised by mbarriers only:
-//  * warp 0, lane 0, issues the 27 * CI/16 MMAs of an output plane into one of two TMEM
+//  * an elected lane of warp 0 issues the 27 * CI/16 MMAs of an output plane into one of two TMEM
 //    accumulators once the three input planes are staged and the accumulator was read
 //    back, and commits them to the accumulator's "done" barrier and to the "free" barrier
 //    of every ring slot whose plane they read last;
